@@ -206,15 +206,41 @@ cudaError_t conv_dgrad(gff_unet* u, int l, View dz, View din, Dims d, cudaStream
     return cudaGetLastError();
 }
 
+// Weight gradient launch: 27 / TG tap groups times voxel chunks.  About four blocks per SM
+// (the shared-memory footprint lets two or three be resident), chunks of at least 512 voxels:
+// a block ends with TG CO CI atomic additions, and shorter chunks would be mostly that.
+template <int CO, int CI, int TG>
+cudaError_t launch_wgrad(const bf16* in, int sin, const bf16* dz, int sdz, float* dW, Dims d, cudaStream_t st) {
+    static_assert(27 % TG == 0 && CO % 16 == 0 && CI % 16 == 0 && CO <= 64, "tap groups and channel tiles");
+    constexpr size_t smem = wgrad_smem<CO, CI, TG>();
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad<CO, CI, TG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    long long chunks = std::max(1LL, std::min((d.V + 511) / 512, 608LL * TG / 27));
+    const long long chunk = ((d.V + chunks - 1) / chunks + WG_KV - 1) / WG_KV * WG_KV;
+    chunks = (d.V + chunk - 1) / chunk;
+    k_wgrad<CO, CI, TG><<<dim3(27 / TG, (unsigned)chunks), 256, smem, st>>>(in, sin, dz, sdz, dW, d, chunk);
+    return cudaGetLastError();
+}
+
 // weight and bias gradients of layer l from its input and dz
 cudaError_t conv_wgrad(gff_unet* u, int l, View in, View dz, Dims d, cudaStream_t st) {
     const int cinp = pad16(kL[l].cin), cout = kL[l].cout;
-    long long chunks = (d.V + 4095) / 4096;
-    if (chunks < 1) chunks = 1;
-    const long long chunk = (d.V + chunks - 1) / chunks;
-    const size_t smem = 64 * (cout + cinp) * sizeof(float);
-    k_wgrad<<<dim3(27, (unsigned)chunks), 256, smem, st>>>(in.p, in.s, cinp, dz.p, dz.s, cout, u->d_g + u->off_w[l], d,
-                                                           chunk);
+    float* dW = u->d_g + u->off_w[l];
+    cudaError_t e = cudaErrorInvalidValue;
+    // taps per block: all 27 where their sums fit the registers and their tiles the shared memory
+#define GFF_WG(CO, CI, TG) \
+    if (cout == CO && cinp == CI) e = launch_wgrad<CO, CI, TG>(in.p, in.s, dz.p, dz.s, dW, d, st);
+    GFF_WG(16, 16, 27)
+    GFF_WG(16, 32, 9)
+    GFF_WG(16, 48, 9)
+    GFF_WG(32, 16, 9)
+    GFF_WG(32, 32, 9)
+    GFF_WG(32, 96, 3)
+    GFF_WG(64, 32, 3)
+    GFF_WG(64, 64, 3)
+    GFF_WG(64, 128, 3)
+#undef GFF_WG
+    if (e != cudaSuccess) return e;
     k_bias_grad<<<grid_of(d.V), 256, 0, st>>>(dz.p, dz.s, cout, d.V, u->d_g + u->off_b[l]);
     return cudaGetLastError();
 }
