@@ -215,7 +215,9 @@ gff_status gff_measure_fp64_peak(double* gflops_out, double* ms_out);
  * <= -2 the register-staged persistent pass (two plane buffers) with -inv
  * blocks blocks.  fwd threads < 0: the register-staged forward pass of those
  * grids with -fwd threads threads.  TMA z blocks < 0: the TMA z pass with the
- * register-staged strip (nz = 64 or 128) and -(TMA z blocks) blocks. */
+ * register-staged strip (nz = 64 or 128) and -(TMA z blocks) blocks.  The
+ * register-staged shapes are FP32's; in FP64 they are accepted and run as the
+ * generic pass of the same threads. */
 gff_status gff_autotune(gff_handle* h, int* tiles_out);
 
 /* Sets the launch shapes instead of tuning them: tiles (host, 12 ints) in the

@@ -42,7 +42,7 @@ struct TableLayout {
 TableLayout table_layout() {
     TableLayout t;
     size_t o = 0;
-    t.tw64 = o; o += 3 * MAXN * sizeof(double2);
+    t.tw64 = o; o += 3 * MAXN * sizeof(int4);
     t.tw32 = o; o += 3 * MAXN * sizeof(float2);
     t.posx = o; o += MAXN * sizeof(int);
     t.fqy = o; o += MAXN * sizeof(int);
@@ -61,7 +61,7 @@ gff_status build_tables(gff_handle* h) {
             return fail(h, GFF_ERR_ARG, "grid axis %d: n = %d unsupported (even, 4..%d, factors 2,3,5)", a, n3[a], MAXN);
     const TableLayout L = table_layout();
     std::vector<unsigned char> host(L.total, 0);
-    double2* tw64 = reinterpret_cast<double2*>(host.data() + L.tw64);
+    int4* tw64 = reinterpret_cast<int4*>(host.data() + L.tw64);
     float2* tw32 = reinterpret_cast<float2*>(host.data() + L.tw32);
     int* posx = reinterpret_cast<int*>(host.data() + L.posx);
     int* fqy = reinterpret_cast<int*>(host.data() + L.fqy);
@@ -74,7 +74,9 @@ gff_status build_tables(gff_handle* h) {
         const double Lj = h->grid.L[a];
         for (int k = 0; k < n; ++k) {
             const double th = twopi * k / n;
-            tw64[a * MAXN + k] = make_double2(std::cos(th), -std::sin(th));
+            const long double thl = 6.283185307179586476925286766559006L * k / n, one = 4611686018427387904.0L;  // 2^62
+            const int2 re = twiddle_limbs(llroundl(std::cos(thl) * one)), im = twiddle_limbs(llroundl(-std::sin(thl) * one));
+            tw64[a * MAXN + k] = make_int4(re.x, re.y, im.x, im.y);
             tw32[a * MAXN + k] = make_float2((float)std::cos(th), (float)-std::sin(th));
             // wave-vector tables: q = 2 pi kappa / n, kappa = k (k < n/2) or k - n
             const int kappa = (2 * k < n) ? k : k - n;
@@ -97,7 +99,7 @@ gff_status build_tables(gff_handle* h) {
     if (e != cudaSuccess) return fail(h, GFF_ERR_CUDA, "tables copy: %s", cudaGetErrorString(e));
     unsigned char* d = static_cast<unsigned char*>(h->tables);
     for (int a = 0; a < 3; ++a) {
-        h->g.tw64[a] = reinterpret_cast<const double2*>(d + L.tw64) + a * MAXN;
+        h->g.tw64[a] = reinterpret_cast<const int4*>(d + L.tw64) + a * MAXN;
         h->g.tw32[a] = reinterpret_cast<const float2*>(d + L.tw32) + a * MAXN;
         for (int kind = 0; kind < 2; ++kind) {
             h->g.qt64[kind][a] = reinterpret_cast<const double*>(d + L.qt64) + (kind * 3 + a) * MAXN;
@@ -444,11 +446,16 @@ GFF_EXPORT gff_status gff_create(const gff_grid* grid, const gff_options* opt, g
         {(void**)&h->d_scal, 64 * sizeof(double), "scalars"},
         {(void**)&h->d_gid, N * sizeof(int), "grain id"},
         {(void**)&h->d_yhist, 2 * f32, "increment history"},
+        {(void**)&h->d_rq2, 2 * (size_t)grid->nz * grid->ny * h->nxh * sizeof(double), "projection factors"},
     };
     for (auto& a : allocs)
         if ((st = dalloc(h, a.p, a.b, a.w)) != GFF_OK) return st;
     cudaError_t e = cudaMallocHost(&h->h_scal, 64 * sizeof(double));
     if (e != cudaSuccess) return fail(h, GFF_ERR_OOM, "pinned scalars: %s", cudaGetErrorString(e));
+    e = fill_rq2(h->g, h->d_rq2, nullptr);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // the handle's stream is set later and may not wait for this one
+    if (e != cudaSuccess) return fail(h, GFF_ERR_CUDA, "projection factors: %s", cudaGetErrorString(e));
+    for (int kind = 0; kind < 2; ++kind) h->g.rq2[kind] = h->d_rq2 + (size_t)kind * grid->nz * grid->ny * h->nxh;
     return GFF_OK;
 }
 
@@ -460,7 +467,7 @@ GFF_EXPORT void gff_destroy(gff_handle* h) {
     dfree(h->d_p); dfree(h->d_Ap); dfree(h->d_K32); dfree(h->d_b32); dfree(h->d_x32); dfree(h->d_r32);
     dfree(h->d_p32); dfree(h->d_Ap32); dfree(h->d_spec); dfree(h->d_Fpi); dfree(h->d_chi); dfree(h->d_Fpi_t);
     dfree(h->d_chi_t); dfree(h->d_dg); dfree(h->d_tau); dfree(h->d_acc); dfree(h->d_flag); dfree(h->d_red);
-    dfree(h->d_scal); dfree(h->d_gq); dfree(h->d_yhist); dfree(h->d_geo32);
+    dfree(h->d_scal); dfree(h->d_gq); dfree(h->d_yhist); dfree(h->d_geo32); dfree(h->d_rq2);
     if (h->h_scal) cudaFreeHost(h->h_scal);
     for (int i = 0; i < h->pipe_nev; ++i) cudaEventDestroy(h->pipe_ev[i]);
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);

@@ -20,13 +20,21 @@
 // conjugate twiddles (digit-reversed in, natural out), so no reordering pass
 // is needed; the projection reads the frequency of each position from a table.
 // The common lengths (16 ... 128) have two-stage plans with compile-time
-// radices (fft2_lines); the others run the generic stages.
+// radices (fft2_lines); the others run the generic stages.  FP64 lines run
+// their stages on 64-bit integers (fft_lines_fx, fixed_bfly.cuh); at 128^3 the
+// FP64 apply takes 1.15 ms where FP64 butterflies took 2.71 ms (forward pass
+// 1.22 -> 0.60, z 0.64 -> 0.25, inverse 0.86 -> 0.31 ms).  What bounds it now:
+// the forward pass the 81 FP64 multiply-adds per voxel of K:x (0.27 ms at the
+// FP64 pipe's rate), before the row transforms and not under them, since one
+// plane fills an SM's shared memory; the others instruction issue (40 - 46 %)
+// of 16 warps per SM.
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
 
 #include "bulk_copy.cuh"
+#include "fixed_bfly.cuh"
 #include "gff_internal.cuh"
 
 namespace gff {
@@ -48,6 +56,14 @@ template <typename C> __device__ __forceinline__ C cmul(C a, C w) {
 }
 template <typename C> __device__ __forceinline__ C cmulc(C a, C w) {
     return mk<C>(a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y);
+}
+// in FP64 with the fused operand fixed: the passes that must agree bit for bit do not depend on the
+// compiler's choice of which product to fuse
+__device__ __forceinline__ double2 cmul(double2 a, double2 w) {
+    return make_double2(__fma_rn(a.x, w.x, -__dmul_rn(a.y, w.y)), __fma_rn(a.x, w.y, __dmul_rn(a.y, w.x)));
+}
+__device__ __forceinline__ double2 cmulc(double2 a, double2 w) {
+    return make_double2(__fma_rn(a.x, w.x, __dmul_rn(a.y, w.y)), __fma_rn(a.y, w.x, -__dmul_rn(a.x, w.y)));
 }
 // multiply by -i (forward) or +i (inverse)
 template <bool INV, typename C> __device__ __forceinline__ C rot90(C a) {
@@ -178,13 +194,28 @@ template <bool INV, typename C> struct Bfly<16, INV, C> {
     }
 };
 
+// The butterfly of a stage: a forward stage multiplies output p by tw(p), an inverse one input p
+// by conj(tw(p)) (p >= 1; twiddled = false: no twiddles).
+template <int R, bool INV, typename C, typename TF> __device__ __forceinline__ void bfly(C* v, bool twiddled, TF tw) {
+    if (INV && twiddled) {
+#pragma unroll
+        for (int p = 1; p < R; ++p) v[p] = cmulc(v[p], tw(p));
+    }
+    Bfly<R, INV, C>::run(v);
+    if (!INV && twiddled) {
+#pragma unroll
+        for (int p = 1; p < R; ++p) v[p] = cmul(v[p], tw(p));
+    }
+}
+template <typename C> __device__ __forceinline__ C no_tw(int) { return C{}; }
+
 // ---------------------------------------------------------------- one radix stage
 // Lines l = ls * NLF + lf start at s + ls*SS + lf*SF; elements are ES apart.
 // Sub-arrays of length `len` are split by radix R with stride m = len / R.
 // Threads take (lf fastest, then butterfly, then ls) so that neighbouring
 // lanes touch neighbouring shared-memory words.
 template <typename T, int R, bool INV>
-__device__ __forceinline__ void run_stage(typename C2<T>::t* s, const typename C2<T>::t* tw, int n, int len,
+__device__ __forceinline__ void run_stage(typename C2<T>::t* s, const typename TwT<T>::t* tw, int n, int len,
                                           int NLF, int SF, int NLS, int SS, int ES, int tid, int nthr) {
     using C = typename C2<T>::t;
     const int m = len / R, nb = n / R, twstep = n / len;
@@ -199,32 +230,16 @@ __device__ __forceinline__ void run_stage(typename C2<T>::t* s, const typename C
         const int j = bb - sub * m;
         C* base = s + lsl * SS + lf * SF + (sub * len + j) * ES;
         C v[R];
-        if (!INV) {
 #pragma unroll
-            for (int q = 0; q < R; ++q) v[q] = base[q * st];
-            Bfly<R, false, C>::run(v);
-            if (j) {
+        for (int q = 0; q < R; ++q) v[q] = base[q * st];
+        bfly<R, INV>(v, j != 0, [&](int p) { return tw[p * j * twstep]; });
 #pragma unroll
-                for (int p = 1; p < R; ++p) v[p] = cmul(v[p], tw[p * j * twstep]);
-            }
-#pragma unroll
-            for (int p = 0; p < R; ++p) base[p * st] = v[p];
-        } else {
-#pragma unroll
-            for (int p = 0; p < R; ++p) v[p] = base[p * st];
-            if (j) {
-#pragma unroll
-                for (int p = 1; p < R; ++p) v[p] = cmulc(v[p], tw[p * j * twstep]);
-            }
-            Bfly<R, true, C>::run(v);
-#pragma unroll
-            for (int q = 0; q < R; ++q) base[q * st] = v[q];
-        }
+        for (int q = 0; q < R; ++q) base[q * st] = v[q];
     }
 }
 
 template <typename T, bool INV>
-__device__ __forceinline__ void stage_dispatch(int R, typename C2<T>::t* s, const typename C2<T>::t* tw, int n,
+__device__ __forceinline__ void stage_dispatch(int R, typename C2<T>::t* s, const typename TwT<T>::t* tw, int n,
                                                int len, int NLF, int SF, int NLS, int SS, int ES, int tid,
                                                int nthr) {
     switch (R) {
@@ -258,7 +273,7 @@ __device__ __forceinline__ int divmod_f(int x, int d, float invd, int& r) {
 // over contiguous runs without twiddles -- the generic stages below with
 // compile-time radices and one (float) division per butterfly.
 template <typename T, int R1, int R2, bool TWIDDLED, bool INV>
-__device__ __forceinline__ void fft2_stage(typename C2<T>::t* s, const typename C2<T>::t* tw, int NLF, float invNLF,
+__device__ __forceinline__ void fft2_stage(typename C2<T>::t* s, const typename TwT<T>::t* tw, int NLF, float invNLF,
                                            int SF, int NLS, int SS, int ES, int tid, int nthr) {
     using C = typename C2<T>::t;
     // TWIDDLED: radix R1, tasks j < R2, elements j + q R2; else radix R2, tasks sub < R1, elements sub R2 + q
@@ -274,22 +289,14 @@ __device__ __forceinline__ void fft2_stage(typename C2<T>::t* s, const typename 
         C v[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) v[q] = base[q * st];
-        if (TWIDDLED && INV && task) {
-#pragma unroll
-            for (int p = 1; p < R; ++p) v[p] = cmulc(v[p], tw[p * task]);
-        }
-        Bfly<R, INV, C>::run(v);
-        if (TWIDDLED && !INV && task) {
-#pragma unroll
-            for (int p = 1; p < R; ++p) v[p] = cmul(v[p], tw[p * task]);
-        }
+        bfly<R, INV>(v, TWIDDLED && task, [&](int p) { return tw[p * task]; });
 #pragma unroll
         for (int p = 0; p < R; ++p) base[p * st] = v[p];
     }
 }
 
 template <typename T, int R1, int R2, bool INV>
-__device__ __forceinline__ void fft2_lines(typename C2<T>::t* s, const typename C2<T>::t* tw, int NLF, int SF,
+__device__ __forceinline__ void fft2_lines(typename C2<T>::t* s, const typename TwT<T>::t* tw, int NLF, int SF,
                                            int NLS, int SS, int ES, int tid, int nthr) {
     const float invNLF = 1.0f / (float)NLF;
     if (!INV) {
@@ -304,11 +311,214 @@ __device__ __forceinline__ void fft2_lines(typename C2<T>::t* s, const typename 
     __syncthreads();
 }
 
+// ---------------------------------------------------------------- FP64 lines in fixed point (fixed_bfly.cuh)
+// The stage of a line the integers do not take, in FP64.  Out of line: it is the exception.
+template <int R, bool INV>
+__device__ __noinline__ void fp64_bfly(double2* base, int st, const int4* tw, int pstep) {
+    double2 v[R];
+    for (int q = 0; q < R; ++q) v[q] = base[q * st];
+    bfly<R, INV>(v, pstep != 0, [&](int p) { return fx::tw_fp64(tw[p * pstep]); });
+    for (int q = 0; q < R; ++q) base[q * st] = v[q];
+}
+
+// Largest exponent key of every line (l as in run_stage) into keys[l]: eight lanes per line, four
+// lines per warp; rows (SF > 1) take neighbouring elements on neighbouring lanes, columns
+// neighbouring lines.
+__device__ __forceinline__ void line_keys(const double2* s, int* keys, int n, int NLF, float invNLF, int SF, int NLS, int SS, int ES,
+                                          int tid, int nthr) {
+    const int lane = tid & 31, L = NLF * NLS;
+    const bool rows = SF > 1;
+    const int part = rows ? lane & 7 : lane >> 2, sub = rows ? lane >> 3 : lane & 3;
+    for (int l0 = (tid >> 5) * 4; l0 < L; l0 += (nthr >> 5) * 4) {  // warp-uniform
+        const int l = l0 + sub;
+        int mk = 0;
+        if (l < L) {
+            int lf;
+            const int ls = divmod_f(l, NLF, invNLF, lf);
+            const double2* b = s + ls * SS + lf * SF;
+#pragma unroll 4
+            for (int e = part; e < n; e += 8) {
+                const double2 v = b[e * ES];
+                mk = fx::key_max(fx::key_max(mk, v.x), v.y);
+            }
+        }
+        const int o = rows ? 1 : 4;
+        mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
+        mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, 2 * o));
+        mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, 4 * o));
+        if (part == 0 && l < L) keys[l] = mk;
+    }
+}
+
+// One radix stage of every line, tasks as in run_stage (m = CM, nb = CNB where not 0).  FIRST:
+// aligns the line's values to its largest exponent (rin: they are integers aligned for this stage
+// already); LAST: rounds back to FP64 (rout: leaves the integers); between stages the shared memory
+// holds the 64-bit integers.  me + de62: the biased exponent of bit 62 after the stage.
+template <int R, bool INV, bool FIRST, bool LAST, int CM, int CNB>
+__device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* keys, int n, int len, int NLF, float invNLF,
+                                         int SF, int NLS, int SS, int ES, int tid, int nthr, int de62, bool rin,
+                                         bool rout) {
+    const int m = CM ? CM : len / R, nb = CNB ? CNB : n / R, twstep = CNB ? 1 : n / len;
+    const int total = NLF * nb * NLS, st = m * ES;
+    for (int idx = tid; idx < total; idx += nthr) {
+        int lf;
+        const int t = divmod_f(idx, NLF, invNLF, lf);
+        const int lsl = t / nb, bb = t - lsl * nb;
+        const int sub = bb / m, j = bb - sub * m;
+        double2* base = s + lsl * SS + lf * SF + (sub * m * R + j) * ES;
+        // a line of zeros (the projection leaves one per plane in a third of the components) is its own transform
+        const int lk = keys[lsl * NLF + lf], me = lk >> 20;
+        if (lk == 0) continue;
+        if (me < fx::ME_MIN || me > fx::ME_MAX) {
+            fp64_bfly<R, INV>(base, st, tw, j * twstep);
+            continue;
+        }
+        fx::Cq f[R];
+        if (FIRST && !rin) {
+            const int key = ((me + 63 - fx::Top<R>::v) << 20) | 0xfffff;
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const double2 v = base[q * st];
+                f[q] = fx::Cq{fx::to_fixed(v.x, key), fx::to_fixed(v.y, key)};
+            }
+        } else {
+            constexpr int H = FIRST ? 0 : fx::headroom(R);
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const longlong2 v = reinterpret_cast<const longlong2&>(base[q * st]);
+                f[q] = fx::Cq{fx::shift_down<H>(v.x), fx::shift_down<H>(v.y)};
+            }
+        }
+        if (INV && j) {
+#pragma unroll
+            for (int p = 1; p < R; ++p) f[p] = fx::twmul<true>(f[p], tw[p * j * twstep]);
+        }
+        fx::Bq<R, INV>::run(f);
+        if (!INV && j) {
+#pragma unroll
+            for (int p = 1; p < R; ++p) f[p] = fx::twmul<false>(f[p], tw[p * j * twstep]);
+        }
+        if (LAST && !rout) {
+            const int e62 = me + de62;
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                base[q * st] = make_double2(fx::from_fixed(f[q].x, e62), fx::from_fixed(f[q].y, e62));
+        } else {
+#pragma unroll
+            for (int q = 0; q < R; ++q) reinterpret_cast<longlong2&>(base[q * st]) = make_longlong2(f[q].x, f[q].y);
+        }
+    }
+    __syncthreads();
+}
+
+// The stage's place in a plan of any number of stages.  Plans put 16, 8, 4, 2 before 5 and 3 (2 may
+// follow 16), and 4 and 8 alone are plans: only those places are compiled.
+template <int R, bool INV>
+__device__ __forceinline__ void fx_stage_any(bool first, bool last, double2* s, const int4* tw, const int* keys, int n, int len,
+                                             int NLF, float invNLF, int SF, int NLS, int SS, int ES, int tid, int nthr, int de62, bool rin, bool rout) {
+    constexpr bool head = R == 16 || R == 8 || R == 4 || R == 2, tail = R == 5 || R == 3;
+    if (first && last) {
+        if constexpr (R == 8 || R == 4)
+            fx_stage<R, INV, true, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+    } else if (first) {
+        if constexpr (INV ? tail : head)
+            fx_stage<R, INV, true, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+    } else if (last) {
+        if constexpr (INV ? head : tail)
+            fx_stage<R, INV, false, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+    } else {
+        if constexpr (tail || R == 2)
+            fx_stage<R, INV, false, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+    }
+}
+
+// lines of one call: ny / 2 or nx / 2 <= 64, 2 W <= 64, 9 W = 36
+constexpr int FX_MAX_LINES = 128;
+__device__ __forceinline__ int* fx_line_keys() {
+    __shared__ int keys[FX_MAX_LINES];
+    return keys;
+}
+// Integers as they enter or leave a transform: IN: aligned for its first stage, their keys given; OUT: left as they are
+// after its last stage, their exponents me + fx_out_exp(plan).
+enum { FX_FP64 = 0, FX_IN = 1, FX_OUT = 2 };
+__host__ __device__ inline int fx_top(int R) {
+    return R == 16 ? fx::Top<16>::v : R == 8 ? fx::Top<8>::v : R == 5 ? fx::Top<5>::v : R == 4 ? fx::Top<4>::v : R == 3 ? fx::Top<3>::v : fx::Top<2>::v;
+}
+// exponent of bit 62 after a forward transform, relative to the line's largest
+__device__ __forceinline__ int fx_out_exp(const AxisPlan& pl) {
+    int e = 62 - fx_top(pl.radix[0]);
+    for (int i = 1; i < pl.nst; ++i) e += fx::headroom(pl.radix[i]);
+    return e;
+}
+
+template <bool INV>
+__device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const AxisPlan& pl, int NLF, int SF, int NLS, int SS, int ES,
+                                          int tid, int nthr, int* keys, int io) {
+    const int n = pl.n;
+    const float invNLF = 1.0f / (float)NLF;
+    const bool rin = INV && (io & FX_IN), rout = !INV && (io & FX_OUT);
+    if (!rin) {
+        line_keys(s, keys, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr);
+        __syncthreads();
+    }
+    const int extra = rin ? 1 : 0;  // integers given are aligned one bit lower (plane_inv_compute)
+    if (pl.nst == 2) {
+        const int r1 = pl.radix[0], r2 = pl.radix[1];
+#define GFF_FX2(A, B)                                                                                                  \
+    if (r1 == A && r2 == B) {                                                                                          \
+        if (!INV) {                                                                                                    \
+            fx_stage<A, false, true, false, B, B>(s, tw, keys, n, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, 0,       \
+                                                  false, rout);                                                        \
+            fx_stage<B, false, false, true, 1, A>(s, tw, keys, n, B, NLF, invNLF, SF, NLS, SS, ES, tid, nthr,          \
+                                                  62 - fx::Top<A>::v + fx::headroom(B), false, rout);                  \
+        } else {                                                                                                       \
+            fx_stage<B, true, true, false, 1, A>(s, tw, keys, n, B, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, 0, rin,   \
+                                                 false);                                                               \
+            fx_stage<A, true, false, true, B, B>(s, tw, keys, n, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr,           \
+                                                 62 - fx::Top<B>::v + fx::headroom(A) + extra, rin, false);            \
+        }                                                                                                              \
+        return;                                                                                                        \
+    }
+        GFF_FX2(16, 8)
+        GFF_FX2(8, 8)
+        GFF_FX2(16, 5)
+        GFF_FX2(16, 3)
+        GFF_FX2(8, 5)
+        GFF_FX2(8, 4)
+        GFF_FX2(8, 3)
+        GFF_FX2(4, 4)
+#undef GFF_FX2
+    }
+    int len = INV ? 1 : n, de62 = extra;
+    for (int i = 0; i < pl.nst; ++i) {
+        const int R = pl.radix[INV ? pl.nst - 1 - i : i];
+        const bool first = i == 0, last = i == pl.nst - 1;
+        if (INV) len *= R;
+#define GFF_FX(RR)                                                                                                     \
+    case RR:                                                                                                           \
+        de62 += first ? 62 - fx::Top<RR>::v : fx::headroom(RR);                                                        \
+        fx_stage_any<RR, INV>(first, last, s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout); \
+        break;
+        switch (R) {
+            GFF_FX(16)
+            GFF_FX(8)
+            GFF_FX(5)
+            GFF_FX(4)
+            GFF_FX(3)
+            GFF_FX(2)
+            default: break;
+        }
+#undef GFF_FX
+        if (!INV) len /= R;
+    }
+}
+
 // Whole transform of a batch of lines; ends with a barrier.  Not inlined:
 // every kernel calls the same four instances (precision x direction).
-template <typename T, bool INV>
-__device__ __noinline__ void fft_lines(typename C2<T>::t* s, const typename C2<T>::t* tw, const AxisPlan& pl, int NLF, int SF,
-                          int NLS, int SS, int ES, int tid, int nthr) {
+template <bool INV>
+__device__ __noinline__ void fft_lines_f32(float2* s, const float2* tw, const AxisPlan& pl, int NLF, int SF, int NLS, int SS, int ES,
+                                           int tid, int nthr) {
+    using T = float;
     const int n = pl.n;
     if (pl.nst == 2) {
         const int r1 = pl.radix[0], r2 = pl.radix[1];
@@ -344,8 +554,17 @@ __device__ __noinline__ void fft_lines(typename C2<T>::t* s, const typename C2<T
     }
 }
 
-template <typename T> __device__ __forceinline__ const typename C2<T>::t* twp(const GridDev& g, int a);
-template <> __device__ __forceinline__ const double2* twp<double>(const GridDev& g, int a) { return g.tw64[a]; }
+template <typename T, bool INV>
+__device__ __forceinline__ void fft_lines(typename C2<T>::t* s, const typename TwT<T>::t* tw, const AxisPlan& pl, int NLF, int SF,
+                                          int NLS, int SS, int ES, int tid, int nthr, int io = 0) {
+    if constexpr (sizeof(T) == 8)
+        fft_lines_fx<INV>(s, tw, pl, NLF, SF, NLS, SS, ES, tid, nthr, fx_line_keys(), io);
+    else
+        fft_lines_f32<INV>(s, tw, pl, NLF, SF, NLS, SS, ES, tid, nthr);
+}
+
+template <typename T> __device__ __forceinline__ const typename TwT<T>::t* twp(const GridDev& g, int a);
+template <> __device__ __forceinline__ const int4* twp<double>(const GridDev& g, int a) { return g.tw64[a]; }
 template <> __device__ __forceinline__ const float2* twp<float>(const GridDev& g, int a) { return g.tw32[a]; }
 template <typename T> __device__ __forceinline__ const T* qtp(const GridDev& g, int kind, int a);
 template <> __device__ __forceinline__ const double* qtp<double>(const GridDev& g, int kind, int a) {
@@ -468,6 +687,15 @@ __device__ __forceinline__ void plane_contract(typename C2<T>::t* s, const T* __
     }
 }
 
+// Half spectra of the two real rows of a packed row at one frequency, from the integers of the x transform
+// (zk, zm: bits of the frequency and its mirror, e62 the exponent of their bit 62).
+__device__ __forceinline__ void split_fx(double2& A, double2& B, const double2& zk, const double2& zm, int e62) {
+    const long long kx = __double_as_longlong(zk.x) >> 1, ky = __double_as_longlong(zk.y) >> 1;
+    const long long mx = __double_as_longlong(zm.x) >> 1, my = __double_as_longlong(zm.y) >> 1;
+    A = make_double2(fx::from_fixed(kx + mx, e62), fx::from_fixed(ky - my, e62));
+    B = make_double2(fx::from_fixed(ky + my, e62), fx::from_fixed(mx - kx, e62));
+}
+
 template <typename T, bool WITH_K, bool VEC>
 __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T* __restrict__ K,
                                                typename C2<T>::t* __restrict__ spec, const GridDev& g, const int c,
@@ -475,8 +703,8 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
     using C = typename C2<T>::t;
     const int nx = g.nx, ny = g.ny, nxh = g.nxh, ls = nxh, half = ny / 2;
     C* s = reinterpret_cast<C*>(sm_raw);
-    C* twx = s + ny * ls;
-    C* twy = twx + nx;
+    auto* twx = reinterpret_cast<typename TwT<T>::t*>(s + ny * ls);
+    auto* twy = twx + nx;
     int* posx = reinterpret_cast<int*>(twy + ny);
     int* posy = posx + nx;  // position of each y frequency after the forward y transform
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -495,7 +723,8 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
     // x transform of the ny/2 packed rows (row pair r at offset 2 r ls); rows are the
     // fast thread index, so that neighbouring lanes read neighbouring rows rather than
     // butterflies 8 or 16 elements apart in one row (fewer shared-memory bank conflicts)
-    fft_lines<T, false>(s, twx, g.ax, half, 2 * ls, 1, 0, 1, tid, nthr);
+    fft_lines<T, false>(s, twx, g.ax, half, 2 * ls, 1, 0, 1, tid, nthr, FX_OUT);
+    const int de62 = sizeof(T) == 8 ? fx_out_exp(g.ax) : 0;
     // split each packed row into the half spectra of its two real rows.  Columns
     // kx = 0 and nx/2 of a real row are real, so one complex y transform of
     // Z = X_0 + i X_h carries both and nx/2 columns are transformed, not nx/2 + 1:
@@ -515,6 +744,17 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
             if (rok && k <= kh) {
                 const C zk = row[posx[k]];
                 const C zm = row[posx[k == 0 ? 0 : nx - k]];
+                if constexpr (sizeof(T) == 8) {  // the row's integers; FP64 where it did not run on integers
+                    const int me = fx_line_keys()[r] >> 20;
+                    if (me >= fx::ME_MIN && me <= fx::ME_MAX) {
+                        split_fx(A[t], B[t], zk, zm, me + de62);
+                        if (k == kh) {
+                            ah = A[t].x;
+                            bh = B[t].x;
+                        }
+                        continue;
+                    }
+                }
                 A[t] = mk<C>((zk.x + zm.x) * (T)0.5, (zk.y - zm.y) * (T)0.5);
                 B[t] = mk<C>((zk.y + zm.y) * (T)0.5, (zm.x - zk.x) * (T)0.5);
                 if (k == kh) {
@@ -590,15 +830,14 @@ template <> __device__ __forceinline__ float rnorm3<float>(float a, float b, flo
 // of the z positions, and the block's column frequencies colk[W]
 // (kx | ky << 16, -1 past the end).
 template <typename T> struct ZTables {
-    typename C2<T>::t* twz;
+    typename TwT<T>::t* twz;
     T *qx, *qy, *qz;
     int *fqz, *colk;
 };
 
 template <typename T> __device__ __forceinline__ ZTables<T> ztables_at(unsigned char* p, const GridDev& g) {
-    using C = typename C2<T>::t;
     ZTables<T> tb;
-    tb.twz = reinterpret_cast<C*>(p);
+    tb.twz = reinterpret_cast<typename TwT<T>::t*>(p);
     tb.qx = reinterpret_cast<T*>(tb.twz + g.nz);
     tb.qy = tb.qx + g.nxh;
     tb.qz = tb.qy + g.ny;
@@ -697,13 +936,56 @@ __device__ __forceinline__ void zrow_proj(typename C2<T>::t& u, typename C2<T>::
         v = cscale(t, d);
     }
 }
+// The FP64 projection also applies the inverse transform's 1 / N (sc; the masks come multiplied by it): it costs nothing in
+// the factor r = sc / |q|^2, which the grid's table holds (a division per frequency is half of the FP64 operations of
+// this pass), and saves the plane pass an FP64 operation per voxel.
+__device__ __forceinline__ void zrow_proj64(double2& u, double2& v, int kx, int ky, int kz, int nx, int ny, int nz, double m0,
+                                            double m1, double m2, double sc, const double* rq2, long long at,
+                                            const ZTables<double>& tb) {
+    if (kx == nx / 2 || ky == ny / 2 || kz == nz / 2) {
+        u = v = make_double2(0.0, 0.0);
+    } else if (kx == 0 && ky == 0) {
+        if (kz == 0) {
+            u = make_double2(u.x * m0, u.y * m1);
+            v = cscale(v, m2);
+        } else {
+            u = make_double2(0.0, 0.0);
+            v = cscale(v, sc);
+        }
+    } else {
+        const double d = tb.qz[kz];
+        double r;
+        if (rq2) {
+            r = __ldg(rq2 + at);
+        } else {
+            const double a = tb.qx[kx], b = tb.qy[ky];
+            r = sc / fma(a, a, fma(b, b, d * d));
+        }
+        const double2 t = make_double2(fma(d, v.x, u.x) * r, fma(d, v.y, u.y) * r);
+        u = t;
+        v = cscale(t, d);
+    }
+}
+// the table: one thread per position (pz, py, kx) of the half spectrum, both kinds; the expression above
+__global__ void __launch_bounds__(256) k_fill_rq2(GridDev g, double* tab) {
+    const int nF = g.ny * g.nxh, total = g.nz * nF;
+    const double sc = 1.0 / (double)g.N;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * total; i += gridDim.x * blockDim.x) {
+        const int kind = i / total, e = i - kind * total;
+        const int pz = e / nF, f = e - pz * nF, py = f / g.nxh, kx = f - py * g.nxh;
+        const int ky = g.fqy[py], kz = g.fqz[pz];
+        const double a = g.qt64[kind][0][kx], b = g.qt64[kind][1][ky], d = g.qt64[kind][2][kz];
+        const bool special = kx == g.nx / 2 || ky == g.ny / 2 || kz == g.nz / 2 || (kx == 0 && ky == 0);
+        tab[i] = special ? 0.0 : sc / fma(a, a, fma(b, b, d * d));
+    }
+}
 
 // Forward z transform, projection and inverse z transform of one loaded strip
 // s = [3][nz][W] (tensor row `row`): the row packed into u (slot 0) and
 // v (slot 2), both transformed, projected, transformed back and unpacked into
 // the three slots; ends with a barrier.
 template <typename T, int W>
-__device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev& g, const ProjArgs& pa, int row,
+__device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev& g, const ProjArgs& pa, int row, int f0,
                                             const ZTables<T>& tb) {
     using C = typename C2<T>::t;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
@@ -711,7 +993,8 @@ __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev&
     for (int e = tid; e < nz * W; e += nthr) s[e] = zpack<T>(s[e], s[nz * W + e], zcol<T>(tb.colk[e % W], tb));
     __syncthreads();
     fft_lines<T, false>(s, tb.twz, g.az, W, 1, 2, 2 * nz * W, W, tid, nthr);
-    const T m0 = (T)pa.mask[3 * row], m1 = (T)pa.mask[3 * row + 1], m2 = (T)pa.mask[3 * row + 2];
+    const T sc = sizeof(T) == 8 ? (T)1 / (T)g.N : (T)1;
+    const T m0 = (T)pa.mask[3 * row] * sc, m1 = (T)pa.mask[3 * row + 1] * sc, m2 = (T)pa.mask[3 * row + 2] * sc;
     for (int e = tid; e < nz * W; e += nthr) {
         const int w = e % W, pz = e / W;
         const int ck = tb.colk[w];
@@ -719,7 +1002,10 @@ __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev&
         const int kx = ck & 0xffff, ky = ck >> 16, kz = tb.fqz[pz];
         C* p0 = s + pz * W + w;
         C u = p0[0], v = p0[2 * nz * W];
-        zrow_proj<T>(u, v, kx, ky, kz, nx, ny, nz, m0, m1, m2, tb);
+        if constexpr (sizeof(T) == 8)
+            zrow_proj64(u, v, kx, ky, kz, nx, ny, nz, m0, m1, m2, sc, g.rq2[pa.kind], (long long)pz * ny * g.nxh + f0 + w, tb);
+        else
+            zrow_proj<T>(u, v, kx, ky, kz, nx, ny, nz, m0, m1, m2, tb);
         p0[0] = u;
         p0[2 * nz * W] = v;
     }
@@ -757,11 +1043,7 @@ __device__ __forceinline__ void zstrip2(typename C2<T>::t* s, const GridDev& g, 
 #pragma unroll
             for (int q = 0; q < R1; ++q) v[q] = b[q * R2 * W];
         }
-        Bfly<R1, false, C>::run(v);
-        if (j) {
-#pragma unroll
-            for (int p = 1; p < R1; ++p) v[p] = cmul(v[p], tb.twz[p * j]);
-        }
+        bfly<R1, false>(v, j != 0, [&](int p) { return tb.twz[p * j]; });
 #pragma unroll
         for (int q = 0; q < R1; ++q) b[q * R2 * W] = v[q];
     }
@@ -778,16 +1060,16 @@ __device__ __forceinline__ void zstrip2(typename C2<T>::t* s, const GridDev& g, 
             u[q] = b[q * W];
             v[q] = b[(2 * nz + q) * W];
         }
-        Bfly<R2, false, C>::run(u);
-        Bfly<R2, false, C>::run(v);
+        bfly<R2, false>(u, false, no_tw<C>);
+        bfly<R2, false>(v, false, no_tw<C>);
         if (ck >= 0) {
             const int kx = ck & 0xffff, ky = ck >> 16;
 #pragma unroll
             for (int q = 0; q < R2; ++q)
                 zrow_proj<T>(u[q], v[q], kx, ky, tb.fqz[sub * R2 + q], nx, ny, nz, m0, m1, m2, tb);
         }
-        Bfly<R2, true, C>::run(u);
-        Bfly<R2, true, C>::run(v);
+        bfly<R2, true>(u, false, no_tw<C>);
+        bfly<R2, true>(v, false, no_tw<C>);
 #pragma unroll
         for (int q = 0; q < R2; ++q) {
             b[q * W] = u[q];
@@ -802,11 +1084,7 @@ __device__ __forceinline__ void zstrip2(typename C2<T>::t* s, const GridDev& g, 
         C v[R1];
 #pragma unroll
         for (int q = 0; q < R1; ++q) v[q] = b[q * R2 * W];
-        if (j) {
-#pragma unroll
-            for (int p = 1; p < R1; ++p) v[p] = cmulc(v[p], tb.twz[p * j]);
-        }
-        Bfly<R1, true, C>::run(v);
+        bfly<R1, true>(v, j != 0, [&](int p) { return tb.twz[p * j]; });
         if (comp == 0) {
             const ZCol<T> c = zcol<T>(tb.colk[w], tb);
 #pragma unroll
@@ -840,7 +1118,7 @@ __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec,
         s[e] = f < nF ? base[cz * nF + f] : mk<C>((T)0, (T)0);
     }
     __syncthreads();
-    zproj_strip<T, W>(s, g, pa, row, tb);
+    zproj_strip<T, W>(s, g, pa, row, f0, tb);
     for (int e = tid; e < 3 * nz * W; e += nthr) {
         const int w = e % W, cz = e / W;
         const int f = f0 + w;
@@ -848,8 +1126,11 @@ __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec,
     }
 }
 
+// FP64 transforms take what registers they get: 128 (16 warps per SM) rather than 190 (8 to 10)
+template <typename T> constexpr int z_min_blocks() { return sizeof(T) == 8 ? 2 : 1; }
+
 template <typename T, int W>
-__global__ void __launch_bounds__(256) k_zproj(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
+__global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
                                               const int* __restrict__ skip) {
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -869,7 +1150,7 @@ template <typename T> size_t zsym_smem(const GridDev& g) {
 }
 
 template <typename T, int W>
-__global__ void __launch_bounds__(256) k_zproj_sym(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
+__global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj_sym(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
                                                   const int* __restrict__ skip) {
     using C = typename C2<T>::t;
     if (skip && *skip) return;
@@ -1013,7 +1294,7 @@ __global__ void __launch_bounds__(BT, ztma_min_blocks<T, W, R1, BT>())
         if constexpr (R1 > 0)
             zstrip2<T, R1, W>(buf[cur], g, pa, s % 3, tb);
         else
-            zproj_strip<T, W>(buf[cur], g, pa, s % 3, tb);
+            zproj_strip<T, W>(buf[cur], g, pa, s % 3, (s / 3) * W, tb);
         fence_proxy_async_smem();  // the transforms' writes, before the asynchronous store reads them
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -1026,12 +1307,84 @@ __global__ void __launch_bounds__(BT, ztma_min_blocks<T, W, R1, BT>())
 }
 
 // ---------------------------------------------------------------- pass 3: inverse 2D transform + epilogue
+// Epilogue of a plane: packed rows (real parts row 2r, imaginary parts row 2r + 1) to y = sc v + ad; PLAIN (FP64, sc = +-1,
+// ad = 0): a sign at most, no FP64 operation.
+template <typename T, bool PLAIN> __device__ __forceinline__ T out_value(T v, T sc, T ad) {
+    if constexpr (PLAIN)
+        return __hiloint2double(__double2hiint(v) ^ (__double2hiint(sc) & 0x80000000), __double2loint(v));
+    else
+        return fma(sc, v, ad);
+}
+template <typename T, bool VEC, bool PLAIN>
+__device__ __forceinline__ void plane_store(const typename C2<T>::t* s, T* __restrict__ yc, const long long pl, const GridDev& g,
+                                            const T sc, const T ad) {
+    using C = typename C2<T>::t;
+    const int nx = g.nx, ny = g.ny, ls = g.nxh, half = ny / 2;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    if (VEC) {
+        // the mirror of the load in pass 1: lanes 2i, 2i+1 each read VW/2 whole
+        // complex values (16 bytes) of packed row r, swap halves, and write VW
+        // voxels of rows 2r (real parts) and 2r+1 (imaginary parts)
+        using VT = typename V16<T>::t;
+        constexpr int VW = V16<T>::n, HW = VW / 2;
+        const int nxv = nx / VW, total = ny * nxv;
+        const int lane = tid & 31;
+        for (int e0 = tid - lane; e0 < total; e0 += nthr) {
+            const int e = e0 + lane;
+            const bool act = e < total;
+            const int p = e & 1, q = e >> 1;
+            const int r = q / nxv, xv = q - r * nxv;
+            VT in;
+            T* ip = reinterpret_cast<T*>(&in);
+#pragma unroll
+            for (int j = 0; j < VW; ++j) ip[j] = (T)0;
+            if (act) in = *reinterpret_cast<const VT*>(s + r * 2 * ls + xv * VW + p * HW);
+            VT o;
+            T* op = reinterpret_cast<T*>(&o);
+#pragma unroll
+            for (int j = 0; j < HW; ++j) {
+                const T recv = __shfl_xor_sync(0xffffffffu, p ? ip[2 * j] : ip[2 * j + 1], 1);
+                op[j] = out_value<T, PLAIN>(p ? recv : ip[2 * j], sc, ad);
+                op[HW + j] = out_value<T, PLAIN>(p ? ip[2 * j + 1] : recv, sc, ad);
+            }
+            if (act) *reinterpret_cast<VT*>(yc + pl + (long long)(2 * r + p) * nx + xv * VW) = o;
+        }
+    } else {
+        for (int e = tid; e < half * nx; e += nthr) {
+            const int r = e / nx, xi = e - r * nx;
+            const long long v0 = pl + (long long)(2 * r) * nx + xi;
+            const C zv = s[r * 2 * ls + xi];
+            yc[v0] = out_value<T, PLAIN>(zv.x, sc, ad);
+            yc[v0 + nx] = out_value<T, PLAIN>(zv.y, sc, ad);
+        }
+    }
+}
+
+// The merge of one packed row (below) in FP64, for the rows the integers do not take; one warp.
+__device__ __noinline__ void merge_row_fp64(double2* row, int ls, const int* posx, int nx, int lane) {
+    const int kh = nx / 2;
+    double2 A[SPLIT_K<double>], B[SPLIT_K<double>];
+    for (int t = 0, k = lane; k <= kh; ++t, k += 32) {
+        A[t] = k < kh ? row[k] : make_double2(row[0].y, 0.0);
+        B[t] = k < kh ? row[ls + k] : make_double2(row[ls].y, 0.0);
+    }
+    __syncwarp();
+    for (int t = 0, k = lane; k <= kh; ++t, k += 32) {
+        if (k == 0 || k == kh) {
+            row[posx[k]] = make_double2(A[t].x, B[t].x);
+        } else {
+            row[posx[k]] = make_double2(A[t].x - B[t].y, A[t].y + B[t].x);
+            row[posx[nx - k]] = make_double2(A[t].x + B[t].y, B[t].x - A[t].y);
+        }
+    }
+}
+
 // Inverse y transform, merge of the packed rows, complex-to-real x transform
 // and epilogue of one plane already in shared memory s (tables loaded).
 template <typename T, bool VEC>
 __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __restrict__ y, const GridDev& g,
                                                   const OutArgs& oa, const int c, const int z,
-                                                  const typename C2<T>::t* twx, const typename C2<T>::t* twy,
+                                                  const typename TwT<T>::t* twx, const typename TwT<T>::t* twy,
                                                   const int* posx) {
     using C = typename C2<T>::t;
     const int nx = g.nx, ny = g.ny, nxh = g.nxh, ls = nxh, half = ny / 2;
@@ -1069,6 +1422,37 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
             }
         }
         __syncwarp();
+        if constexpr (sizeof(T) == 8) {
+            // FP64: one row per warp; aligned to the largest value of both half spectra, one bit below the first
+            // stage's alignment (|A| + |B|), and merged as integers
+            int mkey = 0;
+#pragma unroll
+            for (int t = 0; t < SPLIT_K<T>; ++t)
+                if (kg + SPLIT_G<T> * t <= kh)
+                    mkey = fx::key_max(fx::key_max(fx::key_max(fx::key_max(mkey, A[t].x), A[t].y), B[t].x), B[t].y);
+            mkey = (int)__reduce_max_sync(0xffffffffu, (unsigned)mkey);
+            if (lane == 0) fx_line_keys()[r] = mkey;
+            const int me = mkey >> 20;
+            if (me >= fx::ME_MIN && me <= fx::ME_MAX) {
+                const int key = ((me + 64 - fx_top(g.ax.radix[g.ax.nst - 1])) << 20) | 0xfffff;
+#pragma unroll
+                for (int t = 0; t < SPLIT_K<T>; ++t) {
+                    const int k = kg + SPLIT_G<T> * t;
+                    if (k > kh) continue;
+                    const long long ax = fx::to_fixed(A[t].x, key), ay = fx::to_fixed(A[t].y, key);
+                    const long long bx = fx::to_fixed(B[t].x, key), by = fx::to_fixed(B[t].y, key);
+                    longlong2* z = reinterpret_cast<longlong2*>(row);
+                    if (k == 0 || k == kh) {
+                        z[posx[k]] = make_longlong2(ax, bx);
+                    } else {
+                        z[posx[k]] = make_longlong2(ax - by, ay + bx);
+                        z[posx[nx - k]] = make_longlong2(ax + by, bx - ay);
+                    }
+                }
+            } else {
+                merge_row_fp64(row, ls, posx, nx, lane);
+            }
+        } else {
 #pragma unroll
         for (int t = 0; t < SPLIT_K<T>; ++t) {
             const int k = kg + SPLIT_G<T> * t;
@@ -1081,48 +1465,22 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
                 }
             }
         }
+        }
     }
     __syncthreads();
-    fft_lines<T, true>(s, twx, g.ax, half, 2 * ls, 1, 0, 1, tid, nthr);  // rows fastest, as in pass 1
-    const T sc = (T)oa.scale, ad = (T)oa.add[c];
-    T* yc = y + c * N;
-    if (VEC) {
-        // the mirror of the load in pass 1: lanes 2i, 2i+1 each read VW/2 whole
-        // complex values (16 bytes) of packed row r, swap halves, and write VW
-        // voxels of rows 2r (real parts) and 2r+1 (imaginary parts)
-        using VT = typename V16<T>::t;
-        constexpr int VW = V16<T>::n, HW = VW / 2;
-        const int nxv = nx / VW, total = ny * nxv;
-        const int lane = tid & 31;
-        for (int e0 = tid - lane; e0 < total; e0 += nthr) {
-            const int e = e0 + lane;
-            const bool act = e < total;
-            const int p = e & 1, q = e >> 1;
-            const int r = q / nxv, xv = q - r * nxv;
-            VT in;
-            T* ip = reinterpret_cast<T*>(&in);
-#pragma unroll
-            for (int j = 0; j < VW; ++j) ip[j] = (T)0;
-            if (act) in = *reinterpret_cast<const VT*>(s + r * 2 * ls + xv * VW + p * HW);
-            VT o;
-            T* op = reinterpret_cast<T*>(&o);
-#pragma unroll
-            for (int j = 0; j < HW; ++j) {
-                const T recv = __shfl_xor_sync(0xffffffffu, p ? ip[2 * j] : ip[2 * j + 1], 1);
-                op[j] = fma(sc, p ? recv : ip[2 * j], ad);
-                op[HW + j] = fma(sc, p ? ip[2 * j + 1] : recv, ad);
+    fft_lines<T, true>(s, twx, g.ax, half, 2 * ls, 1, 0, 1, tid, nthr, FX_IN);  // rows fastest, as in pass 1
+    T sc = (T)oa.scale;
+    const T ad = (T)oa.add[c];
+    if constexpr (sizeof(T) == 8) {
+        if (oa.pre) {  // the z pass has applied |scale|
+            sc = sc < 0 ? -1.0 : 1.0;
+            if (ad == 0) {
+                plane_store<T, VEC, true>(s, y + c * N, pl, g, sc, ad);
+                return;
             }
-            if (act) *reinterpret_cast<VT*>(yc + pl + (long long)(2 * r + p) * nx + xv * VW) = o;
-        }
-    } else {
-        for (int e = tid; e < half * nx; e += nthr) {
-            const int r = e / nx, xi = e - r * nx;
-            const long long v0 = pl + (long long)(2 * r) * nx + xi;
-            const C zv = s[r * 2 * ls + xi];
-            yc[v0] = fma(sc, zv.x, ad);
-            yc[v0 + nx] = fma(sc, zv.y, ad);
         }
     }
+    plane_store<T, VEC, false>(s, y + c * N, pl, g, sc, ad);
 }
 
 // Plane (c, z) of the output set to NaN: what an inverse pass leaves where a
@@ -1135,7 +1493,7 @@ __device__ __noinline__ void plane_fill_nan(T* y, const GridDev& g, int c, int z
 }
 
 template <typename T>
-__device__ __forceinline__ void plane_tables(const GridDev& g, typename C2<T>::t* twx, typename C2<T>::t* twy,
+__device__ __forceinline__ void plane_tables(const GridDev& g, typename TwT<T>::t* twx, typename TwT<T>::t* twy,
                                              int* posx) {
     for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
         twx[i] = twp<T>(g, 0)[i];
@@ -1151,8 +1509,8 @@ __device__ __forceinline__ void plane_inv_body(const typename C2<T>::t* __restri
     using C = typename C2<T>::t;
     const int nx = g.nx, ny = g.ny, nxh = g.nxh, ls = nxh;
     C* s = reinterpret_cast<C*>(sm_raw);
-    C* twx = s + ny * ls;
-    C* twy = twx + nx;
+    auto* twx = reinterpret_cast<typename TwT<T>::t*>(s + ny * ls);
+    auto* twy = twx + nx;
     int* posx = reinterpret_cast<int*>(twy + ny);
     const int tid = threadIdx.x, nthr = blockDim.x;
     plane_tables<T>(g, twx, twy, posx);
@@ -1180,8 +1538,8 @@ __global__ void __launch_bounds__(512) k_plane_inv(const typename C2<T>::t* __re
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int nx = g.nx, plane = g.ny * g.nxh;
     C* s = reinterpret_cast<C*>(sm_raw);
-    C* twx = s + plane;
-    C* twy = twx + nx;
+    auto* twx = reinterpret_cast<typename TwT<T>::t*>(s + plane);
+    auto* twy = twx + nx;
     int* posx = reinterpret_cast<int*>(twy + g.ny);
     // in the ny ints after posx that only the forward pass uses (plane_smem_bytes)
     uint64_t* bar = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(posx + nx) + 7) & ~uintptr_t(7));
@@ -1229,8 +1587,8 @@ __global__ void __launch_bounds__(inv_stream_max_threads<T>()) k_plane_inv_strea
     const int nx = g.nx, ny = g.ny, plane = ny * g.nxh;
     const uint32_t bytes = (uint32_t)(plane * sizeof(C));  // multiple of 16 (ny even)
     C* buf[2] = {reinterpret_cast<C*>(sm_raw), reinterpret_cast<C*>(sm_raw) + plane};
-    C* twx = buf[1] + plane;
-    C* twy = twx + nx;
+    auto* twx = reinterpret_cast<typename TwT<T>::t*>(buf[1] + plane);
+    auto* twy = twx + nx;
     int* posx = reinterpret_cast<int*>(twy + ny);
     uint64_t* bar = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(posx + nx) + 7) & ~uintptr_t(7));
     const int total = 9 * g.nz;
@@ -1272,6 +1630,8 @@ __global__ void __launch_bounds__(inv_stream_max_threads<T>()) k_plane_inv_strea
 }
 
 // ---------------------------------------------------------------- pass 3 for two-stage plans, register-staged
+// (FP32; FP64 runs the generic pass: with its transforms on integers the register-staged form, which inlines
+// five butterflies, was slower -- 260 against 229 us at 128 x 128 x 64 -- and starved for instructions)
 // For planes with nx = ny = n = R1 R2 and the two-stage plans 16 x 8 (n = 128)
 // and 8 x 8 (n = 64): the operations of plane_inv_compute in the same order
 // (bit-identical results) with half its passes over shared memory.  Each
@@ -1343,8 +1703,8 @@ __device__ __forceinline__ void inv2_x1(typename C2<T>::t* s, int wg, int lane) 
     for (int q = HQ + 1; q < R2; ++q) za[q] = u0 ? m1[R2 - q] : m2[R2 - 1 - q];
 #pragma unroll
     for (int q = HQ; q < R2; ++q) zb[q] = u0 ? m2[R2 - 1 - q] : m1[R2 - 1 - q];
-    Bfly<R2, true, C>::run(za);
-    Bfly<R2, true, C>::run(zb);
+    bfly<R2, true>(za, false, no_tw<C>);
+    bfly<R2, true>(zb, false, no_tw<C>);
     __syncwarp();  // every lane of the warp has read its rows before any is overwritten
 #pragma unroll
     for (int q = 0; q < R2; ++q) {
@@ -1354,22 +1714,18 @@ __device__ __forceinline__ void inv2_x1(typename C2<T>::t* s, int wg, int lane) 
 }
 
 template <typename T, int R1, int R2>
-__device__ __forceinline__ void inv2_x2(const typename C2<T>::t* s, const typename C2<T>::t* twx2, T* __restrict__ yp,
+__device__ __forceinline__ void inv2_x2(const typename C2<T>::t* s, const typename TwT<T>::t* twx2, T* __restrict__ yp,
                                         T sc, T ad, int wg, int lane) {
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, R2>;
     const int k = lane / P::L2, j = lane % P::L2;
     const int r = inv2_pair(wg, k, P::G2, P::S2);
     const C* Z = s + 2 * r * P::nxh;
-    const C* tw = twx2 + j * P::TWS;  // tw[p] = W_n^(p j)
+    const auto* tw = twx2 + j * P::TWS;  // tw[p] = W_n^(p j)
     C v[R1];
 #pragma unroll
     for (int q = 0; q < R1; ++q) v[q] = Z[swz8(j + R2 * q)];
-    if (j) {
-#pragma unroll
-        for (int p = 1; p < R1; ++p) v[p] = cmulc(v[p], tw[p]);
-    }
-    Bfly<R1, true, C>::run(v);
+    bfly<R1, true>(v, j != 0, [&](int p) { return tw[p]; });
     T* y0 = yp + (long long)(2 * r) * P::n;
 #pragma unroll
     for (int q = 0; q < R1; ++q) {
@@ -1384,8 +1740,8 @@ template <typename T, int BT> constexpr int inv2_min_blocks() { return sizeof(T)
 
 // Y1 .. X2 of one plane already in shared memory s (twiddle tables loaded); writes plane (c, z) of y.
 template <typename T, int R1, int R2>
-__device__ __forceinline__ void inv2_compute(typename C2<T>::t* s, const typename C2<T>::t* twy,
-                                             const typename C2<T>::t* twx2, T* __restrict__ y, const GridDev& g,
+__device__ __forceinline__ void inv2_compute(typename C2<T>::t* s, const typename TwT<T>::t* twy,
+                                             const typename TwT<T>::t* twx2, T* __restrict__ y, const GridDev& g,
                                              const OutArgs& oa, const int c, const int z) {
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, R2>;
@@ -1405,7 +1761,7 @@ __device__ __forceinline__ void inv2_compute(typename C2<T>::t* s, const typenam
                 v[q] = mk<C>(v[q].x - w.y, v[q].y + w.x);
             }
         }
-        Bfly<R2, true, C>::run(v);
+        bfly<R2, true>(v, false, no_tw<C>);
 #pragma unroll
         for (int q = 0; q < R2; ++q) b[q * nxh] = v[q];
     }
@@ -1417,11 +1773,7 @@ __device__ __forceinline__ void inv2_compute(typename C2<T>::t* s, const typenam
         C v[R1];
 #pragma unroll
         for (int q = 0; q < R1; ++q) v[q] = b[q * R2 * nxh];
-        if (j) {
-#pragma unroll
-            for (int p = 1; p < R1; ++p) v[p] = cmulc(v[p], twy[p * j]);
-        }
-        Bfly<R1, true, C>::run(v);
+        bfly<R1, true>(v, j != 0, [&](int p) { return twy[p * j]; });
 #pragma unroll
         for (int q = 0; q < R1; ++q) b[q * R2 * nxh] = v[q];
     }
@@ -1452,8 +1804,8 @@ __global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(con
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* s = reinterpret_cast<C*>(sm_raw);  // [n][nxh]
-    C* twy = s + n * nxh;                  // [n]: W_n^k of the y axis
-    C* twx2 = twy + n;                     // [R2][R1 + 1]: W_n^(p j) of the x axis
+    auto* twy = reinterpret_cast<typename TwT<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
+    auto* twx2 = twy + n;                     // [R2][R1 + 1]: W_n^(p j) of the x axis
     uint64_t* bar =
         reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(twx2 + R2 * P::TWS) + 7) & ~uintptr_t(7));
     const int c = blockIdx.x, z = blockIdx.y;
@@ -1468,7 +1820,7 @@ __global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(con
     for (int i = tid; i < n; i += nthr) twy[i] = twp<T>(g, 1)[i];
     for (int i = tid; i < R2 * P::TWS; i += nthr) {
         const int j = i / P::TWS, p = i - j * P::TWS;
-        twx2[i] = p < R1 ? twp<T>(g, 0)[p * j] : mk<C>((T)0, (T)0);
+        twx2[i] = p < R1 ? twp<T>(g, 0)[p * j] : typename TwT<T>::t{};
     }
     const bool ok = mbar_wait(bar, 0u, g.wait_cycles);
     if (__syncthreads_or(!ok)) {
@@ -1496,15 +1848,15 @@ __global__ void __launch_bounds__(BT, 1) k_plane_inv2s(const typename C2<T>::t* 
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* buf[2] = {reinterpret_cast<C*>(sm_raw), reinterpret_cast<C*>(sm_raw) + plane};
-    C* twy = buf[1] + plane;
-    C* twx2 = twy + n;
+    auto* twy = reinterpret_cast<typename TwT<T>::t*>(buf[1] + plane);
+    auto* twx2 = twy + n;
     uint64_t* bar = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(twx2 + 8 * P::TWS) + 7) & ~uintptr_t(7));
     const uint32_t bytes = (uint32_t)(plane * sizeof(C));  // a multiple of 16 (n even)
     const int total = 9 * g.nz, tid = threadIdx.x, nthr = blockDim.x;
     for (int i = tid; i < n; i += nthr) twy[i] = twp<T>(g, 1)[i];
     for (int i = tid; i < 8 * P::TWS; i += nthr) {
         const int j = i / P::TWS, q = i - j * P::TWS;
-        twx2[i] = q < R1 ? twp<T>(g, 0)[q * j] : mk<C>((T)0, (T)0);
+        twx2[i] = q < R1 ? twp<T>(g, 0)[q * j] : typename TwT<T>::t{};
     }
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -1578,7 +1930,7 @@ int inv2_radix(const GridDev& g) {
 // (Forming K:x in registers at the X1 positions, scalar loads 8 voxels apart,
 // measured 1.3x slower in FP32 at 128^3 than these 16-byte loads.)
 template <typename T, int R1>
-__device__ __forceinline__ void fwd2_x1(typename C2<T>::t* s, const typename C2<T>::t* twx2, int wg, int lane) {
+__device__ __forceinline__ void fwd2_x1(typename C2<T>::t* s, const typename TwT<T>::t* twx2, int wg, int lane) {
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, 8>;
     const int k = lane / P::L2, j = lane % P::L2;
@@ -1587,12 +1939,8 @@ __device__ __forceinline__ void fwd2_x1(typename C2<T>::t* s, const typename C2<
     C v[R1];
 #pragma unroll
     for (int n1 = 0; n1 < R1; ++n1) v[n1] = Z[j + 8 * n1];
-    Bfly<R1, false, C>::run(v);
-    if (j) {
-        const C* tw = twx2 + j * P::TWS;
-#pragma unroll
-        for (int p = 1; p < R1; ++p) v[p] = cmul(v[p], tw[p]);
-    }
+    const auto* tw = twx2 + j * P::TWS;
+    bfly<R1, false>(v, j != 0, [&](int p) { return tw[p]; });
     __syncwarp();  // every lane of the warp has read its packed row before it is overwritten
 #pragma unroll
     for (int p = 0; p < R1; ++p) Z[swz8(j + 8 * p)] = v[p];
@@ -1613,8 +1961,8 @@ __device__ __forceinline__ void fwd2_x2(typename C2<T>::t* s, int wg, int lane) 
         za[q] = A[swz8(c1 * R2 + q)];
         zb[q] = A[swz8(c2 * R2 + q)];
     }
-    Bfly<R2, false, C>::run(za);
-    Bfly<R2, false, C>::run(zb);
+    bfly<R2, false>(za, false, no_tw<C>);
+    bfly<R2, false>(zb, false, no_tw<C>);
     // za[q] holds frequency c1 + R1 q, zb[q] frequency c2 + R1 q; the mirror n - k of
     // c1 + R1 q is c2 + R1 (R2-1-q) for c1 != 0 and R1 (R2 - q) for c1 = 0
     __syncwarp();  // every lane of the warp has read its packed row before the rows are written
@@ -1656,14 +2004,14 @@ __global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(con
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* s = reinterpret_cast<C*>(sm_raw);  // [n][nxh]
-    C* twy = s + n * nxh;                  // [n]: W_n^k of the y axis
-    C* twx2 = twy + n;                     // [8][R1 + 1]: W_n^(p j) of the x axis
+    auto* twy = reinterpret_cast<typename TwT<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
+    auto* twx2 = twy + n;                     // [8][R1 + 1]: W_n^(p j) of the x axis
     const int c = blockIdx.x, z = blockIdx.y;
     const int tid = threadIdx.x, nthr = blockDim.x;
     for (int i = tid; i < n; i += nthr) twy[i] = twp<T>(g, 1)[i];
     for (int i = tid; i < R2 * P::TWS; i += nthr) {
         const int j = i / P::TWS, p = i - j * P::TWS;
-        twx2[i] = p < R1 ? twp<T>(g, 0)[p * j] : mk<C>((T)0, (T)0);
+        twx2[i] = p < R1 ? twp<T>(g, 0)[p * j] : typename TwT<T>::t{};
     }
     plane_contract<T, true, true>(s, x, K, g, c, z, nxh);
     __syncthreads();
@@ -1687,11 +2035,7 @@ __global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(con
         C v[R1];
 #pragma unroll
         for (int q = 0; q < R1; ++q) v[q] = b[q * R2 * nxh];
-        Bfly<R1, false, C>::run(v);
-        if (j) {
-#pragma unroll
-            for (int p = 1; p < R1; ++p) v[p] = cmul(v[p], twy[p * j]);
-        }
+        bfly<R1, false>(v, j != 0, [&](int p) { return twy[p * j]; });
 #pragma unroll
         for (int q = 0; q < R1; ++q) b[q * R2 * nxh] = v[q];
     }
@@ -1704,7 +2048,7 @@ __global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(con
         C v[R2];
 #pragma unroll
         for (int q = 0; q < R2; ++q) v[q] = b[q * nxh];
-        Bfly<R2, false, C>::run(v);
+        bfly<R2, false>(v, false, no_tw<C>);
         if (col == 0) {
 #pragma unroll
             for (int q = 0; q < R2; ++q) b[q * nxh] = v[q];
@@ -1737,7 +2081,7 @@ template <typename T> size_t zproj_smem(const GridDev& g, int W = zproj_width<T>
     return (size_t)3 * g.nz * W * sizeof(C) + ztables_bytes<T>(g.nz, g.ny, g.nxh, W) + 16;
 }
 
-constexpr size_t SMEM_MAX = 227 * 1024;
+constexpr size_t SMEM_MAX = 227 * 1024 - 1024;  // the FP64 transforms' line keys take up to 1 kB of static shared memory
 
 // 16-byte vector access needs nx to hold whole vectors and 16-byte aligned bases
 // (N is a multiple of 4 because nx and ny are even, so component offsets keep the alignment)
@@ -1791,6 +2135,11 @@ int axis_freq_of_pos(int pos, const AxisPlan& p) {
     return f;
 }
 
+cudaError_t fill_rq2(const GridDev& g, double* tab, cudaStream_t st) {
+    k_fill_rq2<<<608, 256, 0, st>>>(g, tab);
+    return cudaGetLastError();
+}
+
 size_t plane_smem_bytes(int nx, int ny, int elem) {
     return (size_t)ny * (nx / 2 + 1) * elem + (size_t)(nx + ny) * elem + (size_t)(nx + ny) * sizeof(int) + 16;
 }
@@ -1802,7 +2151,9 @@ cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, ty
                        const int* skip, cudaStream_t st, bool vin, int planes = 0) {
     // planes > 0: that many z-planes from the ones x, K and spec point at (a chunk of the grid)
     const int nzl = planes > 0 ? planes : g.nz;
-    if (threads < 0 && !(K && vin)) threads = -threads;  // projection alone, unaligned: the generic pass
+    // projection alone, unaligned, FP64 (its lines run in fixed point, in the generic pass only): the generic pass
+    if (threads < 0 && (sizeof(T) == 8 || !(K && vin))) threads = -threads;
+    if constexpr (sizeof(T) == 4)
     if (threads < 0) {  // register-staged pass of the two-stage plans (nx = ny = 64 or 128), -threads threads
         const size_t sm = fwd2_smem<T>(g);
         const dim3 grid(9, nzl);
@@ -1962,10 +2313,14 @@ template <typename T, int W>
 cudaError_t launch_z_tma_w(gff_handle* h, int threads, int blocks, const ProjArgs& pa, const int* skip,
                            cudaStream_t st) {
     if (blocks > 0) return launch_z_tma_k<T, W, 0>(h, threads, blocks, pa, skip, st);
-    switch (z2_radix(h->g)) {
-        case 16: return launch_z_tma_k<T, W, 16>(h, threads, -blocks, pa, skip, st);
-        case 8: return launch_z_tma_k<T, W, 8>(h, threads, -blocks, pa, skip, st);
-        default: return cudaErrorInvalidValue;
+    if constexpr (sizeof(T) == 8) {  // FP64: the generic strip, whose lines run in fixed point
+        return launch_z_tma_k<T, W, 0>(h, threads, -blocks, pa, skip, st);
+    } else {
+        switch (z2_radix(h->g)) {
+            case 16: return launch_z_tma_k<T, W, 16>(h, threads, -blocks, pa, skip, st);
+            case 8: return launch_z_tma_k<T, W, 8>(h, threads, -blocks, pa, skip, st);
+            default: return cudaErrorInvalidValue;
+        }
     }
 }
 
@@ -2009,10 +2364,15 @@ int z_tma_blocks_k(gff_handle* h, int threads) {
 template <typename T, int W>
 int z_tma_blocks_w(gff_handle* h, int threads, bool reg) {
     if (!reg) return z_tma_blocks_k<T, W, 0>(h, threads);
-    switch (z2_radix(h->g)) {
-        case 16: return z_tma_blocks_k<T, W, 16>(h, threads);
-        case 8: return z_tma_blocks_k<T, W, 8>(h, threads);
-        default: return 0;
+    const int r1 = z2_radix(h->g);
+    if constexpr (sizeof(T) == 8) {
+        return r1 && ztma_threads_ok<T>(r1, threads) ? z_tma_blocks_k<T, W, 0>(h, threads) : 0;
+    } else {
+        switch (r1) {
+            case 16: return z_tma_blocks_k<T, W, 16>(h, threads);
+            case 8: return z_tma_blocks_k<T, W, 8>(h, threads);
+            default: return 0;
+        }
     }
 }
 // > 0 blocks of the generic TMA z pass (reg false) or of the register-staged one (reg true); 0 if it cannot run
@@ -2027,6 +2387,8 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
     // planes > 0 (one block per plane only): that many z-planes from the ones spec and y point at
     const int nzl = planes > 0 ? planes : g.nz;
     if (planes > 0 && blocks != 0 && blocks != -1) return cudaErrorInvalidValue;
+    if (sizeof(T) == 8 && blocks < 0) blocks = 0;  // FP64: the generic pass, whose lines run in fixed point
+    if constexpr (sizeof(T) == 4) {
     if (blocks < -1) {  // register-staged persistent pass, -blocks blocks
         const size_t sm = inv2s_smem<T>(g);
         const int r1 = inv2_radix(g);
@@ -2038,10 +2400,8 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
     }
         GFF_INV2S(16, 512)
         GFF_INV2S(8, 512)
-        if constexpr (sizeof(T) == 4) {
-            GFF_INV2S(16, 1024)
-            GFF_INV2S(8, 1024)
-        }
+        GFF_INV2S(16, 1024)
+        GFF_INV2S(8, 1024)
 #undef GFF_INV2S
         return cudaErrorInvalidValue;
     }
@@ -2061,6 +2421,7 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
         GFF_INV2(8, 512)
 #undef GFF_INV2
         return cudaErrorInvalidValue;
+    }
     }
     if (blocks > 0) {
         const size_t sm = plane_stream_smem<T>(g);
@@ -2141,28 +2502,32 @@ int inv_stream_blocks(const GridDev& g, int threads, bool vout) {
 
 // blocks of the persistent register-staged inverse pass: all that fit at once, at most one per plane; 0 if it
 // cannot run on this grid (plan, shared memory) with this many threads
-template <typename T, int R1, int BT>
-int inv2s_blocks_k(const GridDev& g) {
-    const size_t sm = inv2s_smem<T>(g);
-    int dev = 0, nsm = 0, per = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    allow_smem(k_plane_inv2s<T, R1, BT>, sm);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_plane_inv2s<T, R1, BT>, BT, sm) != cudaSuccess ||
-        per < 1)
+template <int R1, int BT>
+int inv2s_blocks_k(const GridDev& g, int nsm) {
+    const size_t sm = inv2s_smem<float>(g);
+    int per = 0;
+    allow_smem(k_plane_inv2s<float, R1, BT>, sm);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_plane_inv2s<float, R1, BT>, BT, sm) != cudaSuccess || per < 1)
         return 0;
-    const int total = 9 * g.nz;
-    return nsm * per < total ? nsm * per : total;
+    return nsm * per;
 }
 template <typename T>
 int inv2s_blocks(const GridDev& g, int threads) {
     if (inv2s_smem<T>(g) > SMEM_MAX) return 0;
     const int r1 = inv2_radix(g);
-    if (threads == 512) return r1 == 16 ? inv2s_blocks_k<T, 16, 512>(g) : (r1 == 8 ? inv2s_blocks_k<T, 8, 512>(g) : 0);
-    if constexpr (sizeof(T) == 4)
-        if (threads == 1024)
-            return r1 == 16 ? inv2s_blocks_k<T, 16, 1024>(g) : (r1 == 8 ? inv2s_blocks_k<T, 8, 1024>(g) : 0);
-    return 0;
+    int dev = 0, nsm = 0;
+    if (!r1 || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    int n = 0;
+    if constexpr (sizeof(T) == 8) {
+        n = threads == 512 ? nsm : 0;  // accepted; runs as one block per plane (launch_inv)
+    } else {
+        if (threads == 512) n = r1 == 16 ? inv2s_blocks_k<16, 512>(g, nsm) : inv2s_blocks_k<8, 512>(g, nsm);
+        if (threads == 1024) n = r1 == 16 ? inv2s_blocks_k<16, 1024>(g, nsm) : inv2s_blocks_k<8, 1024>(g, nsm);
+    }
+    const int total = 9 * g.nz;
+    return n < total ? n : total;
 }
 
 template <typename T>
@@ -2175,7 +2540,8 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     Tune& tn = h->tune[tune_index<T>()];
     const bool vin = vec_ok<T>(g, x) && vec_ok<T>(g, K);
     // forward pass: 256 or 512 threads, or (two-stage plans, nx = ny) the register-staged pass (-256, -512)
-    const bool f2 = inv2_radix(g) > 0 && fwd2_smem<T>(g) <= SMEM_MAX;
+    const bool staged = sizeof(T) == 4;  // FP64 maps the register-staged shapes onto the generic passes
+    const bool f2 = staged && inv2_radix(g) > 0 && fwd2_smem<T>(g) <= SMEM_MAX;
     const int tp[4] = {256, 512, -256, -512};
     const bool tv[4] = {true, true, f2, f2};
     int b = -1;
@@ -2197,7 +2563,7 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
         zv[i] = zb[i] > 0;
     }
     for (int i = 15; i < NZC; ++i) {  // negative: register-staged strip
-        zb[i] = -z_tma_blocks<T>(h, wz[i], tz[i], true);
+        zb[i] = staged ? -z_tma_blocks<T>(h, wz[i], tz[i], true) : 0;
         zv[i] = zb[i] < 0;
     }
     ProjArgs pa;
@@ -2220,8 +2586,8 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     const bool vout = vec_ok<T>(g, y);
     const int ti[8] = {256, 512, inv_stream_max_threads<T>() / 2, inv_stream_max_threads<T>(), 256, 512, 512, 1024};
     int ib[8] = {0, 0, inv_stream_blocks<T>(g, 512, vout), inv_stream_blocks<T>(g, 1024, vout), -1, -1,
-                 -inv2s_blocks<T>(g, 512), -inv2s_blocks<T>(g, 1024)};
-    const bool r2 = inv2_radix(g) > 0 && inv2_smem<T>(g) <= SMEM_MAX;
+                 staged ? -inv2s_blocks<T>(g, 512) : 0, staged ? -inv2s_blocks<T>(g, 1024) : 0};
+    const bool r2 = staged && inv2_radix(g) > 0 && inv2_smem<T>(g) <= SMEM_MAX;
     const bool iv[8] = {true, true, ib[2] > 0, ib[3] > 0, r2, r2, ib[6] < -1, ib[7] < -1};
     int* err = h->d_flag + 2;
     e = pick_fastest(8, iv, reps, st, [&](int i) { return launch_inv<T>(g, ti[i], ib[i], spec, y, oa, nullptr, st, vout, err); }, &b);
@@ -2313,7 +2679,7 @@ __global__ void __launch_bounds__(512) k_plane_fwd_batch(const RveApply* __restr
 }
 
 template <typename T, int W>
-__global__ void __launch_bounds__(256) k_zproj_batch(const RveApply* __restrict__ rv, const int* __restrict__ start,
+__global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj_batch(const RveApply* __restrict__ rv, const int* __restrict__ start,
                                                     int n, ProjArgs pa) {
     const int r = find_rve(start, n, blockIdx.x);
     const RveApply& a = rv[r];
@@ -2400,6 +2766,8 @@ cudaError_t launch_galerkin(const gff_handle* h, const T* x, const T* K, T* y, c
     const Tune& tn = h->tune[tune_index<T>()];
     const bool vin = vec_ok<T>(g, x) && (!K || vec_ok<T>(g, K));
     const bool vout = vec_ok<T>(g, y);
+    OutArgs oo = oa;
+    oo.pre = pa.sym ? 0 : 1;
     if (ev) cudaEventRecord(ev[0], h->stream);
     cudaError_t e = launch_fwd<T>(g, tn.t_fwd, x, K, spec, skip, h->stream, vin);
     if (e != cudaSuccess) return e;
@@ -2413,7 +2781,7 @@ cudaError_t launch_galerkin(const gff_handle* h, const T* x, const T* K, T* y, c
         e = launch_z<T>(g, tn.wz, tn.t_z, spec, pa, skip, h->stream);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[2], h->stream);
-    e = launch_inv<T>(g, tn.t_inv, tn.inv_blocks, spec, y, oa, skip, h->stream, vout, h->d_flag + 2);
+    e = launch_inv<T>(g, tn.t_inv, tn.inv_blocks, spec, y, oo, skip, h->stream, vout, h->d_flag + 2);
     if (ev) cudaEventRecord(ev[3], h->stream);
     return e;
 }
@@ -2454,6 +2822,8 @@ cudaError_t launch_galerkin_host(gff_handle* h, const T* x_host, T* y_host, T* x
     cudaEvent_t* ev = h->pipe_ev;  // [0] start, [1] done, [2, 2 + nch) copied in, [2 + nch, 2 + 2 nch) computed
     const bool vin = vec_ok<T>(g, xd) && vec_ok<T>(g, K);
     const bool vout = vec_ok<T>(g, yd);
+    OutArgs oo = oa;
+    oo.pre = pa.sym ? 0 : 1;
     int t_inv = tn.t_inv, b_inv = tn.inv_blocks;
     if (b_inv < -1) {
         t_inv = 256;
@@ -2487,7 +2857,7 @@ cudaError_t launch_galerkin_host(gff_handle* h, const T* x_host, T* y_host, T* x
     if (e != cudaSuccess) return e;
     for (int c = 0; c < nch; ++c) {
         const int z0 = c * g.nz / nch, z1 = (c + 1) * g.nz / nch;
-        e = launch_inv<T>(g, t_inv, b_inv, spec + z0 * pspec, yd + z0 * plane, oa, nullptr, st, vout, h->d_flag + 2,
+        e = launch_inv<T>(g, t_inv, b_inv, spec + z0 * pspec, yd + z0 * plane, oo, nullptr, st, vout, h->d_flag + 2,
                           z1 - z0);
         if (e == cudaSuccess) e = cudaEventRecord(ev[2 + nch + c], st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, ev[2 + nch + c], 0);
@@ -2528,7 +2898,7 @@ constexpr long long NOALLOC_MAX_VOXELS = 32768;  // e.g. 32^3, 16 x 32 x 64, ...
 constexpr size_t NOALLOC_SPEC_BYTES = 9ull * (NOALLOC_MAX_VOXELS / 4 * 3) * sizeof(double2);
 
 struct NoallocTables {
-    double2 tw64[3][MAXN];
+    int4 tw64[3][MAXN];
     float2 tw32[3][MAXN];
     int posx[MAXN], fqy[MAXN], fqz[MAXN];
     double qt64[2][3][MAXN];
@@ -2592,7 +2962,9 @@ __global__ void k_noalloc_tables(NoallocTables* t, AxisPlan ax, AxisPlan ay, Axi
         for (int k = threadIdx.x; k < n; k += blockDim.x) {
             double sn, cs;
             sincospi(2.0 * k / n, &sn, &cs);
-            t->tw64[a][k] = make_double2(cs, -sn);
+            const double one = 4611686018427387904.0;  // 2^62
+            const int2 re = twiddle_limbs(llrint(cs * one)), im = twiddle_limbs(llrint(-sn * one));
+            t->tw64[a][k] = make_int4(re.x, re.y, im.x, im.y);
             t->tw32[a][k] = make_float2((float)cs, (float)-sn);
             const int kappa = (2 * k < n) ? k : k - n;
             const double qc = 2.0 * 3.141592653589793238462643383279502884 * kappa / L[a];
@@ -2680,6 +3052,7 @@ __attribute__((visibility("default"))) gff_status gff_project_noalloc(const gff_
             g.qt32[kind][a] = dt->qt32[kind][a];
         }
     }
+    g.rq2[0] = g.rq2[1] = nullptr;
     g.posx = dt->posx;
     g.fqy = dt->fqy;
     g.fqz = dt->fqz;

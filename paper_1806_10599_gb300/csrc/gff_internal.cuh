@@ -18,6 +18,16 @@ constexpr int NSLIP = 12;
 template <typename T> struct C2;
 template <> struct C2<double> { using t = double2; };
 template <> struct C2<float> { using t = float2; };
+// twiddles: FP32 complex; for FP64 data 62-bit fixed point in limbs (re high, re low, im high, im low; fixed_bfly.cuh)
+template <typename T> struct TwT;
+template <> struct TwT<double> { using t = int4; };
+template <> struct TwT<float> { using t = float2; };
+// limbs (h, l), c = h 2^32 + l with |l| <= 2^31 - 1 or l = -2^31 avoided by moving one unit: c is changed by at most 2^-62
+inline __host__ __device__ int2 twiddle_limbs(long long c) {
+    long long l = c - (((c + 0x80000000LL) >> 32) << 32);
+    if (l == -0x80000000LL) ++l, ++c;
+    return make_int2((int)((c - l) >> 32), (int)l);
+}
 
 // Mixed-radix plan of one axis: n = radix[0] * ... * radix[nst-1].
 // The forward transform is decimation in frequency in place: natural input,
@@ -35,13 +45,15 @@ struct GridDev {
     int nx, ny, nz, nxh;
     long long N;
     AxisPlan ax, ay, az;
-    const double2* tw64[3];  // W_n^k = exp(-2 pi i k / n), k < n, per axis (x, y, z)
+    const int4* tw64[3];     // W_n^k = exp(-2 pi i k / n), k < n, per axis (x, y, z), in limbs (TwT)
     const float2* tw32[3];
     const int* posx;         // [nx]: position of natural frequency kx after the forward x pass
     const int* fqy;          // [ny]: frequency held at position py after the forward y pass
     const int* fqz;          // [nz]
     const double* qt64[2][3];  // [kind][axis][k]: q~ (continuous) or q~' (discrete) per FFT index
     const float* qt32[2][3];
+    const double* rq2[2];      // [kind][nz][ny nxh] in the order of the half spectrum: 1 / (N |q|^2), 0 where the projection
+                               // is zero or special (null: the z pass divides instead)
     long long wait_cycles;     // budget of the first wait on each bulk load (BULK_WAIT_CYCLES by default)
 };
 
@@ -56,6 +68,7 @@ struct ProjArgs {
 struct OutArgs {
     double scale;
     double add[9];
+    int pre = 1;  // FP64: 1: the z pass has multiplied by 1 / N = |scale| already; 0 (small strain): it has not
 };
 
 // ---- batched launches: one launch serves several RVEs of different sizes.
@@ -141,6 +154,7 @@ struct gff_handle {
     int nxh = 0;
     gff::GridDev g{};
     void* tables = nullptr;  // backing store of GridDev pointers
+    double* d_rq2 = nullptr;  // backing store of GridDev::rq2
 
     // microstructure
     int ngrains = 0;
@@ -252,6 +266,8 @@ template <typename T>
 cudaError_t launch_galerkin_host(gff_handle* h, const T* x_host, T* y_host, T* xd, T* yd, const T* K,
                                  const ProjArgs& pa, const OutArgs& oa, typename C2<T>::t* spec);
 size_t plane_smem_bytes(int nx, int ny, int elem);
+// fills GridDev::rq2 (tab: 2 nz ny nxh doubles) from the grid's other tables
+cudaError_t fill_rq2(const GridDev& g, double* tab, cudaStream_t st);
 // Mixed-radix plan of one axis (false: n unsupported) and the frequency held
 // at position pos after the forward (decimation in frequency) transform:
 // pos = sum_i p_i m_i with m_i = n / (r_0 ... r_i), frequency p_0 + r_0 p_1 + ...
