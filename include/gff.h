@@ -275,10 +275,9 @@ gff_status gff_set_strain_measure(gff_handle* h, int mode);
  *   gff_step_report.cp_fallbacks);
  * GFF_RETURN_MAP_F32_FIRST: the same FP64 iteration preceded by that
  *   iteration in FP32 (elastic state formed from the small quantities F - I
- *   and Fp^-1 - I) down to FP32 resolution and then with its residual in sums
- *   of two floats down to the tolerance; the FP64 iteration then starts from
- *   its root.  The FP64 residual still decides convergence, so the root is
- *   GFF_RETURN_MAP_FP64's to the return-map tolerance;
+ *   and Fp^-1 - I) down to FP32 resolution; the FP64 iteration then starts
+ *   from its root.  The FP64 residual still decides convergence, so the root
+ *   is GFF_RETURN_MAP_FP64's to the return-map tolerance;
  * GFF_RETURN_MAP_DEFAULT (a new handle's mode): GFF_RETURN_MAP_F32_FIRST when
  *   the handle's precision is GFF_PREC_MIXED, GFF_RETURN_MAP_FP64 in
  *   GFF_PREC_FP64;

@@ -309,14 +309,6 @@ gff_status upload_grains(gff_handle* h, const std::vector<double>& quat, const s
             for (int k = 0; k < 12; ++k) d[G32_NRM + k] = (float)geo[GEO_NRM + k];
             for (int k = 0; k < 36; ++k) d[G32_C6 + k] = (float)geo[GEO_C6 + k];
             for (int k = 0; k < 85; ++k) d[G32_PC + k] = (float)nrmprm[41 * (size_t)ng + 144 * (size_t)g + k];
-            auto pair = [&](int at, double v) {
-                const float hi = (float)v;
-                d[G32_FF + 2 * at] = hi;
-                d[G32_FF + 2 * at + 1] = (float)(v - (double)hi);
-            };
-            for (int k = 0; k < 36; ++k) pair(GFF_DIR + k, geo[GEO_DIR + k]);
-            for (int k = 0; k < 12; ++k) pair(GFF_NRM + k, geo[GEO_NRM + k]);
-            for (int k = 0; k < 36; ++k) pair(GFF_C6 + k, geo[GEO_C6 + k]);
         }
         GFF_TRY(cudaMemcpy(h->d_geo32, g32.data(), g32.size() * sizeof(float), cudaMemcpyHostToDevice));
     }

@@ -141,11 +141,7 @@ constexpr int GEO_S0 = 0, GEO_DIR = 108, GEO_NRM = 144, GEO_C6 = 156, GEO_STRIDE
 // pre-iteration of the return map (slip directions [12][3], plane normals
 // [4][3], Voigt stiffness [6][6], the small-strain factors P [5][12] and
 // C5^-1 [5][5]).
-constexpr int G32_S0 = 0, G32_C = 108, G32_DIR = 189, G32_NRM = 225, G32_C6 = 237, G32_PC = 273;
-// the slip directions, plane normals and Voigt stiffness again as unevaluated sums of two floats (pairs h, l; 8-byte
-// aligned), for the refinement in float pairs
-constexpr int G32_FF = 384, GFF_DIR = 0, GFF_NRM = 36, GFF_C6 = 48, GFF_COUNT = 84, G32_STRIDE = 576;
-static_assert(G32_FF + 2 * GFF_COUNT <= G32_STRIDE && G32_STRIDE % 2 == 0, "float pairs fit");
+constexpr int G32_S0 = 0, G32_C = 108, G32_DIR = 189, G32_NRM = 225, G32_C6 = 237, G32_PC = 273, G32_STRIDE = 384;
 
 }  // namespace gff
 

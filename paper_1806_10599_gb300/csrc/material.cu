@@ -15,13 +15,12 @@
 // Newton iterate when there is one (else from 0) and takes its steps with the
 // per-grain small-elastic-strain Jacobian, solved as a 5x5 system on the
 // deviatoric strains (cp_correction_lowrank); the residual is always exact,
-// so it converges to the same root.  In mixed precision it first runs in FP32
-// and then in float pairs, and FP64 confirms (cp_presolve_f32, cp_refine_ff).  The exact 12x12 Jacobian is assembled
+// so it converges to the same root.  The exact 12x12 Jacobian is assembled
 // once, at the root, for the tangent (LU with partial pivoting).  If the fast
 // iteration fails, the return map restarts from dg = 0 with exact Newton
 // steps (12x12 LU with partial pivoting) -- the fallback; a handle can also
 // ask for that exact iteration alone (gff_set_return_map).
-// Otherwise everything is FP64.  One thread per voxel.
+// Everything is FP64.  One thread per voxel.
 #include <cmath>
 
 #include "gff_internal.cuh"
@@ -635,204 +634,6 @@ __device__ __noinline__ bool cp_presolve_f32(const double* F, const double* A, c
     return false;
 }
 
-// ---------------------------------------------------------------- refinement in float pairs
-// The same iteration once more, with the residual in unevaluated sums of two floats (about 47 bits)
-// and the corrections in FP32: from FP32 resolution down to the return map's tolerance at FP32
-// rates (an SM executes 128 FP32 operations per clock and 2 in FP64; a residual takes about 6000
-// of the former or 480 of the latter, 47 against 240 clocks).  The elastic state is formed from
-// f = F - I and a = Fp^-1_n - I as in the FP32 pre-iteration, so E keeps 47 relative bits where
-// Ce - I in FP64 keeps about 43.  The FP64 iteration that follows evaluates its residual at the
-// result and is done if that is within the tolerance; it decides convergence as before.
-// Increments of a 64^3 history at return-map tolerance 1e-14, return maps: 12.2 -> 5.6 ms (the FP64
-// iteration took 2.4 corrections per evaluation before and none now).  What bounds it: issue of the
-// FP32 instructions at 8 warps per SM, then the one FP64 residual.
-struct ff {
-    float h, l;
-};
-__device__ __forceinline__ ff ff_quick(float s, float t) {  // s + t, |s| >= |t|
-    const float h = __fadd_rn(s, t);
-    return ff{h, __fsub_rn(t, __fsub_rn(h, s))};
-}
-__device__ __forceinline__ ff ff_two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    return ff{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb))};
-}
-__device__ __forceinline__ ff ff_neg(ff a) { return ff{-a.h, -a.l}; }
-__device__ __forceinline__ ff ff_add(ff a, ff b) {
-    const ff s = ff_two_sum(a.h, b.h);
-    return ff_quick(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ ff ff_mul(ff a, ff b) {
-    const float p = __fmul_rn(a.h, b.h);
-    return ff_quick(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
-}
-// acc + a b, the low part left to grow (ff_norm at the end of a sum)
-__device__ __forceinline__ ff ff_mac(ff acc, ff a, ff b) {
-    const float p = __fmul_rn(a.h, b.h);
-    const float e = __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p)));
-    const ff s = ff_two_sum(acc.h, p);
-    return ff{s.h, __fadd_rn(acc.l, __fadd_rn(s.l, e))};
-}
-__device__ __forceinline__ ff ff_norm(ff a) { return ff_quick(a.h, a.l); }
-__device__ __forceinline__ ff ff_recip(ff a) {  // a not tiny or huge
-    const float q = __frcp_rn(a.h);
-    const float e = __fmaf_rn(-a.l, q, __fmaf_rn(-a.h, q, 1.f));
-    return ff_quick(q, __fmul_rn(q, e));
-}
-__device__ __forceinline__ ff ff_from(double d) {
-    const float h = (float)d;
-    return ff{h, (float)(d - (double)h)};
-}
-__device__ __forceinline__ ff ff_ld(const float* __restrict__ g, int at) {
-    const float2 v = __ldg(reinterpret_cast<const float2*>(g + G32_FF) + at);
-    return ff{v.x, v.y};
-}
-__device__ __forceinline__ void ff_mm(const ff* a, const ff* b, ff* c) {  // c = a b
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-            c[3 * i + j] = ff_norm(ff_mac(ff_mac(ff_mul(a[3 * i], b[j]), a[3 * i + 1], b[3 + j]), a[3 * i + 2], b[6 + j]));
-}
-
-// elastic_tau_f32 in float pairs.  The loops over slip planes stay loops: unrolled, the code of the refinement
-// would not fit the instruction cache.
-__device__ __forceinline__ void elastic_tau_ff(const ff* f, const ff* a, const ff* dg, const float* __restrict__ g, ff* tau) {
-    const ff zero{0.f, 0.f};
-    ff t[9], q[9];
-    {
-        ff Lp[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) Lp[k] = zero;
-#pragma unroll 1
-        for (int p = 0; p < 4; ++p) {
-            ff v[3] = {zero, zero, zero};
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) v[j] = ff_mac(v[j], dg[3 * p + i], ff_ld(g, GFF_DIR + 3 * (3 * p + i) + j));
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                v[j] = ff_norm(v[j]);
-#pragma unroll
-                for (int k = 0; k < 3; ++k) Lp[3 * j + k] = ff_mac(Lp[3 * j + k], v[j], ff_ld(g, GFF_NRM + 3 * p + k));
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) Lp[k] = ff_norm(Lp[k]);
-        ff_mm(a, Lp, t);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) q[k] = ff_add(ff_add(a[k], ff_neg(Lp[k])), ff_neg(t[k]));  // Fp^-1 - I
-    }
-    ff_mm(f, q, t);
-    ff G[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) G[k] = ff_add(ff_add(q[k], f[k]), t[k]);  // Fe - I
-    // 2 E = G + G^T + G^T G in Voigt order 11, 22, 33, 23, 13, 12
-    const int vi[6] = {0, 1, 2, 1, 0, 0}, vj[6] = {0, 1, 2, 2, 2, 1};
-    ff e2[6];
-#pragma unroll
-    for (int I = 0; I < 6; ++I) {
-        const int i = vi[I], j = vj[I];
-        const ff gg = ff_norm(ff_mac(ff_mac(ff_mul(G[i], G[j]), G[3 + i], G[3 + j]), G[6 + i], G[6 + j]));
-        e2[I] = ff_add(ff_add(G[3 * i + j], G[3 * j + i]), gg);
-    }
-    ff sv[6];
-#pragma unroll
-    for (int I = 0; I < 6; ++I) {
-        ff s = zero;
-#pragma unroll
-        for (int J = 0; J < 6; ++J) {  // engineering shears 2 E; normal strains E
-            const ff c = ff_ld(g, GFF_C6 + 6 * I + J);
-            s = ff_mac(s, J < 3 ? ff{0.5f * c.h, 0.5f * c.l} : c, e2[J]);
-        }
-        sv[I] = ff_norm(s);
-    }
-    const ff E2[9] = {e2[0], e2[5], e2[4], e2[5], e2[1], e2[3], e2[4], e2[3], e2[2]};
-    const ff S[9] = {sv[0], sv[5], sv[4], sv[5], sv[1], sv[3], sv[4], sv[3], sv[2]};
-    ff M[9];
-    ff_mm(E2, S, M);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) M[k] = ff_add(M[k], S[k]);  // Ce S
-#pragma unroll 1
-    for (int p = 0; p < 4; ++p) {
-        ff Mm[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            ff s = zero;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) s = ff_mac(s, M[3 * j + k], ff_ld(g, GFF_NRM + 3 * p + k));
-            Mm[j] = ff_norm(s);
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            ff s = zero;
-#pragma unroll
-            for (int j = 0; j < 3; ++j) s = ff_mac(s, Mm[j], ff_ld(g, GFF_DIR + 3 * (3 * p + i) + j));
-            tau[3 * p + i] = ff_norm(s);
-        }
-    }
-}
-
-// Refines dg64 (in/out) until max |r| <= rtol is expected of the FP64 residual; left as it is if the
-// iteration leaves the FP32 range or stalls.  Not inlined: see cp_presolve_f32.
-__device__ __noinline__ void cp_refine_ff(const double* F, const double* A, const double* chin, const float* __restrict__ g,
-                                          const CPParamsDev& pr, double coef, double* dg64) {
-    ff f[9], a[9], chn[NSLIP], dg[NSLIP], tau[NSLIP];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const double I = (k % 4) == 0 ? 1.0 : 0.0;
-        f[k] = ff_from(F[k] - I);
-        a[k] = ff_from(A[k] - I);
-    }
-    for (int s = 0; s < NSLIP; ++s) {
-        chn[s] = ff_from(chin[s]);
-        dg[s] = ff_from(dg64[s]);
-    }
-    const ff cf = ff_from(coef), c = ff_from(pr.c), d = ff_from(pr.d), it0 = ff_from(pr.itau0);
-    F32Consts k;
-    k.cf = cf.h;
-    k.c = c.h;
-    k.d = d.h;
-    k.it0 = it0.h;
-    k.p = (int)pr.p;
-    const float rtol = (float)pr.rtol;
-    float prev = 3.0e38f;
-    for (int it = 0; it < 6; ++it) {
-        elastic_tau_ff(f, a, dg, g, tau);
-        float chi[NSLIP], dh[NSLIP], r[NSLIP], iden[NSLIP], dgh[NSLIP], x[NSLIP];
-        float rmax = 0.f;
-#pragma unroll 1
-        for (int s = 0; s < NSLIP; ++s) {
-            const ff ds = dg[s];
-            const ff ad = ds.h < 0.f ? ff_neg(ds) : ds;
-            const ff id = ff_recip(ff_norm(ff_mac(ff{1.f, 0.f}, d, ad)));
-            const ff ch = ff_mul(ff_norm(ff_mac(chn[s], c, ds)), id);
-            const ff xs = ff_mul(ff_add(tau[s], ff_neg(ch)), it0);
-            const ff ax = xs.h < 0.f ? ff_neg(xs) : xs;
-            ff pw{1.f, 0.f}, b = ax;
-            for (int e = k.p - 1; e; e >>= 1) {
-                if (e & 1) pw = ff_mul(pw, b);
-                b = ff_mul(b, b);
-            }
-            const ff rate = ff_mul(cf, ff_mul(pw, ax));
-            const ff rs = ff_add(ds, xs.h < 0.f ? rate : ff_neg(rate));
-            chi[s] = ch.h;
-            dh[s] = (float)k.p * pw.h;
-            r[s] = rs.h;
-            iden[s] = id.h;
-            dgh[s] = ds.h;
-            rmax = fmaxf(rmax, fabsf(rs.h));
-        }
-        if (!(rmax < 1e30f) || (it > 0 && rmax > 0.5f * prev)) return;  // the last iterate kept is the better one
-        for (int s = 0; s < NSLIP; ++s) dg64[s] = (double)dg[s].h + (double)dg[s].l;
-        if (rmax <= 0.5f * rtol) return;
-        if (!cp_correction_f32(g + G32_PC, dgh, k, chi, dh, iden, r, x)) return;
-        for (int s = 0; s < NSLIP; ++s) dg[s] = ff_add(dg[s], ff{-x[s], 0.f});
-        prev = rmax;
-    }
-}
-
 // Local Newton on dg from the given start.  lowrank: corrections from the
 // small-elastic-strain Jacobian in precision TJ; otherwise the exact
 // Jacobian with pivoting in FP64.
@@ -1237,10 +1038,8 @@ __device__ void cp_update(const double* F, const double* A, const double* chin, 
         double dgs[NSLIP];
         for (int a = 0; a < NSLIP; ++a) dgs[a] = dg[a];
         int it32 = 0;
-        if (cp_presolve_f32(F, A, chin, g32, pr, coef, dgs, &it32)) {
-            cp_refine_ff(F, A, chin, g32, pr, coef, dgs);
+        if (cp_presolve_f32(F, A, chin, g32, pr, coef, dgs, &it32))
             for (int a = 0; a < NSLIP; ++a) dg[a] = dgs[a];
-        }
         out.iters32 = it32;
     }
     // FP64 corrections: J is ill-conditioned (cond ~ 1e8 and more) once slip
