@@ -36,13 +36,14 @@ gff_status fail(gff_handle* h, gff_status st, const char* fmt, ...) {
 
 // ------------------------------------------------------------------ axis plans and tables
 struct TableLayout {
-    size_t tw64, tw32, posx, fqy, fqz, qt64, qt32, total;
+    size_t tw64, twd, tw32, posx, fqy, fqz, qt64, qt32, total;
 };
 
 TableLayout table_layout() {
     TableLayout t;
     size_t o = 0;
     t.tw64 = o; o += 3 * MAXN * sizeof(int4);
+    t.twd = o; o += 3 * MAXN * sizeof(double2);
     t.tw32 = o; o += 3 * MAXN * sizeof(float2);
     t.posx = o; o += MAXN * sizeof(int);
     t.fqy = o; o += MAXN * sizeof(int);
@@ -62,6 +63,7 @@ gff_status build_tables(gff_handle* h) {
     const TableLayout L = table_layout();
     std::vector<unsigned char> host(L.total, 0);
     int4* tw64 = reinterpret_cast<int4*>(host.data() + L.tw64);
+    double2* twd = reinterpret_cast<double2*>(host.data() + L.twd);
     float2* tw32 = reinterpret_cast<float2*>(host.data() + L.tw32);
     int* posx = reinterpret_cast<int*>(host.data() + L.posx);
     int* fqy = reinterpret_cast<int*>(host.data() + L.fqy);
@@ -77,6 +79,7 @@ gff_status build_tables(gff_handle* h) {
             const long double thl = 6.283185307179586476925286766559006L * k / n, one = 4611686018427387904.0L;  // 2^62
             const int2 re = twiddle_limbs(llroundl(std::cos(thl) * one)), im = twiddle_limbs(llroundl(-std::sin(thl) * one));
             tw64[a * MAXN + k] = make_int4(re.x, re.y, im.x, im.y);
+            twd[a * MAXN + k] = make_double2(std::cos(th), -std::sin(th));
             tw32[a * MAXN + k] = make_float2((float)std::cos(th), (float)-std::sin(th));
             // wave-vector tables: q = 2 pi kappa / n, kappa = k (k < n/2) or k - n
             const int kappa = (2 * k < n) ? k : k - n;
@@ -100,6 +103,7 @@ gff_status build_tables(gff_handle* h) {
     unsigned char* d = static_cast<unsigned char*>(h->tables);
     for (int a = 0; a < 3; ++a) {
         h->g.tw64[a] = reinterpret_cast<const int4*>(d + L.tw64) + a * MAXN;
+        h->g.twd[a] = reinterpret_cast<const double2*>(d + L.twd) + a * MAXN;
         h->g.tw32[a] = reinterpret_cast<const float2*>(d + L.tw32) + a * MAXN;
         for (int kind = 0; kind < 2; ++kind) {
             h->g.qt64[kind][a] = reinterpret_cast<const double*>(d + L.qt64) + (kind * 3 + a) * MAXN;
@@ -905,6 +909,8 @@ gff_status newton_increment(gff_handle* h, double dt, const double* Fbar, const 
     const ProjArgs pa = proj_args(h, mask);
     const OutArgs ores = out_args(h, -1.0, add9);
     const bool mixed = h->opt.precision == GFF_PREC_MIXED;
+    ProjArgs pres = pa;  // the residual's projection
+    pres.butterflies = mixed && !pa.sym ? 1 : 0;
     int newton = 0, cgsum = 0;
     double res = 0.0, nb = 0.0, nP = 0.0, rr_b = 0.0;
     bool conv = false;
@@ -947,7 +953,7 @@ gff_status newton_increment(gff_handle* h, double dt, const double* Fbar, const 
         GFF_TRY(cudaEventRecord(ev[0], h->stream));
         GFF_TRY(launch_constitutive(h, h->d_Fk, dt, mixed ? TANGENT_F32 : TANGENT_F64, warm_dg, CONST_P));
         GFF_TRY(cudaEventRecord(ev[1], h->stream));
-        GFF_TRY(launch_galerkin<double>(h, h->d_P, (const double*)nullptr, h->d_b, pa, ores, h->d_spec));
+        GFF_TRY(launch_galerkin<double>(h, h->d_P, (const double*)nullptr, h->d_b, pres, ores, h->d_spec));
         GFF_TRY(launch_dot<double>(h->d_b, h->d_b, n, h->d_red, h->d_scal, h->stream));
         GFF_TRY(launch_dot<double>(h->d_P, h->d_P, n, h->d_red + RED_BLOCKS, h->d_scal + 1, h->stream));
         GFF_TRY(cudaMemcpyAsync(h->d_scal + 2, h->d_flag, sizeof(int), cudaMemcpyDeviceToDevice, h->stream));

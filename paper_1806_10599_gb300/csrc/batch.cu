@@ -434,7 +434,9 @@ gff_status setup(Batch& B) {
         int* szc = szr + (m + 1);
         std::vector<int> s_pl, s_zr, s_zc;
         const gff_handle* rep = B.h[sc.rves[0]];  // the class's own tuned shapes
-        sc.res = class_launch<double>(rc, B.d_res + cbase, spl, szr, rep->tune[0], false, s_pl, s_zr);
+        Tune tres = rep->tune[0];
+        if (B.mixed) tres.wz = ZB_WIDTH, tres.t_z = 256;  // the FP64-butterfly residual's width
+        sc.res = class_launch<double>(rc, B.d_res + cbase, spl, szr, tres, false, s_pl, s_zr);
         if (B.mixed)
             sc.cg = class_launch<float>(gc, B.d_cga + cbase, spl, szc, rep->tune[1], true, s_pl, s_zc);
         else
@@ -477,6 +479,7 @@ gff_status set_residual_epilogue(Batch& B, const double* add9) {
         for (int r : sc.rves) {
             OutArgs& o = oa[pos++];
             o.scale = -1.0 / (double)B.h[r]->N;
+            o.pre = B.mixed ? 0 : 1;
             for (int c = 0; c < 9; ++c) o.add[c] = add9[c];
         }
     for (int i = 0; i < B.n; ++i)
@@ -493,7 +496,9 @@ cudaError_t apply_classes(Batch& B, int which, const ProjArgs& pa, cudaStream_t 
     cudaError_t e = cudaEventRecord(B.fork[which], s);
     for (SizeClass& sc : B.cls) {
         if (e == cudaSuccess) e = cudaStreamWaitEvent(sc.s[which], B.fork[which], 0);
-        if (e == cudaSuccess) e = launch_galerkin_batch<T>(which ? sc.cg : sc.res, pa, sc.s[which]);
+        ProjArgs p = pa;
+        p.butterflies = which == 0 && B.mixed ? 1 : 0;  // as gff_step's residual
+        if (e == cudaSuccess) e = launch_galerkin_batch<T>(which ? sc.cg : sc.res, p, sc.s[which]);
         if (e == cudaSuccess) e = cudaEventRecord(sc.done[which], sc.s[which]);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, sc.done[which], 0);
     }

@@ -32,6 +32,7 @@
 #include <cstdint>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "bulk_copy.cuh"
 #include "fixed_bfly.cuh"
@@ -39,6 +40,10 @@
 
 namespace gff {
 namespace {
+
+// twiddles as a pass reads them: limbs where FP64 data runs on integers (FX), else complex numbers
+template <typename T, bool FX> using TwP = typename std::conditional<FX, typename TwT<T>::t, typename C2<T>::t>::type;
+template <typename T> constexpr bool on_int = sizeof(T) == 8;  // the usual path of T
 
 template <typename C>
 __device__ __forceinline__ C mk(decltype(C::x) a, decltype(C::x) b) {
@@ -56,14 +61,6 @@ template <typename C> __device__ __forceinline__ C cmul(C a, C w) {
 }
 template <typename C> __device__ __forceinline__ C cmulc(C a, C w) {
     return mk<C>(a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y);
-}
-// in FP64 with the fused operand fixed: the passes that must agree bit for bit do not depend on the
-// compiler's choice of which product to fuse
-__device__ __forceinline__ double2 cmul(double2 a, double2 w) {
-    return make_double2(__fma_rn(a.x, w.x, -__dmul_rn(a.y, w.y)), __fma_rn(a.x, w.y, __dmul_rn(a.y, w.x)));
-}
-__device__ __forceinline__ double2 cmulc(double2 a, double2 w) {
-    return make_double2(__fma_rn(a.x, w.x, __dmul_rn(a.y, w.y)), __fma_rn(a.y, w.x, -__dmul_rn(a.x, w.y)));
 }
 // multiply by -i (forward) or +i (inverse)
 template <bool INV, typename C> __device__ __forceinline__ C rot90(C a) {
@@ -215,7 +212,7 @@ template <typename C> __device__ __forceinline__ C no_tw(int) { return C{}; }
 // Threads take (lf fastest, then butterfly, then ls) so that neighbouring
 // lanes touch neighbouring shared-memory words.
 template <typename T, int R, bool INV>
-__device__ __forceinline__ void run_stage(typename C2<T>::t* s, const typename TwT<T>::t* tw, int n, int len,
+__device__ __forceinline__ void run_stage(typename C2<T>::t* s, const typename C2<T>::t* tw, int n, int len,
                                           int NLF, int SF, int NLS, int SS, int ES, int tid, int nthr) {
     using C = typename C2<T>::t;
     const int m = len / R, nb = n / R, twstep = n / len;
@@ -239,7 +236,7 @@ __device__ __forceinline__ void run_stage(typename C2<T>::t* s, const typename T
 }
 
 template <typename T, bool INV>
-__device__ __forceinline__ void stage_dispatch(int R, typename C2<T>::t* s, const typename TwT<T>::t* tw, int n,
+__device__ __forceinline__ void stage_dispatch(int R, typename C2<T>::t* s, const typename C2<T>::t* tw, int n,
                                                int len, int NLF, int SF, int NLS, int SS, int ES, int tid,
                                                int nthr) {
     switch (R) {
@@ -273,7 +270,7 @@ __device__ __forceinline__ int divmod_f(int x, int d, float invd, int& r) {
 // over contiguous runs without twiddles -- the generic stages below with
 // compile-time radices and one (float) division per butterfly.
 template <typename T, int R1, int R2, bool TWIDDLED, bool INV>
-__device__ __forceinline__ void fft2_stage(typename C2<T>::t* s, const typename TwT<T>::t* tw, int NLF, float invNLF,
+__device__ __forceinline__ void fft2_stage(typename C2<T>::t* s, const typename C2<T>::t* tw, int NLF, float invNLF,
                                            int SF, int NLS, int SS, int ES, int tid, int nthr) {
     using C = typename C2<T>::t;
     // TWIDDLED: radix R1, tasks j < R2, elements j + q R2; else radix R2, tasks sub < R1, elements sub R2 + q
@@ -296,7 +293,7 @@ __device__ __forceinline__ void fft2_stage(typename C2<T>::t* s, const typename 
 }
 
 template <typename T, int R1, int R2, bool INV>
-__device__ __forceinline__ void fft2_lines(typename C2<T>::t* s, const typename TwT<T>::t* tw, int NLF, int SF,
+__device__ __forceinline__ void fft2_lines(typename C2<T>::t* s, const typename C2<T>::t* tw, int NLF, int SF,
                                            int NLS, int SS, int ES, int tid, int nthr) {
     const float invNLF = 1.0f / (float)NLF;
     if (!INV) {
@@ -515,10 +512,9 @@ __device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const Axis
 
 // Whole transform of a batch of lines; ends with a barrier.  Not inlined:
 // every kernel calls the same four instances (precision x direction).
-template <bool INV>
-__device__ __noinline__ void fft_lines_f32(float2* s, const float2* tw, const AxisPlan& pl, int NLF, int SF, int NLS, int SS, int ES,
+template <typename T, bool INV>
+__device__ __noinline__ void fft_lines_fp(typename C2<T>::t* s, const typename C2<T>::t* tw, const AxisPlan& pl, int NLF, int SF, int NLS, int SS, int ES,
                                            int tid, int nthr) {
-    using T = float;
     const int n = pl.n;
     if (pl.nst == 2) {
         const int r1 = pl.radix[0], r2 = pl.radix[1];
@@ -554,18 +550,28 @@ __device__ __noinline__ void fft_lines_f32(float2* s, const float2* tw, const Ax
     }
 }
 
-template <typename T, bool INV>
-__device__ __forceinline__ void fft_lines(typename C2<T>::t* s, const typename TwT<T>::t* tw, const AxisPlan& pl, int NLF, int SF,
+// FX: FP64 data on integers (everything but the residuals of mixed precision, ProjArgs::butterflies)
+template <typename T, bool INV, bool FX>
+__device__ __forceinline__ void fft_lines(typename C2<T>::t* s, const TwP<T, FX>* tw, const AxisPlan& pl, int NLF, int SF,
                                           int NLS, int SS, int ES, int tid, int nthr, int io = 0) {
-    if constexpr (sizeof(T) == 8)
+    if constexpr (FX)
         fft_lines_fx<INV>(s, tw, pl, NLF, SF, NLS, SS, ES, tid, nthr, fx_line_keys(), io);
     else
-        fft_lines_f32<INV>(s, tw, pl, NLF, SF, NLS, SS, ES, tid, nthr);
+        fft_lines_fp<T, INV>(s, tw, pl, NLF, SF, NLS, SS, ES, tid, nthr);
 }
 
-template <typename T> __device__ __forceinline__ const typename TwT<T>::t* twp(const GridDev& g, int a);
-template <> __device__ __forceinline__ const int4* twp<double>(const GridDev& g, int a) { return g.tw64[a]; }
-template <> __device__ __forceinline__ const float2* twp<float>(const GridDev& g, int a) { return g.tw32[a]; }
+template <typename T, bool FX> __device__ __forceinline__ const TwP<T, FX>* twp(const GridDev& g, int a) {
+    if constexpr (sizeof(T) == 4)
+        return g.tw32[a];
+    else if constexpr (FX)
+        return g.tw64[a];
+    else
+        return g.twd[a];
+}
+// the twiddle area of a pass's shared memory (entries of one size either way)
+template <typename T, bool FX> __device__ __forceinline__ TwP<T, FX>* as_tw(typename TwT<T>::t* p) {
+    return reinterpret_cast<TwP<T, FX>*>(p);
+}
 template <typename T> __device__ __forceinline__ const T* qtp(const GridDev& g, int kind, int a);
 template <> __device__ __forceinline__ const double* qtp<double>(const GridDev& g, int kind, int a) {
     return g.qt64[kind][a];
@@ -696,7 +702,7 @@ __device__ __forceinline__ void split_fx(double2& A, double2& B, const double2& 
     B = make_double2(fx::from_fixed(ky + my, e62), fx::from_fixed(mx - kx, e62));
 }
 
-template <typename T, bool WITH_K, bool VEC>
+template <typename T, bool WITH_K, bool VEC, bool FX = on_int<T>>
 __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T* __restrict__ K,
                                                typename C2<T>::t* __restrict__ spec, const GridDev& g, const int c,
                                                const int z, unsigned char* sm_raw) {
@@ -710,11 +716,11 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
     const int tid = threadIdx.x, nthr = blockDim.x;
 
     for (int i = tid; i < nx; i += nthr) {
-        twx[i] = twp<T>(g, 0)[i];
+        as_tw<T, FX>(twx)[i] = twp<T, FX>(g, 0)[i];
         posx[i] = g.posx[i];
     }
     for (int i = tid; i < ny; i += nthr) {
-        twy[i] = twp<T>(g, 1)[i];
+        as_tw<T, FX>(twy)[i] = twp<T, FX>(g, 1)[i];
         posy[g.fqy[i]] = i;
     }
 
@@ -723,8 +729,8 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
     // x transform of the ny/2 packed rows (row pair r at offset 2 r ls); rows are the
     // fast thread index, so that neighbouring lanes read neighbouring rows rather than
     // butterflies 8 or 16 elements apart in one row (fewer shared-memory bank conflicts)
-    fft_lines<T, false>(s, twx, g.ax, half, 2 * ls, 1, 0, 1, tid, nthr, FX_OUT);
-    const int de62 = sizeof(T) == 8 ? fx_out_exp(g.ax) : 0;
+    fft_lines<T, false, FX>(s, as_tw<T, FX>(twx), g.ax, half, 2 * ls, 1, 0, 1, tid, nthr, FX_OUT);
+    const int de62 = FX ? fx_out_exp(g.ax) : 0;
     // split each packed row into the half spectra of its two real rows.  Columns
     // kx = 0 and nx/2 of a real row are real, so one complex y transform of
     // Z = X_0 + i X_h carries both and nx/2 columns are transformed, not nx/2 + 1:
@@ -744,7 +750,7 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
             if (rok && k <= kh) {
                 const C zk = row[posx[k]];
                 const C zm = row[posx[k == 0 ? 0 : nx - k]];
-                if constexpr (sizeof(T) == 8) {  // the row's integers; FP64 where it did not run on integers
+                if constexpr (FX) {  // the row's integers; FP64 where it did not run on integers
                     const int me = fx_line_keys()[r] >> 20;
                     if (me >= fx::ME_MIN && me <= fx::ME_MAX) {
                         split_fx(A[t], B[t], zk, zm, me + de62);
@@ -782,7 +788,7 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
         }
     }
     __syncthreads();
-    fft_lines<T, false>(s, twy, g.ay, kh, 1, 1, 0, ls, tid, nthr);
+    fft_lines<T, false, FX>(s, as_tw<T, FX>(twy), g.ay, kh, 1, 1, 0, ls, tid, nthr);
     {
         // X_0(k) = (Z(k) + conj Z(-k)) / 2, X_h(k) = (Z(k) - conj Z(-k)) / 2i (one position per thread)
         C zp, zq;
@@ -807,13 +813,13 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
     for (int e = tid; e < nq; e += nthr) dst4[e] = src4[e];
 }
 
-template <typename T, bool WITH_K, bool VEC>
+template <typename T, bool WITH_K, bool VEC, bool FX = on_int<T>>
 __global__ void __launch_bounds__(512) k_plane_fwd(const T* __restrict__ x, const T* __restrict__ K,
                                                    typename C2<T>::t* __restrict__ spec, GridDev g,
                                                    const int* __restrict__ skip) {
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    plane_fwd_body<T, WITH_K, VEC>(x, K, spec, g, blockIdx.x, blockIdx.y, sm_raw);
+    plane_fwd_body<T, WITH_K, VEC, FX>(x, K, spec, g, blockIdx.x, blockIdx.y, sm_raw);
 }
 
 // ---------------------------------------------------------------- pass 2: z transform + projection
@@ -849,11 +855,11 @@ template <typename T> __host__ __device__ constexpr size_t ztables_bytes(int nz,
     return (size_t)nz * sizeof(typename C2<T>::t) + (size_t)(nxh + ny + nz) * sizeof(T) + (size_t)(nz + W) * sizeof(int);
 }
 
-template <typename T>
+template <typename T, bool FX = on_int<T>>
 __device__ __forceinline__ void zproj_tables(const GridDev& g, const ProjArgs& pa, const ZTables<T>& tb) {
     const int tid = threadIdx.x, nthr = blockDim.x;
     for (int i = tid; i < g.nz; i += nthr) {
-        tb.twz[i] = twp<T>(g, 2)[i];
+        as_tw<T, FX>(tb.twz)[i] = twp<T, FX>(g, 2)[i];
         tb.qz[i] = qtp<T>(g, pa.kind, 2)[i];
         tb.fqz[i] = g.fqz[i];
     }
@@ -984,7 +990,7 @@ __global__ void __launch_bounds__(256) k_fill_rq2(GridDev g, double* tab) {
 // s = [3][nz][W] (tensor row `row`): the row packed into u (slot 0) and
 // v (slot 2), both transformed, projected, transformed back and unpacked into
 // the three slots; ends with a barrier.
-template <typename T, int W>
+template <typename T, int W, bool FX = on_int<T>>
 __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev& g, const ProjArgs& pa, int row, int f0,
                                             const ZTables<T>& tb) {
     using C = typename C2<T>::t;
@@ -992,8 +998,8 @@ __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev&
     const int tid = threadIdx.x, nthr = blockDim.x;
     for (int e = tid; e < nz * W; e += nthr) s[e] = zpack<T>(s[e], s[nz * W + e], zcol<T>(tb.colk[e % W], tb));
     __syncthreads();
-    fft_lines<T, false>(s, tb.twz, g.az, W, 1, 2, 2 * nz * W, W, tid, nthr);
-    const T sc = sizeof(T) == 8 ? (T)1 / (T)g.N : (T)1;
+    fft_lines<T, false, FX>(s, as_tw<T, FX>(tb.twz), g.az, W, 1, 2, 2 * nz * W, W, tid, nthr);
+    const T sc = FX ? (T)1 / (T)g.N : (T)1;
     const T m0 = (T)pa.mask[3 * row] * sc, m1 = (T)pa.mask[3 * row + 1] * sc, m2 = (T)pa.mask[3 * row + 2] * sc;
     for (int e = tid; e < nz * W; e += nthr) {
         const int w = e % W, pz = e / W;
@@ -1002,7 +1008,7 @@ __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev&
         const int kx = ck & 0xffff, ky = ck >> 16, kz = tb.fqz[pz];
         C* p0 = s + pz * W + w;
         C u = p0[0], v = p0[2 * nz * W];
-        if constexpr (sizeof(T) == 8)
+        if constexpr (FX)
             zrow_proj64(u, v, kx, ky, kz, nx, ny, nz, m0, m1, m2, sc, g.rq2[pa.kind], (long long)pz * ny * g.nxh + f0 + w, tb);
         else
             zrow_proj<T>(u, v, kx, ky, kz, nx, ny, nz, m0, m1, m2, tb);
@@ -1010,7 +1016,7 @@ __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev&
         p0[2 * nz * W] = v;
     }
     __syncthreads();
-    fft_lines<T, true>(s, tb.twz, g.az, W, 1, 2, 2 * nz * W, W, tid, nthr);
+    fft_lines<T, true, FX>(s, as_tw<T, FX>(tb.twz), g.az, W, 1, 2, 2 * nz * W, W, tid, nthr);
     for (int e = tid; e < nz * W; e += nthr) zunpack<T>(s[e], zcol<T>(tb.colk[e % W], tb), s[e], s[nz * W + e]);
     __syncthreads();
 }
@@ -1097,7 +1103,7 @@ __device__ __forceinline__ void zstrip2(typename C2<T>::t* s, const GridDev& g, 
     __syncthreads();
 }
 
-template <typename T, int W>
+template <typename T, int W, bool FX = on_int<T>>
 __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec, const GridDev& g,
                                            const ProjArgs& pa, const int blk, unsigned char* sm_raw) {
     using C = typename C2<T>::t;
@@ -1110,7 +1116,7 @@ __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec,
     const int row = blk % 3;
     const int f0 = (blk / 3) * W;
     C* base = spec + 3 * row * nz * nF;  // component 3 row, z = 0
-    zproj_tables<T>(g, pa, tb);
+    zproj_tables<T, FX>(g, pa, tb);
     zproj_columns<T, W>(g, f0, tb);
     for (int e = tid; e < 3 * nz * W; e += nthr) {
         const int w = e % W, cz = e / W;  // cz = (component within the row) * nz + z
@@ -1118,7 +1124,7 @@ __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec,
         s[e] = f < nF ? base[cz * nF + f] : mk<C>((T)0, (T)0);
     }
     __syncthreads();
-    zproj_strip<T, W>(s, g, pa, row, f0, tb);
+    zproj_strip<T, W, FX>(s, g, pa, row, f0, tb);
     for (int e = tid; e < 3 * nz * W; e += nthr) {
         const int w = e % W, cz = e / W;
         const int f = f0 + w;
@@ -1126,15 +1132,13 @@ __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec,
     }
 }
 
-// FP64 transforms take what registers they get: 128 (16 warps per SM) rather than 190 (8 to 10)
-template <typename T> constexpr int z_min_blocks() { return sizeof(T) == 8 ? 2 : 1; }
-
-template <typename T, int W>
-__global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
+// FP64 transforms on integers take what registers they get: 128 (16 warps per SM) rather than 190 (8 to 10)
+template <typename T, int W, bool FX = on_int<T>>
+__global__ void __launch_bounds__(256, FX ? 2 : 1) k_zproj(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
                                               const int* __restrict__ skip) {
     if (skip && *skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    zproj_body<T, W>(spec, g, pa, blockIdx.x, sm_raw);
+    zproj_body<T, W, FX>(spec, g, pa, blockIdx.x, sm_raw);
 }
 
 // ---------------------------------------------------------------- small-strain variant: symmetric projection
@@ -1150,7 +1154,7 @@ template <typename T> size_t zsym_smem(const GridDev& g) {
 }
 
 template <typename T, int W>
-__global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj_sym(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
+__global__ void __launch_bounds__(256, on_int<T> ? 2 : 1) k_zproj_sym(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
                                                   const int* __restrict__ skip) {
     using C = typename C2<T>::t;
     if (skip && *skip) return;
@@ -1169,7 +1173,7 @@ __global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj_sym(typename C
         s[e] = f < nF ? spec[(long long)cz * nF + f] : mk<C>((T)0, (T)0);
     }
     __syncthreads();
-    fft_lines<T, false>(s, tb.twz, g.az, W, 1, 9, nz * W, W, tid, nthr);
+    fft_lines<T, false, on_int<T>>(s, tb.twz, g.az, W, 1, 9, nz * W, W, tid, nthr);
     for (int e = tid; e < nz * W; e += nthr) {
         const int w = e % W, pz = e / W;
         const int ck = tb.colk[w];
@@ -1213,7 +1217,7 @@ __global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj_sym(typename C
         for (int c = 0; c < 9; ++c) p0[c * nz * W] = v[c];
     }
     __syncthreads();
-    fft_lines<T, true>(s, tb.twz, g.az, W, 1, 9, nz * W, W, tid, nthr);
+    fft_lines<T, true, on_int<T>>(s, tb.twz, g.az, W, 1, 9, nz * W, W, tid, nthr);
     for (int e = tid; e < 9 * nz * W; e += nthr) {
         const int w = e % W, cz = e / W;
         const int f = f0 + w;
@@ -1381,10 +1385,10 @@ __device__ __noinline__ void merge_row_fp64(double2* row, int ls, const int* pos
 
 // Inverse y transform, merge of the packed rows, complex-to-real x transform
 // and epilogue of one plane already in shared memory s (tables loaded).
-template <typename T, bool VEC>
+template <typename T, bool VEC, bool FX = on_int<T>>
 __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __restrict__ y, const GridDev& g,
                                                   const OutArgs& oa, const int c, const int z,
-                                                  const typename TwT<T>::t* twx, const typename TwT<T>::t* twy,
+                                                  typename TwT<T>::t* twx, typename TwT<T>::t* twy,
                                                   const int* posx) {
     using C = typename C2<T>::t;
     const int nx = g.nx, ny = g.ny, nxh = g.nxh, ls = nxh, half = ny / 2;
@@ -1398,7 +1402,7 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
         s[yy * ls] = mk<C>(a.x - b.y, a.y + b.x);
     }
     __syncthreads();
-    fft_lines<T, true>(s, twy, g.ay, kh0, 1, 1, 0, ls, tid, nthr);
+    fft_lines<T, true, FX>(s, as_tw<T, FX>(twy), g.ay, kh0, 1, 1, 0, ls, tid, nthr);
     // merge the half spectra of rows 2r, 2r+1 into one packed complex row
     // Z_k = A_k + i B_k over all k (Hermitian symmetry of real rows), in the
     // digit-reversed order the inverse x pass expects; the real column nx/2
@@ -1422,7 +1426,7 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
             }
         }
         __syncwarp();
-        if constexpr (sizeof(T) == 8) {
+        if constexpr (FX) {
             // FP64: one row per warp; aligned to the largest value of both half spectra, one bit below the first
             // stage's alignment (|A| + |B|), and merged as integers
             int mkey = 0;
@@ -1468,10 +1472,10 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
         }
     }
     __syncthreads();
-    fft_lines<T, true>(s, twx, g.ax, half, 2 * ls, 1, 0, 1, tid, nthr, FX_IN);  // rows fastest, as in pass 1
+    fft_lines<T, true, FX>(s, as_tw<T, FX>(twx), g.ax, half, 2 * ls, 1, 0, 1, tid, nthr, FX_IN);  // rows fastest, as in pass 1
     T sc = (T)oa.scale;
     const T ad = (T)oa.add[c];
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (FX) {
         if (oa.pre) {  // the z pass has applied |scale|
             sc = sc < 0 ? -1.0 : 1.0;
             if (ad == 0) {
@@ -1492,17 +1496,17 @@ __device__ __noinline__ void plane_fill_nan(T* y, const GridDev& g, int c, int z
     for (int e = threadIdx.x; e < g.ny * g.nx; e += blockDim.x) yc[e] = nanv;
 }
 
-template <typename T>
+template <typename T, bool FX = on_int<T>>
 __device__ __forceinline__ void plane_tables(const GridDev& g, typename TwT<T>::t* twx, typename TwT<T>::t* twy,
                                              int* posx) {
     for (int i = threadIdx.x; i < g.nx; i += blockDim.x) {
-        twx[i] = twp<T>(g, 0)[i];
+        as_tw<T, FX>(twx)[i] = twp<T, FX>(g, 0)[i];
         posx[i] = g.posx[i];
     }
-    for (int i = threadIdx.x; i < g.ny; i += blockDim.x) twy[i] = twp<T>(g, 1)[i];
+    for (int i = threadIdx.x; i < g.ny; i += blockDim.x) as_tw<T, FX>(twy)[i] = twp<T, FX>(g, 1)[i];
 }
 
-template <typename T, bool VEC>
+template <typename T, bool VEC, bool FX = on_int<T>>
 __device__ __forceinline__ void plane_inv_body(const typename C2<T>::t* __restrict__ spec, T* __restrict__ y,
                                                const GridDev& g, const OutArgs& oa, const int c, const int z,
                                                unsigned char* sm_raw) {
@@ -1513,7 +1517,7 @@ __device__ __forceinline__ void plane_inv_body(const typename C2<T>::t* __restri
     auto* twy = twx + nx;
     int* posx = reinterpret_cast<int*>(twy + ny);
     const int tid = threadIdx.x, nthr = blockDim.x;
-    plane_tables<T>(g, twx, twy, posx);
+    plane_tables<T, FX>(g, twx, twy, posx);
     const C* in = spec + ((long long)c * g.nz + z) * (long long)ny * nxh;
     {
         const int nq = ny * nxh * (int)sizeof(C) / 16;
@@ -1522,14 +1526,14 @@ __device__ __forceinline__ void plane_inv_body(const typename C2<T>::t* __restri
         for (int e = tid; e < nq; e += nthr) dst4[e] = __ldg(src4 + e);
     }
     __syncthreads();
-    plane_inv_compute<T, VEC>(s, y, g, oa, c, z, twx, twy, posx);
+    plane_inv_compute<T, VEC, FX>(s, y, g, oa, c, z, twx, twy, posx);
 }
 
 // One block per plane (c, z) = (blockIdx.x, blockIdx.y).  The half-spectrum
 // plane is one contiguous run: a single bulk asynchronous copy brings it into
 // shared memory while the threads load the tables.  The wait is bounded
 // (timeout -> *err = 1 when err is set, and the block leaves).
-template <typename T, bool VEC>
+template <typename T, bool VEC, bool FX = on_int<T>>
 __global__ void __launch_bounds__(512) k_plane_inv(const typename C2<T>::t* __restrict__ spec, T* __restrict__ y,
                                                    GridDev g, OutArgs oa, const int* __restrict__ skip,
                                                    int* __restrict__ err) {
@@ -1551,7 +1555,7 @@ __global__ void __launch_bounds__(512) k_plane_inv(const typename C2<T>::t* __re
     __syncthreads();  // the barrier is initialised before any thread waits on it
     if (threadIdx.x == 0)  // plane * sizeof(C) is a multiple of 16 (ny even), the plane start too
         bulk_load(s, spec + ((long long)c * g.nz + z) * plane, (uint32_t)(plane * sizeof(C)), bar);
-    plane_tables<T>(g, twx, twy, posx);
+    plane_tables<T, FX>(g, twx, twy, posx);
     const bool ok = mbar_wait(bar, 0u, g.wait_cycles);
     if (__syncthreads_or(!ok)) {
         if (threadIdx.x == 0) {
@@ -1562,7 +1566,7 @@ __global__ void __launch_bounds__(512) k_plane_inv(const typename C2<T>::t* __re
         __syncthreads();
         return;
     }
-    plane_inv_compute<T, VEC>(s, y, g, oa, c, z, twx, twy, posx);
+    plane_inv_compute<T, VEC, FX>(s, y, g, oa, c, z, twx, twy, posx);
 }
 
 // Persistent variant: each block walks the planes p = blockIdx.x + k gridDim.x
@@ -1817,10 +1821,10 @@ __global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(con
     __syncthreads();
     if (tid == 0)  // n nxh sizeof(C) is a multiple of 16 (n even), the plane start too
         bulk_load(s, spec + ((long long)c * g.nz + z) * (n * nxh), (uint32_t)(n * nxh * sizeof(C)), bar);
-    for (int i = tid; i < n; i += nthr) twy[i] = twp<T>(g, 1)[i];
+    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, on_int<T>>(g, 1)[i];
     for (int i = tid; i < R2 * P::TWS; i += nthr) {
         const int j = i / P::TWS, p = i - j * P::TWS;
-        twx2[i] = p < R1 ? twp<T>(g, 0)[p * j] : typename TwT<T>::t{};
+        twx2[i] = p < R1 ? twp<T, on_int<T>>(g, 0)[p * j] : typename TwT<T>::t{};
     }
     const bool ok = mbar_wait(bar, 0u, g.wait_cycles);
     if (__syncthreads_or(!ok)) {
@@ -1853,10 +1857,10 @@ __global__ void __launch_bounds__(BT, 1) k_plane_inv2s(const typename C2<T>::t* 
     uint64_t* bar = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(twx2 + 8 * P::TWS) + 7) & ~uintptr_t(7));
     const uint32_t bytes = (uint32_t)(plane * sizeof(C));  // a multiple of 16 (n even)
     const int total = 9 * g.nz, tid = threadIdx.x, nthr = blockDim.x;
-    for (int i = tid; i < n; i += nthr) twy[i] = twp<T>(g, 1)[i];
+    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, on_int<T>>(g, 1)[i];
     for (int i = tid; i < 8 * P::TWS; i += nthr) {
         const int j = i / P::TWS, q = i - j * P::TWS;
-        twx2[i] = q < R1 ? twp<T>(g, 0)[q * j] : typename TwT<T>::t{};
+        twx2[i] = q < R1 ? twp<T, on_int<T>>(g, 0)[q * j] : typename TwT<T>::t{};
     }
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -2008,10 +2012,10 @@ __global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(con
     auto* twx2 = twy + n;                     // [8][R1 + 1]: W_n^(p j) of the x axis
     const int c = blockIdx.x, z = blockIdx.y;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    for (int i = tid; i < n; i += nthr) twy[i] = twp<T>(g, 1)[i];
+    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, on_int<T>>(g, 1)[i];
     for (int i = tid; i < R2 * P::TWS; i += nthr) {
         const int j = i / P::TWS, p = i - j * P::TWS;
-        twx2[i] = p < R1 ? twp<T>(g, 0)[p * j] : typename TwT<T>::t{};
+        twx2[i] = p < R1 ? twp<T, on_int<T>>(g, 0)[p * j] : typename TwT<T>::t{};
     }
     plane_contract<T, true, true>(s, x, K, g, c, z, nxh);
     __syncthreads();
@@ -2148,7 +2152,7 @@ namespace {
 
 template <typename T>
 cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, typename C2<T>::t* spec,
-                       const int* skip, cudaStream_t st, bool vin, int planes = 0) {
+                       const int* skip, cudaStream_t st, bool vin, int planes = 0, bool butterflies = false) {
     // planes > 0: that many z-planes from the ones x, K and spec point at (a chunk of the grid)
     const int nzl = planes > 0 ? planes : g.nz;
     // projection alone, unaligned, FP64 (its lines run in fixed point, in the generic pass only): the generic pass
@@ -2182,6 +2186,16 @@ cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, ty
             k_plane_fwd<T, true, false><<<gridA, threads, smA, st>>>(x, K, spec, g, skip);
         }
     } else {
+        if constexpr (sizeof(T) == 8)
+            if (butterflies) {
+                allow_smem(k_plane_fwd<T, false, true, false>, smA);
+                allow_smem(k_plane_fwd<T, false, false, false>, smA);
+                if (vin)
+                    k_plane_fwd<T, false, true, false><<<gridA, threads, smA, st>>>(x, nullptr, spec, g, skip);
+                else
+                    k_plane_fwd<T, false, false, false><<<gridA, threads, smA, st>>>(x, nullptr, spec, g, skip);
+                return cudaGetLastError();
+            }
         if (vin) {
             allow_smem(k_plane_fwd<T, false, true>, smA);
             k_plane_fwd<T, false, true><<<gridA, threads, smA, st>>>(x, nullptr, spec, g, skip);
@@ -2193,12 +2207,12 @@ cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, ty
     return cudaGetLastError();
 }
 
-template <typename T, int W>
+template <typename T, int W, bool FX = on_int<T>>
 cudaError_t launch_z_w(const GridDev& g, int threads, typename C2<T>::t* spec, const ProjArgs& pa, const int* skip,
                        cudaStream_t st) {
     const size_t smB = zproj_smem<T>(g, W);
-    allow_smem(k_zproj<T, W>, smB);
-    k_zproj<T, W><<<zproj_blocks(g, W), threads, smB, st>>>(spec, g, pa, skip);
+    allow_smem(k_zproj<T, W, FX>, smB);
+    k_zproj<T, W, FX><<<zproj_blocks(g, W), threads, smB, st>>>(spec, g, pa, skip);
     return cudaGetLastError();
 }
 
@@ -2666,7 +2680,7 @@ __device__ __forceinline__ int find_rve(const int* __restrict__ start, int n, in
     return r;
 }
 
-template <typename T, bool WITH_K, bool VEC>
+template <typename T, bool WITH_K, bool VEC, bool FX = on_int<T>>
 __global__ void __launch_bounds__(512) k_plane_fwd_batch(const RveApply* __restrict__ rv, const int* __restrict__ start,
                                                          int n) {
     const int r = find_rve(start, n, blockIdx.x);
@@ -2674,21 +2688,21 @@ __global__ void __launch_bounds__(512) k_plane_fwd_batch(const RveApply* __restr
     if (a.skip && *a.skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int local = blockIdx.x - start[r];
-    plane_fwd_body<T, WITH_K, VEC>(static_cast<const T*>(a.x), static_cast<const T*>(a.K),
+    plane_fwd_body<T, WITH_K, VEC, FX>(static_cast<const T*>(a.x), static_cast<const T*>(a.K),
                                    static_cast<typename C2<T>::t*>(a.spec), a.g, local % 9, local / 9, sm_raw);
 }
 
-template <typename T, int W>
-__global__ void __launch_bounds__(256, z_min_blocks<T>()) k_zproj_batch(const RveApply* __restrict__ rv, const int* __restrict__ start,
+template <typename T, int W, bool FX = on_int<T>>
+__global__ void __launch_bounds__(256, FX ? 2 : 1) k_zproj_batch(const RveApply* __restrict__ rv, const int* __restrict__ start,
                                                     int n, ProjArgs pa) {
     const int r = find_rve(start, n, blockIdx.x);
     const RveApply& a = rv[r];
     if (a.skip && *a.skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    zproj_body<T, W>(static_cast<typename C2<T>::t*>(a.spec), a.g, pa, blockIdx.x - start[r], sm_raw);
+    zproj_body<T, W, FX>(static_cast<typename C2<T>::t*>(a.spec), a.g, pa, blockIdx.x - start[r], sm_raw);
 }
 
-template <typename T, bool VEC>
+template <typename T, bool VEC, bool FX = on_int<T>>
 __global__ void __launch_bounds__(512) k_plane_inv_batch(const RveApply* __restrict__ rv, const int* __restrict__ start,
                                                          int n) {
     const int r = find_rve(start, n, blockIdx.x);
@@ -2696,14 +2710,14 @@ __global__ void __launch_bounds__(512) k_plane_inv_batch(const RveApply* __restr
     if (a.skip && *a.skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int local = blockIdx.x - start[r];
-    plane_inv_body<T, VEC>(static_cast<const typename C2<T>::t*>(a.spec), static_cast<T*>(a.y), a.g, a.oa,
+    plane_inv_body<T, VEC, FX>(static_cast<const typename C2<T>::t*>(a.spec), static_cast<T*>(a.y), a.g, a.oa,
                            local % 9, local / 9, sm_raw);
 }
 
-template <typename T, int W>
+template <typename T, int W, bool FX = on_int<T>>
 cudaError_t launch_zb(const BatchLaunch& bl, const ProjArgs& pa, cudaStream_t st) {
-    allow_smem(k_zproj_batch<T, W>, bl.smem_z);
-    k_zproj_batch<T, W><<<bl.blocks_z, bl.tn.t_z, bl.smem_z, st>>>(bl.rv, bl.start_z, bl.n, pa);
+    allow_smem(k_zproj_batch<T, W, FX>, bl.smem_z);
+    k_zproj_batch<T, W, FX><<<bl.blocks_z, bl.tn.t_z, bl.smem_z, st>>>(bl.rv, bl.start_z, bl.n, pa);
     return cudaGetLastError();
 }
 
@@ -2711,6 +2725,25 @@ cudaError_t launch_zb(const BatchLaunch& bl, const ProjArgs& pa, cudaStream_t st
 
 template <typename T>
 cudaError_t launch_galerkin_batch(const BatchLaunch& bl, const ProjArgs& pa, cudaStream_t st) {
+    if constexpr (sizeof(T) == 8)
+        if (pa.butterflies && !bl.withK) {
+            if (bl.tn.wz != ZB_WIDTH) return cudaErrorInvalidValue;
+            allow_smem(k_plane_fwd_batch<T, false, true, false>, bl.smem_plane);
+            allow_smem(k_plane_fwd_batch<T, false, false, false>, bl.smem_plane);
+            allow_smem(k_plane_inv_batch<T, true, false>, bl.smem_plane);
+            allow_smem(k_plane_inv_batch<T, false, false>, bl.smem_plane);
+            if (bl.vin)
+                k_plane_fwd_batch<T, false, true, false><<<bl.blocks_plane, bl.tn.t_fwd, bl.smem_plane, st>>>(bl.rv, bl.start_plane, bl.n);
+            else
+                k_plane_fwd_batch<T, false, false, false><<<bl.blocks_plane, bl.tn.t_fwd, bl.smem_plane, st>>>(bl.rv, bl.start_plane, bl.n);
+            cudaError_t e = launch_zb<T, ZB_WIDTH, false>(bl, pa, st);
+            if (e != cudaSuccess) return e;
+            if (bl.vout)
+                k_plane_inv_batch<T, true, false><<<bl.blocks_plane, bl.tn.t_inv, bl.smem_plane, st>>>(bl.rv, bl.start_plane, bl.n);
+            else
+                k_plane_inv_batch<T, false, false><<<bl.blocks_plane, bl.tn.t_inv, bl.smem_plane, st>>>(bl.rv, bl.start_plane, bl.n);
+            return cudaGetLastError();
+        }
     if (bl.withK) {
         if (bl.vin) {
             allow_smem(k_plane_fwd_batch<T, true, true>, bl.smem_plane);
@@ -2768,6 +2801,21 @@ cudaError_t launch_galerkin(const gff_handle* h, const T* x, const T* K, T* y, c
     const bool vout = vec_ok<T>(g, y);
     OutArgs oo = oa;
     oo.pre = pa.sym ? 0 : 1;
+    if constexpr (sizeof(T) == 8)
+        if (pa.butterflies && !K) {
+            oo.pre = 0;
+            cudaError_t e = launch_fwd<T>(g, 512, x, K, spec, skip, h->stream, vin, 0, true);
+            if (e == cudaSuccess) e = launch_z_w<T, ZB_WIDTH, false>(g, 256, spec, pa, skip, h->stream);
+            if (e != cudaSuccess) return e;
+            const size_t sm = plane_smem_bytes(g.nx, g.ny, sizeof(typename C2<T>::t));
+            allow_smem(k_plane_inv<T, true, false>, sm);
+            allow_smem(k_plane_inv<T, false, false>, sm);
+            if (vout)
+                k_plane_inv<T, true, false><<<dim3(9, g.nz), 512, sm, h->stream>>>(spec, y, g, oo, skip, h->d_flag + 2);
+            else
+                k_plane_inv<T, false, false><<<dim3(9, g.nz), 512, sm, h->stream>>>(spec, y, g, oo, skip, h->d_flag + 2);
+            return cudaGetLastError();
+        }
     if (ev) cudaEventRecord(ev[0], h->stream);
     cudaError_t e = launch_fwd<T>(g, tn.t_fwd, x, K, spec, skip, h->stream, vin);
     if (e != cudaSuccess) return e;
@@ -3053,6 +3101,7 @@ __attribute__((visibility("default"))) gff_status gff_project_noalloc(const gff_
         }
     }
     g.rq2[0] = g.rq2[1] = nullptr;
+    g.twd[0] = g.twd[1] = g.twd[2] = nullptr;
     g.posx = dt->posx;
     g.fqy = dt->fqy;
     g.fqz = dt->fqz;

@@ -46,6 +46,7 @@ struct GridDev {
     long long N;
     AxisPlan ax, ay, az;
     const int4* tw64[3];     // W_n^k = exp(-2 pi i k / n), k < n, per axis (x, y, z), in limbs (TwT)
+    const double2* twd[3];   // the same in FP64, for the FP64 butterflies (ProjArgs::butterflies)
     const float2* tw32[3];
     const int* posx;         // [nx]: position of natural frequency kx after the forward x pass
     const int* fqy;          // [ny]: frequency held at position py after the forward y pass
@@ -62,6 +63,11 @@ struct ProjArgs {
     int kind;        // GFF_PROJ_*
     float mask[9];   // 1 = stress-controlled component (zero frequency keeps it)
     int sym = 0;     // 1: small-strain variant, projection onto compatible symmetric fields
+    // FP64 data, no K: 1: transforms by FP64 butterflies instead of integers.  The residuals of mixed precision, which
+    // round to FP32 right after: a residual that differs in its last bits moves the converged fields by 1e-8 (rounding
+    // of the FP32 vectors, amplified by the soft plastic modes), and runs and state files of earlier builds would no
+    // longer be repeated bit for bit.  These projections are 4 % of a mixed increment.
+    int butterflies = 0;
 };
 
 // Output epilogue of the inverse plane pass: out = scale * y + add[c].
@@ -273,6 +279,8 @@ cudaError_t fill_rq2(const GridDev& g, double* tab, cudaStream_t st);
 // pos = sum_i p_i m_i with m_i = n / (r_0 ... r_i), frequency p_0 + r_0 p_1 + ...
 bool make_axis_plan(int n, AxisPlan& p);
 int axis_freq_of_pos(int pos, const AxisPlan& p);
+// columns per block of the FP64-butterfly z pass (ProjArgs::butterflies)
+constexpr int ZB_WIDTH = 8;
 // Blocks of the z pass: one per tensor row (3) and W (ky, kx) columns.
 inline int zproj_blocks(const GridDev& g, int W) { return 3 * (int)(((long long)g.ny * g.nxh + W - 1) / W); }
 // Times every candidate launch shape of the three kernels on the handle's own
