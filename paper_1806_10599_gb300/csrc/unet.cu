@@ -72,6 +72,9 @@ struct gff_unet {
     float* Y = nullptr;
     float* dY = nullptr;
     double* d_loss = nullptr;
+    // host arrays on their way in: grown by the calls that take them, given back with the network
+    void* stage = nullptr;
+    size_t stage_bytes = 0;
     // training samples (grid sample_n): inputs [V][IN_CH] bf16, targets [V][9] f32
     int sample_n = 0;
     std::vector<bf16*> sx;
@@ -169,6 +172,28 @@ gff_status ensure_buffers(gff_unet* u, int n) {
     u->dY = reinterpret_cast<float*>(b + odY);
     u->d_loss = reinterpret_cast<double*>(b + oL);
     u->n = n;
+    return GFF_OK;
+}
+
+gff_status ensure_stage(gff_unet* u, size_t bytes) {
+    if (u->stage_bytes >= bytes) return GFF_OK;
+    cudaFree(u->stage);
+    u->stage = nullptr;
+    u->stage_bytes = 0;
+    const cudaError_t e = cudaMalloc(&u->stage, bytes);
+    if (e != cudaSuccess) return ufail(u, GFF_ERR_OOM, "U-Net host arrays", e);
+    u->stage_bytes = bytes;
+    return GFF_OK;
+}
+
+// host inputs x [V][IN_CH] rounded to bfloat16 at dst (device)
+gff_status load_inputs(gff_unet* u, const float* x, long long V, bf16* dst) {
+    const long long n = V * IN_CH;
+    gff_status st = ensure_stage(u, (size_t)n * sizeof(float));
+    if (st != GFF_OK) return st;
+    UTRY(cudaMemcpy(u->stage, x, (size_t)n * sizeof(float), cudaMemcpyHostToDevice));
+    k_to_bf16<<<grid_of(n / 4), 256>>>(static_cast<const float*>(u->stage), dst, n);
+    UTRY(cudaGetLastError());
     return GFF_OK;
 }
 
@@ -288,8 +313,8 @@ gff_status back_layer(gff_unet* u, int l, View in, View out, View da, View* din,
 gff_status backward(gff_unet* u, View X, cudaStream_t st) {
     const Dims d0 = dims_of(u->n, 0), d1 = dims_of(u->n, 1), d2 = dims_of(u->n, 2), d3 = dims_of(u->n, 3);
     UTRY(cudaMemsetAsync(u->d_g, 0, u->nparam * sizeof(float), st));
-    k_head_bwd<<<grid_of(d0.V), 256, 0, st>>>(u->D1.p, u->D1.s, u->d_whr, u->dY, u->gD1.p, u->gD1.s,
-                                             u->d_g + u->off_hw, u->d_g + u->off_hb, HEAD_IN, HEAD_OUT, d0.V);
+    k_head_bwd<HEAD_IN, HEAD_OUT><<<(int)std::min(304LL, (d0.V + 255) / 256), 256, 0, st>>>(
+        u->D1.p, u->D1.s, u->d_whr, u->dY, u->gD1.p, u->gD1.s, u->d_g + u->off_hw, u->d_g + u->off_hb, d0.V);
     UTRY(cudaGetLastError());
     gff_status s;
 #define B_(expr) \
@@ -489,6 +514,7 @@ UEXPORT void gff_unet_destroy(gff_unet* u) {
     cudaFree(u->d_wd);
     cudaFree(u->d_whr);
     cudaFree(u->arena);
+    cudaFree(u->stage);
     for (auto p : u->sx) cudaFree(p);
     for (auto p : u->sy) cudaFree(p);
     delete u;
@@ -503,20 +529,16 @@ UEXPORT size_t gff_unet_num_params(const gff_unet* u) {
     return n + HEAD_OUT * HEAD_IN + HEAD_OUT;
 }
 
-// logical (unpadded) order: per layer W[27][cout][cin] then b[cout]; head W[9][16], b[9]
+// The parameters lie on the device in the order of gff_unet_get_params: no layer's input channels need padding.
+constexpr bool no_padding() {
+    for (const LayerDef& l : kL)
+        if (l.cin % 16) return false;
+    return true;
+}
+static_assert(no_padding(), "the logical and the device order of the parameters agree");
+
 static gff_status copy_params(gff_unet* u, float* host, const float* src_dev) {
-    std::vector<float> all(u->nparam);
-    cudaError_t e = cudaMemcpy(all.data(), src_dev, u->nparam * sizeof(float), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return ufail(u, GFF_ERR_CUDA, "U-Net params", e);
-    size_t k = 0;
-    for (int l = 0; l < NL; ++l) {
-        const int ci = kL[l].cin, cip = pad16(ci), co = kL[l].cout;
-        for (int t = 0; t < 27; ++t)
-            for (int o = 0; o < co; ++o)
-                for (int i = 0; i < ci; ++i) host[k++] = all[u->off_w[l] + ((size_t)t * co + o) * cip + i];
-        for (int o = 0; o < co; ++o) host[k++] = all[u->off_b[l] + o];
-    }
-    for (int j = 0; j < HEAD_OUT * HEAD_IN + HEAD_OUT; ++j) host[k++] = all[u->off_hw + j];
+    UTRY(cudaMemcpy(host, src_dev, u->nparam * sizeof(float), cudaMemcpyDeviceToHost));
     return GFF_OK;
 }
 
@@ -527,17 +549,7 @@ UEXPORT gff_status gff_unet_get_params(gff_unet* u, float* host) {
 
 UEXPORT gff_status gff_unet_set_params(gff_unet* u, const float* host) {
     if (!u || !host) return GFF_ERR_ARG;
-    std::vector<float> all(u->nparam, 0.f);
-    size_t k = 0;
-    for (int l = 0; l < NL; ++l) {
-        const int ci = kL[l].cin, cip = pad16(ci), co = kL[l].cout;
-        for (int t = 0; t < 27; ++t)
-            for (int o = 0; o < co; ++o)
-                for (int i = 0; i < ci; ++i) all[u->off_w[l] + ((size_t)t * co + o) * cip + i] = host[k++];
-        for (int o = 0; o < co; ++o) all[u->off_b[l] + o] = host[k++];
-    }
-    for (int j = 0; j < HEAD_OUT * HEAD_IN + HEAD_OUT; ++j) all[u->off_hw + j] = host[k++];
-    cudaError_t e = cudaMemcpy(u->d_w, all.data(), u->nparam * sizeof(float), cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMemcpy(u->d_w, host, u->nparam * sizeof(float), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return ufail(u, GFF_ERR_CUDA, "U-Net params", e);
     gff_status st = refresh_copies(u, nullptr);
     if (st != GFF_OK) return st;
@@ -554,27 +566,17 @@ UEXPORT gff_status gff_unet_eval_host(gff_unet* u, int n, const float* x, const 
     gff_status st = ensure_buffers(u, n);
     if (st != GFF_OK) return st;
     const long long V = (long long)n * n * n;
-    std::vector<bf16> xb((size_t)V * IN_CH);
-    for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16(x[i]);
-    UTRY(cudaMemcpy(u->X.p, xb.data(), xb.size() * sizeof(bf16), cudaMemcpyHostToDevice));
+    if ((st = load_inputs(u, x, V, u->X.p)) != GFF_OK) return st;
     if ((st = forward(u, u->X, nullptr)) != GFF_OK) return st;
     UTRY(cudaMemcpy(y, u->Y, (size_t)V * 9 * sizeof(float), cudaMemcpyDeviceToHost));
     if (!target) return GFF_OK;
-    float* dT = nullptr;
-    UTRY(cudaMalloc(&dT, (size_t)V * 9 * sizeof(float)));
-    cudaError_t e = cudaMemcpy(dT, target, (size_t)V * 9 * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(u->d_loss, 0, sizeof(double));
-    if (e == cudaSuccess) {
-        k_mse<<<grid_of(V * 9), 256>>>(u->Y, dT, u->dY, V * 9, u->d_loss);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess && (st = backward(u, u->X, nullptr)) != GFF_OK) {
-        cudaFree(dT);
-        return st;
-    }
-    if (e == cudaSuccess && loss) e = cudaMemcpy(loss, u->d_loss, sizeof(double), cudaMemcpyDeviceToHost);
-    cudaFree(dT);
-    if (e != cudaSuccess) return ufail(u, GFF_ERR_CUDA, "U-Net eval", e);
+    float* dT = static_cast<float*>(u->stage);  // the inputs have been rounded: their place is free
+    UTRY(cudaMemcpy(dT, target, (size_t)V * 9 * sizeof(float), cudaMemcpyHostToDevice));
+    UTRY(cudaMemset(u->d_loss, 0, sizeof(double)));
+    k_mse<<<grid_of(V * 9), 256>>>(u->Y, dT, u->dY, V * 9, u->d_loss);
+    UTRY(cudaGetLastError());
+    if ((st = backward(u, u->X, nullptr)) != GFF_OK) return st;
+    if (loss) UTRY(cudaMemcpy(loss, u->d_loss, sizeof(double), cudaMemcpyDeviceToHost));
     return grads ? copy_params(u, grads, u->d_g) : GFF_OK;
 }
 
@@ -640,18 +642,16 @@ UEXPORT gff_status gff_unet_add_sample_host(gff_unet* u, int n, const float* x, 
     if (!u || !x || !target || n < 8 || n % 8) return u ? ufail(u, GFF_ERR_ARG, "bad sample args") : GFF_ERR_ARG;
     if (u->sample_n && u->sample_n != n) return ufail(u, GFF_ERR_ARG, "all samples must share one grid");
     const long long V = (long long)n * n * n;
-    std::vector<bf16> xb((size_t)V * IN_CH);
-    for (size_t i = 0; i < xb.size(); ++i) xb[i] = __float2bfloat16(x[i]);
     bf16* dx = nullptr;
     float* dt = nullptr;
-    UTRY(cudaMalloc(&dx, xb.size() * sizeof(bf16)));
+    UTRY(cudaMalloc(&dx, (size_t)V * IN_CH * sizeof(bf16)));
     cudaError_t e = cudaMalloc(&dt, (size_t)V * 9 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemcpy(dx, xb.data(), xb.size() * sizeof(bf16), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(dt, target, (size_t)V * 9 * sizeof(float), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
+    gff_status ls = e == cudaSuccess ? load_inputs(u, x, V, dx) : ufail(u, GFF_ERR_CUDA, "U-Net sample", e);
+    if (ls != GFF_OK) {
         cudaFree(dx);
         cudaFree(dt);
-        return ufail(u, GFF_ERR_CUDA, "U-Net sample", e);
+        return ls;
     }
     double en = 0.0;
     for (long long i = 0; i < V * 9; ++i) en += (double)target[i] * target[i];

@@ -327,35 +327,70 @@ __global__ void k_head_fwd(const bf16* __restrict__ a, int sa, const float* __re
 }
 
 // head backward: da[v][i] = bf16(sum_o Wr[o][i] dy[v][o]); dW[o][i] += sum_v dy[v][o] a[v][i]; db[o] += sum_v dy[v][o]
+// A block walks tiles of 256 voxels: each thread loads and back-propagates one voxel (32 and 36 contiguous
+// bytes) and leaves a and dy in shared memory; then thread t < CO CI + CO keeps one weight's or bias's sum over the
+// tile in a register.  One atomic addition per sum and block: with one voxel per thread and shared-memory
+// atomics for all 153 sums of every voxel a 64^3 call took 816 us.
+template <int CI, int CO>
 __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ a, int sa, const float* __restrict__ Wr,
                                                   const float* __restrict__ dy, bf16* __restrict__ da, int sda,
-                                                  float* __restrict__ dW, float* __restrict__ db, int cin, int cout,
-                                                  long long V) {
-    __shared__ float pw[16 * 16 + 16];
-    for (int e = threadIdx.x; e < 16 * 16 + 16; e += blockDim.x) pw[e] = 0.f;
-    __syncthreads();
-    float lw[9 * 16], lb[9];
-    for (int k = 0; k < cout * cin; ++k) lw[k] = 0.f;
-    for (int o = 0; o < cout; ++o) lb[o] = 0.f;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
-        float xi[16], g[9];
-        for (int i = 0; i < cin; ++i) xi[i] = __bfloat162float(a[v * sa + i]);
-        for (int o = 0; o < cout; ++o) {
-            g[o] = dy[v * cout + o];
-            lb[o] += g[o];
-            for (int i = 0; i < cin; ++i) lw[o * cin + i] = fmaf(g[o], xi[i], lw[o * cin + i]);
+                                                  float* __restrict__ dW, float* __restrict__ db, long long V) {
+    static_assert(CI % 8 == 0 && CO * CI + CO <= 256, "one thread per sum");
+    __shared__ float sx[256][CI + 1], sg[256][CO];  // odd strides: a thread's row and a column of rows hit distinct banks
+    __shared__ float sw[CO * CI];
+    const int tid = threadIdx.x;
+    for (int e = tid; e < CO * CI; e += 256) sw[e] = Wr[e];
+    const int o = tid < CO * CI ? tid / CI : tid - CO * CI, i = tid < CO * CI ? tid % CI : CI;  // i = CI: the bias
+    float acc = 0.f;
+    for (long long v0 = (long long)blockIdx.x * 256; v0 < V; v0 += (long long)gridDim.x * 256) {
+        const int nv = (int)min(256LL, V - v0);
+        __syncthreads();  // the previous tile's readers are done (and sw is loaded)
+        if (tid < nv) {
+            const long long v = v0 + tid;
+            float g[CO];
+#pragma unroll
+            for (int k = 0; k < CO; ++k) sg[tid][k] = g[k] = dy[v * CO + k];
+#pragma unroll
+            for (int q = 0; q < CI / 8; ++q) {
+                const uint4 raw = *reinterpret_cast<const uint4*>(a + v * sa + 8 * q);
+                const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&raw);
+                uint4 outv;
+                __nv_bfloat162* d2 = reinterpret_cast<__nv_bfloat162*>(&outv);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int c = 8 * q + 2 * e;
+                    sx[tid][c] = __low2float(h[e]);
+                    sx[tid][c + 1] = __high2float(h[e]);
+                    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                    for (int k = 0; k < CO; ++k) {
+                        s0 = fmaf(sw[k * CI + c], g[k], s0);
+                        s1 = fmaf(sw[k * CI + c + 1], g[k], s1);
+                    }
+                    d2[e] = __floats2bfloat162_rn(s0, s1);
+                }
+                *reinterpret_cast<uint4*>(da + v * sda + 8 * q) = outv;
+            }
+            sx[tid][CI] = 1.f;
         }
-        for (int i = 0; i < cin; ++i) {
-            float s = 0.f;
-            for (int o = 0; o < cout; ++o) s = fmaf(Wr[o * cin + i], g[o], s);
-            da[v * sda + i] = __float2bfloat16(s);
-        }
+        __syncthreads();
+        if (tid < CO * CI + CO)
+            for (int r = 0; r < nv; ++r) acc = fmaf(sg[r][o], sx[r][i], acc);
     }
-    for (int k = 0; k < cout * cin; ++k) atomicAdd(pw + k, lw[k]);
-    for (int o = 0; o < cout; ++o) atomicAdd(pw + 256 + o, lb[o]);
-    __syncthreads();
-    for (int k = threadIdx.x; k < cout * cin; k += blockDim.x) atomicAdd(dW + k, pw[k]);
-    for (int o = threadIdx.x; o < cout; o += blockDim.x) atomicAdd(db + o, pw[256 + o]);
+    if (tid < CO * CI)
+        atomicAdd(dW + tid, acc);
+    else if (tid < CO * CI + CO)
+        atomicAdd(db + o, acc);
+}
+
+// y = bfloat16(x), n a multiple of 4 (host arrays arrive as FP32 and are rounded here: the same rounding on one host
+// thread took 4 ms for the inputs of a 64^3 grid)
+__global__ void __launch_bounds__(256) k_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, long long n) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n / 4; i += (long long)gridDim.x * blockDim.x) {
+        const float4 v = reinterpret_cast<const float4*>(x)[i];
+        __nv_bfloat162 p[2] = {__floats2bfloat162_rn(v.x, v.y), __floats2bfloat162_rn(v.z, v.w)};
+        reinterpret_cast<uint2*>(y)[i] = *reinterpret_cast<const uint2*>(p);
+    }
 }
 
 // mean squared error: dy = 2 (y - t) / n, loss += sum (y - t)^2 / n
