@@ -665,130 +665,134 @@ __device__ bool cp_local_solve(const double* F, const double* A, const double* c
     return false;
 }
 
-// Consistent tangent K = dP/dF at the converged return map, in precision T
-// (the grain's S0 and C given in T, so no conversions in the loops):
-//   K = dP/dF|_dg + (dP/ddg) (ddg/dF),  J ddg/dF = (coef/g) h' dtau/dF|_dg.
-template <typename T>
-__device__ __forceinline__ bool cp_tangent_core(const T* F, const T* A, const T* dg, const T* __restrict__ S0,
-                                                const T* __restrict__ C, const CPParamsDev& pr, double coef,
-                                                const ElStateT<T>& st, const T* chi, const T* dh, T* K) {
-    T J[NSLIP * NSLIP];
-    int piv[NSLIP];
-    const T cg = (T)(coef / pr.tau0);
-    T FeS[9];
-    mm(st.Fe, st.S, FeS);
-    // column b of the exact Jacobian dr_a/ddg_b (as cp_jacobian_exact) and dP/ddg_b (12 x 9) from
-    // one derivative of the elastic state per slip system
-    T dPb[NSLIP * 9];
-    {
-        const T cc = (T)pr.c, d = (T)pr.d;
-        for (int b = 0; b < NSLIP; ++b) {
-            T dFpi[9], dFe[9], dCe[9], dS[9], t1[9], t2[9], t3[9], t4[9];
-            dstate_ddg(F, A, S0 + 9 * b, C, st, dFpi, dFe, dCe, dS);
-            {
-                T dM[9];
-                mm(dCe, st.S, dM);
-                mm(st.Ce, dS, t1);
+// Voigt (11, 22, 33, 23, 13, 12) stiffness times a strain in engineering shears, as a symmetric 3x3
+__device__ __forceinline__ void c6_apply(const double* __restrict__ C6, const double* e, double* S) {
+    double sv[6];
 #pragma unroll
-                for (int k = 0; k < 9; ++k) dM[k] += t1[k];
-                for (int a = 0; a < NSLIP; ++a) {
-                    T dtau = (T)0;
+    for (int I = 0; I < 6; ++I) {
+        double t = 0.0;
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) dtau = fma(dM[k], __ldg(S0 + 9 * a + k), dtau);
-                    T v = -cg * dh[a] * dtau;
-                    if (a == b) {
-                        const T den = (T)1 + d * fabs(dg[a]);
-                        const T dchi = (cc - d * sgn(dg[a]) * chi[a]) / den;
-                        v += (T)1 + cg * dh[a] * dchi;
-                    }
-                    J[a * NSLIP + b] = v;
-                }
-            }
-            mm(dFe, st.S, t1);
-            mmt(t1, st.Fpi, t2);  // dFe S Fpi^T
-            mm(st.Fe, dS, t1);
-            mmt(t1, st.Fpi, t3);  // Fe dS Fpi^T
-            mmt(FeS, dFpi, t4);   // Fe S dFpi^T
-#pragma unroll
-            for (int k = 0; k < 9; ++k) dPb[9 * b + k] = t2[k] + t3[k] + t4[k];
-        }
+        for (int J = 0; J < 6; ++J) t = fma(__ldg(C6 + 6 * I + J), e[J], t);
+        sv[I] = t;
     }
-    if (!lu_factor<NSLIP>(J, piv)) return false;
-    T SFt[9];
-    mmt(st.S, st.Fpi, SFt);  // S Fpi^T
-    for (int kl = 0; kl < 9; ++kl) {
-        const int k = kl / 3, l = kl % 3;
-        // dFe = E_kl Fpi: row k equals row l of Fpi
-        T dFe[9];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) dFe[q] = (T)0;
-        dFe[3 * k] = st.Fpi[3 * l];
-        dFe[3 * k + 1] = st.Fpi[3 * l + 1];
-        dFe[3 * k + 2] = st.Fpi[3 * l + 2];
-        T t1[9], t2[9], dCe[9], hE[9], dS[9];
-        mtm(dFe, st.Fe, t1);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                dCe[3 * i + j] = t1[3 * i + j] + t1[3 * j + i];
-                hE[3 * i + j] = (T)0.5 * dCe[3 * i + j];
-            }
-        c_ddot(C, hE, dS);
-        // dP at fixed dg = dFe S Fpi^T + Fe dS Fpi^T
-        T dP[9], t3[9];
-        mm(dFe, SFt, dP);
-        mm(st.Fe, dS, t3);
-        mmt(t3, st.Fpi, t1);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) dP[q] += t1[q];
-        // dtau_a = (dCe S + Ce dS) : S0_a ; J ddg = (coef/g) h'_a dtau_a
-        T dM[9];
-        mm(dCe, st.S, dM);
-        mm(st.Ce, dS, t2);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) dM[q] += t2[q];
-        T rhs[NSLIP];
-        for (int a = 0; a < NSLIP; ++a) {
-            T dtau = (T)0;
-#pragma unroll
-            for (int q = 0; q < 9; ++q) dtau = fma(dM[q], __ldg(S0 + 9 * a + q), dtau);
-            rhs[a] = cg * dh[a] * dtau;
-        }
-        lu_solve<NSLIP>(J, piv, rhs);
-        for (int b = 0; b < NSLIP; ++b)
-#pragma unroll
-            for (int q = 0; q < 9; ++q) dP[q] = fma(dPb[9 * b + q], rhs[b], dP[q]);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) K[9 * q + kl] = dP[q];
-    }
-    return true;
+    S[0] = sv[0], S[4] = sv[1], S[8] = sv[2];
+    S[5] = S[7] = sv[3];
+    S[2] = S[6] = sv[4];
+    S[1] = S[3] = sv[5];
 }
 
-// The tangent from the FP64 state of the converged return map, computed in T.
-template <typename T>
-__device__ bool cp_tangent(const double* Fd, const double* Ad, const double* dgd, const T* __restrict__ S0,
-                           const T* __restrict__ C, const CPParamsDev& pr, double coef, const ElState& sd,
-                           const double* chid, const double* dhd, T* K) {
-    T F[9], A[9], dg[NSLIP], chi[NSLIP], dh[NSLIP];
-    ElStateT<T> st;
+// dM = dCe S + Ce dS, dS = C : dCe / 2, for dCe = a (x) b + b (x) a
+__device__ __forceinline__ void dmandel(const double* a, const double* b, const double* S, const double* Ce,
+                                        const double* __restrict__ C6, double* dM) {
+    double dCe[9], dS[9], t[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        F[k] = (T)Fd[k];
-        A[k] = (T)Ad[k];
-        st.Fpi[k] = (T)sd.Fpi[k];
-        st.Fe[k] = (T)sd.Fe[k];
-        st.Ce[k] = (T)sd.Ce[k];
-        st.S[k] = (T)sd.S[k];
-        st.M[k] = (T)sd.M[k];
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) dCe[3 * i + j] = a[i] * b[j] + b[i] * a[j];
+    const double e[6] = {0.5 * dCe[0], 0.5 * dCe[4], 0.5 * dCe[8], dCe[5], dCe[2], dCe[1]};
+    c6_apply(C6, e, dS);
+    mm(dCe, S, dM);
+    mm(Ce, dS, t);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) dM[k] += t[k];
+}
+
+// Consistent tangent K = dP/dF at the converged return map, written to K[(9 q + kl) ldk] (and rounded to K32 when given).
+// The slips enter only through L = sum_b ddg_b S0_b, so the 12 x 12 system J ddg = (coef/tau0) h' dtau/dF with
+// J = D - (coef/tau0) diag(h') dtau/ddg, D diagonal, is solved for L: with g_b = (coef/tau0) h'_b / D_b,
+// G = sum_b g_b S0_b (x) S0_b and dM (the change of the Mandel stress Ce S, tau_b = M : S0_b) linear in L and dF,
+//   (I - G dM/dL) L_kl = G dM/dF_kl,
+// a 9 x 9 system of order one where J's rows are scaled by h' over many decades, and
+//   dP_kl = dFe S Fp^-T + Fe dS Fp^-T + Fe S dFp^-T,  dFp^-1 = -A L_kl,  dFe = E_kl Fp^-1 - F A L_kl.
+// About 7 k FP64 operations where twelve slip derivatives, the 12 x 12 LU and nine solves take 11.5 k, and 1.3 kB of
+// local arrays per thread where those took 2.6 kB, which did not fit the SM's L1: gff_constitutive of 48^3 plastic
+// voxels 8.2 -> 6.8 ms, the return maps from zero slip being most of what is left.
+__device__ bool cp_tangent_f64(const double* F, const double* A, const double* dg, const double* __restrict__ geo,
+                               const CPParamsDev& pr, double coef, const ElState& st, const double* chi, const double* dh,
+                               double* __restrict__ K, float* __restrict__ K32, long long ldk) {
+    const double* S0 = geo + GEO_S0;
+    const double* C6 = geo + GEO_C6;
+    constexpr int NT = 9;
+    double B[NT * NT], R[NT * NT];  // I - G dM/dL, row-major; R[9 kl + .]: G dM/dF_kl, then L_kl
+    int piv[NT];
+    double H[9], Gm[9];
+    mm(F, A, H);
+    mtm(st.Fe, H, Gm);
+    {
+        const double cg = coef / pr.tau0;
+        double G[45];  // packed lower triangle
+#pragma unroll
+        for (int k = 0; k < 45; ++k) G[k] = 0.0;
+#pragma unroll 1
+        for (int b = 0; b < NSLIP; ++b) {
+            // D = 1 + f dchi, dchi = (c - d sgn(dg) chi) / den, den = 1 + d |dg|: g = f / D = f den / (den + f (c - d sgn chi))
+            const double f = cg * dh[b], den = fma(pr.d, fabs(dg[b]), 1.0);
+            const double g = f * den / fma(f, pr.c - pr.d * sgn(dg[b]) * chi[b], den);
+            double Sb[9];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) Sb[k] = __ldg(S0 + 9 * b + k);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const double gs = g * Sb[i];
+#pragma unroll
+                for (int j = 0; j <= i; ++j) G[i * (i + 1) / 2 + j] = fma(gs, Sb[j], G[i * (i + 1) / 2 + j]);
+            }
+        }
+        // columns 0..8: L = e_i (x) e_j (dFe = -H e_i (x) e_j); 9..17: dF = e_k (x) e_l
+#pragma unroll 1
+        for (int col = 0; col < 18; ++col) {
+            const int cc = col < 9 ? col : col - 9, i = cc / 3, j = cc - 3 * i;
+            double a[3], b[3], dM[9];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                a[k] = col < 9 ? (k == j ? 1.0 : 0.0) : st.Fpi[3 * j + k];
+                b[k] = col < 9 ? -Gm[3 * k + i] : st.Fe[3 * i + k];
+            }
+            dmandel(a, b, st.S, st.Ce, C6, dM);
+#pragma unroll
+            for (int r = 0; r < 9; ++r) {
+                double t = 0.0;
+#pragma unroll
+                for (int k = 0; k < 9; ++k) t = fma(G[r >= k ? r * (r + 1) / 2 + k : k * (k + 1) / 2 + r], dM[k], t);
+                if (col < 9)
+                    B[NT * r + cc] = (r == cc ? 1.0 : 0.0) - t;
+                else
+                    R[NT * cc + r] = t;
+            }
+        }
     }
-    for (int a = 0; a < NSLIP; ++a) {
-        dg[a] = (T)dgd[a];
-        chi[a] = (T)chid[a];
-        dh[a] = (T)dhd[a];
-        st.tau[a] = (T)sd.tau[a];
+    if (!lu_factor<NT>(B, piv)) return false;
+    double FeS[9], SFt[9];
+    mm(st.Fe, st.S, FeS);
+    mmt(st.S, st.Fpi, SFt);  // S Fpi^T
+#pragma unroll 1
+    for (int kl = 0; kl < 9; ++kl) {
+        const int k = kl / 3, l = kl - 3 * k;
+        lu_solve<NT>(B, piv, R + NT * kl);
+        double L[9], dFpi[9], dFe[9], t[9], dS[9], dP[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) L[q] = -R[NT * kl + q];
+        mm(A, L, dFpi);
+        mm(H, L, dFe);
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+            if (q / 3 == k) dFe[q] += st.Fpi[3 * l + q % 3];
+        mtm(dFe, st.Fe, t);  // dCe = t + t^T
+        const double e[6] = {t[0], t[4], t[8], t[5] + t[7], t[2] + t[6], t[1] + t[3]};
+        c6_apply(C6, e, dS);
+        mm(dFe, SFt, dP);
+        mm(st.Fe, dS, t);
+        double t2[9], t3[9];
+        mmt(t, st.Fpi, t2);
+        mmt(FeS, dFpi, t3);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const double v = dP[q] + t2[q] + t3[q];
+            K[(9 * q + kl) * ldk] = v;
+            if (K32) K32[(9 * q + kl) * ldk] = (float)v;
+        }
     }
-    return cp_tangent_core<T>(F, A, dg, S0, C, pr, coef, st, chi, dh, K);
+    return true;
 }
 
 // The elastic state at slips dg in FP32, in the displacement-gradient form of the
@@ -1021,13 +1025,11 @@ __device__ __noinline__ bool cp_tangent_f32(const double* Fd, const double* Ad, 
     return true;
 }
 
-// Return map (FP64) and, when K is not null, the tangent in precision T.
-template <typename T>
+// Return map (FP64).
 __device__ void cp_update(const double* F, const double* A, const double* chin, double dt,
                           const double* __restrict__ S0, const double* __restrict__ C, const double* __restrict__ H,
-                          const T* __restrict__ S0t, const T* __restrict__ Ct, const CPParamsDev& pr,
-                          const double* dg0 /* 12 or null */, T* K /* 81 or null */, CPOut& out,
-                          bool exact_only = false, const float* __restrict__ g32 = nullptr) {
+                          const CPParamsDev& pr, const double* dg0 /* 12 or null */, CPOut& out, bool exact_only = false,
+                          const float* __restrict__ g32 = nullptr) {
     const double coef = dt * pr.gdot0;
     const int p = (int)pr.p;
     double dg[NSLIP], dh[NSLIP], chi[NSLIP];
@@ -1064,7 +1066,6 @@ __device__ void cp_update(const double* F, const double* A, const double* chin, 
         out.dg[a] = dg[a];
         out.tau[a] = st.tau[a];
     }
-    if (K && conv) out.ok = cp_tangent<T>(F, A, dg, S0t, Ct, pr, coef, st, chi, dh, K);
 }
 
 __device__ void svk_update(const double* F, const double* __restrict__ C, double* P, double* K) {
@@ -1227,19 +1228,15 @@ struct ConstArgs {
 // F32T: the crystal-plasticity tangent is computed in FP32 and only K32 is
 // written (mixed precision); otherwise the tangent is FP64, written to K and,
 // when K32 is set, also rounded into K32.
-// The tangent alone, at the slips dg of the last return map (stored by a
-// PART_P launch): the elastic state and the residual terms are rebuilt at dg
-// -- the same function of the same values, so K equals what the return map's
-// own tangent would have been, bit for bit.
-template <typename T>
+// The FP64 tangent at the slips dg of the last return map: the elastic state and the residual terms are rebuilt at
+// dg, in the launch of the return map and in one of its own alike, so K is the same bit for bit.
 __device__ bool cp_tangent_at(const double* F, const double* A, const double* chin, const double* dg, double dt,
-                              const double* __restrict__ geo, const T* __restrict__ S0t, const T* __restrict__ Ct,
-                              const CPParamsDev& pr, T* K) {
+                              const double* __restrict__ geo, const CPParamsDev& pr, double* K, float* K32, long long ldk) {
     const double coef = dt * pr.gdot0;
     ElState st;
     double chi[NSLIP], dh[NSLIP], r[NSLIP], iden[NSLIP];
     cp_residual(F, A, chin, dg, geo, pr, coef, (int)pr.p, st, chi, dh, r, iden);
-    return cp_tangent<T>(F, A, dg, S0t, Ct, pr, coef, st, chi, dh, K);
+    return cp_tangent_f64(F, A, dg, geo, pr, coef, st, chi, dh, K, K32, ldk);
 }
 
 // PART_ALL: return map, P and the tangent; PART_P: return map and P (K left as
@@ -1280,14 +1277,7 @@ __device__ __forceinline__ void constitutive_voxel(const ConstArgs& a, const lon
             if (F32T) {
                 ok = cp_tangent_f32(F, A, chin, dg, a.dt, g32, pr, a.K32 + v, N);
             } else {
-                double K[81];
-                ok = cp_tangent_at<double>(F, A, chin, dg, a.dt, geo, geo + GEO_S0, C, pr, K);
-#pragma unroll
-                for (int k = 0; k < 81; ++k) a.K[k * N + v] = K[k];
-                if (a.K32) {
-#pragma unroll
-                    for (int k = 0; k < 81; ++k) a.K32[k * N + v] = (float)K[k];
-                }
+                ok = cp_tangent_at(F, A, chin, dg, a.dt, geo, pr, a.K + v, a.K32 ? a.K32 + v : nullptr, N);
             }
             if (!ok) atomicAdd(a.flag, 1);
             return;
@@ -1297,24 +1287,11 @@ __device__ __forceinline__ void constitutive_voxel(const ConstArgs& a, const lon
         if (warm)
             for (int s2 = 0; s2 < NSLIP; ++s2) dg0[s2] = a.dg[s2 * N + v];
         CPOut o;
-        if (PART == PART_P) {
-            cp_update<double>(F, A, chin, a.dt, geo, C, a.H + 144LL * gi, geo + GEO_S0, C, pr, warm ? dg0 : nullptr,
-                              (double*)nullptr, o, a.exact != 0, a.f32first ? g32 : nullptr);
-        } else if (F32T) {  // the return map, then the tangent as a tangent-only launch forms it
-            cp_update<float>(F, A, chin, a.dt, geo, C, a.H + 144LL * gi, g32 + G32_S0, g32 + G32_C, pr,
-                             warm ? dg0 : nullptr, (float*)nullptr, o, a.exact != 0, a.f32first ? g32 : nullptr);
-            if (o.ok) o.ok = cp_tangent_f32(F, A, chin, o.dg, a.dt, g32, pr, a.K32 + v, N);
-        } else {
-            double K[81];
-            cp_update<double>(F, A, chin, a.dt, geo, C, a.H + 144LL * gi, geo + GEO_S0, C, pr, warm ? dg0 : nullptr,
-                              K, o, a.exact != 0, a.f32first ? g32 : nullptr);
-#pragma unroll
-            for (int k = 0; k < 81; ++k) a.K[k * N + v] = K[k];
-            if (a.K32) {
-#pragma unroll
-                for (int k = 0; k < 81; ++k) a.K32[k * N + v] = (float)K[k];
-            }
-        }
+        cp_update(F, A, chin, a.dt, geo, C, a.H + 144LL * gi, pr, warm ? dg0 : nullptr, o, a.exact != 0,
+                  a.f32first ? g32 : nullptr);
+        if (PART == PART_ALL && o.ok)  // then the tangent as a tangent-only launch forms it
+            o.ok = F32T ? cp_tangent_f32(F, A, chin, o.dg, a.dt, g32, pr, a.K32 + v, N)
+                        : cp_tangent_at(F, A, chin, o.dg, a.dt, geo, pr, a.K + v, a.K32 ? a.K32 + v : nullptr, N);
         if (!o.ok) atomicAdd(a.flag, 1);
         n_fb = o.fallback ? 1 : 0;
         n_it = o.iters;
