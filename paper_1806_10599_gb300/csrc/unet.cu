@@ -199,16 +199,37 @@ gff_status load_inputs(gff_unet* u, const float* x, long long V, bf16* dst) {
 
 View slice(View v, int c0) { return View{v.p + c0, v.s}; }
 
+// A convolution's launch: the voxels a warp takes (16 MW) and the output channels (8 NT) from what fills the GPU.
+// Blocks of 64 MW voxels while at least 304 (two per SM) remain; a grid too small for that even at MW = 1 splits its
+// channels over blocks as well, down to 8 per warp (each split re-reads the input rows, from L2).
+template <int NT, int MW, bool RELU>
+void launch_conv(View in, int cin, const bf16* W, int cout, const float* b, View out, Dims d, cudaStream_t st) {
+    k_conv3<NT, MW, RELU><<<dim3((unsigned)((d.V + 64 * MW - 1) / (64 * MW)), cout / (8 * NT)), 128, 0, st>>>(
+        in.p, in.s, cin, W, cout, b, out.p, out.s, d);
+}
+template <int NT, bool RELU>
+void launch_conv_nt(View in, int cin, const bf16* W, int cout, const float* b, View out, Dims d, cudaStream_t st) {
+    if (NT <= 8 && d.V >= 304 * 256)
+        launch_conv<NT, (NT <= 8 ? 4 : 2), RELU>(in, cin, W, cout, b, out, d, st);
+    else if (d.V >= 304 * 128)
+        launch_conv<NT, 2, RELU>(in, cin, W, cout, b, out, d, st);
+    else if (NT <= 2 || d.V >= 304 * 64)
+        launch_conv<NT, 1, RELU>(in, cin, W, cout, b, out, d, st);
+    else if (d.V >= 76 * 64)
+        launch_conv<2, 1, RELU>(in, cin, W, cout, b, out, d, st);
+    else
+        launch_conv<1, 1, RELU>(in, cin, W, cout, b, out, d, st);
+}
+
 // forward conv of layer l: in (cinp channels) -> out (cout channels), leaky ReLU
 cudaError_t conv_fwd(gff_unet* u, int l, View in, View out, Dims d, cudaStream_t st) {
     const int cinp = pad16(kL[l].cin), cout = kL[l].cout;
     const bf16* W = u->d_wf + u->off_w[l];
     const float* b = u->d_w + u->off_b[l];
-    const int blocks = (int)((d.V + 63) / 64);
     switch (cout) {
-        case 16: k_conv3<2, true><<<blocks, 128, 0, st>>>(in.p, in.s, cinp, W, b, out.p, out.s, d); break;
-        case 32: k_conv3<4, true><<<blocks, 128, 0, st>>>(in.p, in.s, cinp, W, b, out.p, out.s, d); break;
-        case 64: k_conv3<8, true><<<blocks, 128, 0, st>>>(in.p, in.s, cinp, W, b, out.p, out.s, d); break;
+        case 16: launch_conv_nt<2, true>(in, cinp, W, cout, b, out, d, st); break;
+        case 32: launch_conv_nt<4, true>(in, cinp, W, cout, b, out, d, st); break;
+        case 64: launch_conv_nt<8, true>(in, cinp, W, cout, b, out, d, st); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -218,14 +239,13 @@ cudaError_t conv_fwd(gff_unet* u, int l, View in, View out, Dims d, cudaStream_t
 cudaError_t conv_dgrad(gff_unet* u, int l, View dz, View din, Dims d, cudaStream_t st) {
     const int cinp = pad16(kL[l].cin), cout = kL[l].cout;
     const bf16* W = u->d_wd + u->off_w[l];
-    const int blocks = (int)((d.V + 63) / 64);
     switch (cinp) {
-        case 16: k_conv3<2, false><<<blocks, 128, 0, st>>>(dz.p, dz.s, cout, W, nullptr, din.p, din.s, d); break;
-        case 32: k_conv3<4, false><<<blocks, 128, 0, st>>>(dz.p, dz.s, cout, W, nullptr, din.p, din.s, d); break;
-        case 48: k_conv3<6, false><<<blocks, 128, 0, st>>>(dz.p, dz.s, cout, W, nullptr, din.p, din.s, d); break;
-        case 64: k_conv3<8, false><<<blocks, 128, 0, st>>>(dz.p, dz.s, cout, W, nullptr, din.p, din.s, d); break;
-        case 96: k_conv3<12, false><<<blocks, 128, 0, st>>>(dz.p, dz.s, cout, W, nullptr, din.p, din.s, d); break;
-        case 128: k_conv3<16, false><<<blocks, 128, 0, st>>>(dz.p, dz.s, cout, W, nullptr, din.p, din.s, d); break;
+        case 16: launch_conv_nt<2, false>(dz, cout, W, cinp, nullptr, din, d, st); break;
+        case 32: launch_conv_nt<4, false>(dz, cout, W, cinp, nullptr, din, d, st); break;
+        case 48: launch_conv_nt<6, false>(dz, cout, W, cinp, nullptr, din, d, st); break;
+        case 64: launch_conv_nt<8, false>(dz, cout, W, cinp, nullptr, din, d, st); break;
+        case 96: launch_conv_nt<12, false>(dz, cout, W, cinp, nullptr, din, d, st); break;
+        case 128: launch_conv_nt<16, false>(dz, cout, W, cinp, nullptr, din, d, st); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -53,58 +53,80 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint
 }
 
 // out[v, co] = act(bias[co] + sum_{t, ci} W[t][co][ci] in[nb(v, t), ci])
-// in: cin channels (multiple of 16) at stride sin; W: [27][NT*8][cin] bf16;
-// out: NT*8 channels at stride sout.  RELU: leaky ReLU (slope LEAK for z <= 0).
-// Block = 4 warps = 64 voxels.
-template <int NT, bool RELU>
+// in: cin channels (multiple of 16) at stride sin; W: [27][cout][cin] bf16;
+// out: cout channels at stride sout.  RELU: leaky ReLU (slope LEAK for z <= 0).
+// A warp takes MW tiles of 16 voxels and NT tiles of 8 output channels (blockIdx.y: which of cout / (8 NT) groups), a
+// block four warps = 64 MW voxels.  Each output's sum runs over t and then ci whatever the split, so the bits do not
+// depend on it.  Bound: the loads of the weight fragments (two 4-byte loads per tile of 8 channels and k16 step), hence
+// MW tiles of voxels per fragment where the grid is large enough to fill the GPU all the same, and the channels split
+// over blocks where it is not (conv_shape in unet.cu).
+template <int NT, int MW, bool RELU>
 __global__ void __launch_bounds__(128) k_conv3(const bf16* __restrict__ in, int sin, int cin,
-                                               const bf16* __restrict__ W, const float* __restrict__ bias,
+                                               const bf16* __restrict__ W, int cout, const float* __restrict__ bias,
                                                bf16* __restrict__ out, int sout, Dims d) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, tq = lane & 3;
-    const long long v0 = ((long long)blockIdx.x * 4 + warp) * 16;
+    const int co0 = blockIdx.y * (NT * 8);
+    const long long v0 = ((long long)blockIdx.x * 4 + warp) * (16 * MW);
     if (v0 >= d.V) return;
-    const long long va = v0 + g, vb = v0 + g + 8;
-    const bool oka = va < d.V, okb = vb < d.V;
-    float acc[NT][4];
+    // this lane's rows g and g + 8 of every tile (clamped to the first voxel past the end)
+    int z[2 * MW], y[2 * MW], x[2 * MW];
 #pragma unroll
-    for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
-    const int cout = NT * 8;
+    for (int m = 0; m < 2 * MW; ++m) {
+        const long long v = v0 + 8 * m + g, vc = v < d.V ? v : v0;
+        const int plane = d.ny * d.nx;
+        z[m] = (int)(vc / plane);
+        const int rem = (int)(vc - (long long)z[m] * plane);
+        y[m] = rem / d.nx;
+        x[m] = rem - y[m] * d.nx;
+    }
+    float acc[MW][NT][4];
+#pragma unroll
+    for (int m = 0; m < MW; ++m)
+#pragma unroll
+        for (int j = 0; j < NT; ++j) acc[m][j][0] = acc[m][j][1] = acc[m][j][2] = acc[m][j][3] = 0.f;
     for (int t = 0; t < 27; ++t) {
-        const long long qa = neighbour(d, oka ? va : v0, t);
-        const long long qb = neighbour(d, okb ? vb : v0, t);
-        const bf16* ra = in + qa * sin + 2 * tq;
-        const bf16* rb = in + qb * sin + 2 * tq;
-        const bf16* wt = W + (long long)t * cout * cin + (long long)g * cin + 2 * tq;
+        const bf16* r[2 * MW];
+#pragma unroll
+        for (int m = 0; m < 2 * MW; ++m) r[m] = in + neighbour_of(d, z[m], y[m], x[m], t) * sin + 2 * tq;
+        const bf16* wt = W + ((long long)t * cout + co0 + g) * cin + 2 * tq;
         for (int kc = 0; kc < cin; kc += 16) {
-            uint32_t a[4];
-            a[0] = *reinterpret_cast<const uint32_t*>(ra + kc);
-            a[1] = *reinterpret_cast<const uint32_t*>(rb + kc);
-            a[2] = *reinterpret_cast<const uint32_t*>(ra + kc + 8);
-            a[3] = *reinterpret_cast<const uint32_t*>(rb + kc + 8);
+            uint32_t a[MW][4];
+#pragma unroll
+            for (int m = 0; m < MW; ++m) {
+                a[m][0] = *reinterpret_cast<const uint32_t*>(r[2 * m] + kc);
+                a[m][1] = *reinterpret_cast<const uint32_t*>(r[2 * m + 1] + kc);
+                a[m][2] = *reinterpret_cast<const uint32_t*>(r[2 * m] + kc + 8);
+                a[m][3] = *reinterpret_cast<const uint32_t*>(r[2 * m + 1] + kc + 8);
+            }
 #pragma unroll
             for (int j = 0; j < NT; ++j) {
                 uint32_t b[2];
                 const bf16* wj = wt + (long long)j * 8 * cin + kc;
                 b[0] = __ldg(reinterpret_cast<const unsigned int*>(wj));
                 b[1] = __ldg(reinterpret_cast<const unsigned int*>(wj + 8));
-                mma_bf16(acc[j], a, b);
+#pragma unroll
+                for (int m = 0; m < MW; ++m) mma_bf16(acc[m][j], a[m], b);
             }
         }
     }
 #pragma unroll
-    for (int j = 0; j < NT; ++j) {
-        const int co = j * 8 + 2 * tq;
-        const float b0 = bias ? bias[co] : 0.f, b1 = bias ? bias[co + 1] : 0.f;
-        float r0 = acc[j][0] + b0, r1 = acc[j][1] + b1, r2 = acc[j][2] + b0, r3 = acc[j][3] + b1;
-        if (RELU) {
-            r0 = r0 > 0.f ? r0 : LEAK * r0;
-            r1 = r1 > 0.f ? r1 : LEAK * r1;
-            r2 = r2 > 0.f ? r2 : LEAK * r2;
-            r3 = r3 > 0.f ? r3 : LEAK * r3;
+    for (int m = 0; m < MW; ++m) {
+        const long long va = v0 + 16 * m + g, vb = va + 8;
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            const int co = co0 + j * 8 + 2 * tq;
+            const float b0 = bias ? bias[co] : 0.f, b1 = bias ? bias[co + 1] : 0.f;
+            float r0 = acc[m][j][0] + b0, r1 = acc[m][j][1] + b1, r2 = acc[m][j][2] + b0, r3 = acc[m][j][3] + b1;
+            if (RELU) {
+                r0 = r0 > 0.f ? r0 : LEAK * r0;
+                r1 = r1 > 0.f ? r1 : LEAK * r1;
+                r2 = r2 > 0.f ? r2 : LEAK * r2;
+                r3 = r3 > 0.f ? r3 : LEAK * r3;
+            }
+            if (va < d.V) *reinterpret_cast<__nv_bfloat162*>(out + va * sout + co) = __floats2bfloat162_rn(r0, r1);
+            if (vb < d.V) *reinterpret_cast<__nv_bfloat162*>(out + vb * sout + co) = __floats2bfloat162_rn(r2, r3);
         }
-        if (oka) *reinterpret_cast<__nv_bfloat162*>(out + va * sout + co) = __floats2bfloat162_rn(r0, r1);
-        if (okb) *reinterpret_cast<__nv_bfloat162*>(out + vb * sout + co) = __floats2bfloat162_rn(r2, r3);
     }
 }
 
