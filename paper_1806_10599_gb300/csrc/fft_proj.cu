@@ -642,8 +642,8 @@ __device__ __forceinline__ void plane_contract(typename C2<T>::t* s, const T* __
                     VT kv[9], xq[9];
 #pragma unroll
                     for (int d = 0; d < 9; ++d) {
-                        kv[d] = __ldg(reinterpret_cast<const VT*>(Kc + d * N + v0));
-                        xq[d] = __ldg(reinterpret_cast<const VT*>(x + d * N + v0));
+                        kv[d] = load_dev(reinterpret_cast<const VT*>(Kc + d * N + v0));
+                        xq[d] = load_dev(reinterpret_cast<const VT*>(x + d * N + v0));
                     }
 #pragma unroll
                     for (int j = 0; j < VW; ++j) {
@@ -653,7 +653,7 @@ __device__ __forceinline__ void plane_contract(typename C2<T>::t* s, const T* __
                         acc[j] = t;
                     }
                 } else {
-                    const VT xv4 = __ldg(reinterpret_cast<const VT*>(x + c * N + v0));
+                    const VT xv4 = load_dev(reinterpret_cast<const VT*>(x + c * N + v0));
 #pragma unroll
                     for (int j = 0; j < VW; ++j) acc[j] = V16<T>::get(xv4, j);
                 }
@@ -681,12 +681,12 @@ __device__ __forceinline__ void plane_contract(typename C2<T>::t* s, const T* __
                 const T* Kc = K + (long long)c * 9 * N;
 #pragma unroll
                 for (int d = 0; d < 9; ++d) {
-                    a = fma(__ldg(Kc + d * N + v0), __ldg(x + d * N + v0), a);
-                    b = fma(__ldg(Kc + d * N + v1), __ldg(x + d * N + v1), b);
+                    a = fma(load_dev(Kc + d * N + v0), load_dev(x + d * N + v0), a);
+                    b = fma(load_dev(Kc + d * N + v1), load_dev(x + d * N + v1), b);
                 }
             } else {
-                a = __ldg(x + c * N + v0);
-                b = __ldg(x + c * N + v1);
+                a = load_dev(x + c * N + v0);
+                b = load_dev(x + c * N + v1);
             }
             s[r * 2 * ls + xi] = mk<C>(a, b);
         }
@@ -705,7 +705,7 @@ __device__ __forceinline__ void split_fx(double2& A, double2& B, const double2& 
 template <typename T, bool WITH_K, bool VEC, bool FX = on_int<T>>
 __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T* __restrict__ K,
                                                typename C2<T>::t* __restrict__ spec, const GridDev& g, const int c,
-                                               const int z, unsigned char* sm_raw) {
+                                               const int z, unsigned char* sm_raw, const int* skip) {
     using C = typename C2<T>::t;
     const int nx = g.nx, ny = g.ny, nxh = g.nxh, ls = nxh, half = ny / 2;
     C* s = reinterpret_cast<C*>(sm_raw);
@@ -723,6 +723,8 @@ __device__ __forceinline__ void plane_fwd_body(const T* __restrict__ x, const T*
         as_tw<T, FX>(twy)[i] = twp<T, FX>(g, 1)[i];
         posy[g.fqy[i]] = i;
     }
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
 
     plane_contract<T, WITH_K, VEC>(s, x, K, g, c, z, ls);
     __syncthreads();
@@ -817,9 +819,9 @@ template <typename T, bool WITH_K, bool VEC, bool FX = on_int<T>>
 __global__ void __launch_bounds__(512) k_plane_fwd(const T* __restrict__ x, const T* __restrict__ K,
                                                    typename C2<T>::t* __restrict__ spec, GridDev g,
                                                    const int* __restrict__ skip) {
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    plane_fwd_body<T, WITH_K, VEC, FX>(x, K, spec, g, blockIdx.x, blockIdx.y, sm_raw);
+    plane_fwd_body<T, WITH_K, VEC, FX>(x, K, spec, g, blockIdx.x, blockIdx.y, sm_raw, skip);
 }
 
 // ---------------------------------------------------------------- pass 2: z transform + projection
@@ -1105,7 +1107,8 @@ __device__ __forceinline__ void zstrip2(typename C2<T>::t* s, const GridDev& g, 
 
 template <typename T, int W, bool FX = on_int<T>>
 __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec, const GridDev& g,
-                                           const ProjArgs& pa, const int blk, unsigned char* sm_raw) {
+                                           const ProjArgs& pa, const int blk, unsigned char* sm_raw,
+                                           const int* skip) {
     using C = typename C2<T>::t;
     const int nz = g.nz;
     C* s = reinterpret_cast<C*>(sm_raw);  // [3][nz][W]
@@ -1118,6 +1121,8 @@ __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec,
     C* base = spec + 3 * row * nz * nF;  // component 3 row, z = 0
     zproj_tables<T, FX>(g, pa, tb);
     zproj_columns<T, W>(g, f0, tb);
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
     for (int e = tid; e < 3 * nz * W; e += nthr) {
         const int w = e % W, cz = e / W;  // cz = (component within the row) * nz + z
         const int f = f0 + w;
@@ -1136,9 +1141,9 @@ __device__ __forceinline__ void zproj_body(typename C2<T>::t* __restrict__ spec,
 template <typename T, int W, bool FX = on_int<T>>
 __global__ void __launch_bounds__(256, FX ? 2 : 1) k_zproj(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
                                               const int* __restrict__ skip) {
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    zproj_body<T, W, FX>(spec, g, pa, blockIdx.x, sm_raw);
+    zproj_body<T, W, FX>(spec, g, pa, blockIdx.x, sm_raw, skip);
 }
 
 // ---------------------------------------------------------------- small-strain variant: symmetric projection
@@ -1157,7 +1162,7 @@ template <typename T, int W>
 __global__ void __launch_bounds__(256, on_int<T> ? 2 : 1) k_zproj_sym(typename C2<T>::t* __restrict__ spec, GridDev g, ProjArgs pa,
                                                   const int* __restrict__ skip) {
     using C = typename C2<T>::t;
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int nz = g.nz, nx = g.nx, ny = g.ny;
     C* s = reinterpret_cast<C*>(sm_raw);  // [9][nz][W]
@@ -1167,6 +1172,8 @@ __global__ void __launch_bounds__(256, on_int<T> ? 2 : 1) k_zproj_sym(typename C
     const int f0 = blockIdx.x * W;
     zproj_tables<T>(g, pa, tb);
     zproj_columns<T, W>(g, f0, tb);
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
     for (int e = tid; e < 9 * nz * W; e += nthr) {
         const int w = e % W, cz = e / W;  // cz = component * nz + z
         const int f = f0 + w;
@@ -1254,7 +1261,7 @@ __global__ void __launch_bounds__(BT, ztma_min_blocks<T, W, R1, BT>())
     k_zproj_tma(const __grid_constant__ CUtensorMap tm, GridDev g, ProjArgs pa, const int* __restrict__ skip,
                 int* __restrict__ err) {
     using C = typename C2<T>::t;
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     unsigned char* p = sm_raw + ((128u - (smem_addr(sm_raw) & 127u)) & 127u);  // 128-byte aligned boxes
     const size_t sb = zstrip_bytes<T, W>(g.nz);
@@ -1272,6 +1279,8 @@ __global__ void __launch_bounds__(BT, ztma_min_blocks<T, W, R1, BT>())
         mbar_init_fence();
     }
     __syncthreads();
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
     int s = blockIdx.x;
     if (threadIdx.x == 0 && s < total) tma_load_3d(buf[0], &tm, (s / 3) * W * K, 0, 3 * (s % 3), &bar[0], bytes);
     uint32_t phase[2] = {0u, 0u};
@@ -1538,7 +1547,7 @@ __global__ void __launch_bounds__(512) k_plane_inv(const typename C2<T>::t* __re
                                                    GridDev g, OutArgs oa, const int* __restrict__ skip,
                                                    int* __restrict__ err) {
     using C = typename C2<T>::t;
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int nx = g.nx, plane = g.ny * g.nxh;
     C* s = reinterpret_cast<C*>(sm_raw);
@@ -1552,10 +1561,12 @@ __global__ void __launch_bounds__(512) k_plane_inv(const typename C2<T>::t* __re
         mbar_init(bar, 1);
         mbar_init_fence();
     }
+    plane_tables<T, FX>(g, twx, twy, posx);
     __syncthreads();  // the barrier is initialised before any thread waits on it
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
     if (threadIdx.x == 0)  // plane * sizeof(C) is a multiple of 16 (ny even), the plane start too
         bulk_load(s, spec + ((long long)c * g.nz + z) * plane, (uint32_t)(plane * sizeof(C)), bar);
-    plane_tables<T, FX>(g, twx, twy, posx);
     const bool ok = mbar_wait(bar, 0u, g.wait_cycles);
     if (__syncthreads_or(!ok)) {
         if (threadIdx.x == 0) {
@@ -1586,7 +1597,7 @@ __global__ void __launch_bounds__(inv_stream_max_threads<T>()) k_plane_inv_strea
                                                           T* __restrict__ y, GridDev g, OutArgs oa,
                                                           const int* __restrict__ skip, int* __restrict__ err) {
     using C = typename C2<T>::t;
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int nx = g.nx, ny = g.ny, plane = ny * g.nxh;
     const uint32_t bytes = (uint32_t)(plane * sizeof(C));  // multiple of 16 (ny even)
@@ -1603,6 +1614,8 @@ __global__ void __launch_bounds__(inv_stream_max_threads<T>()) k_plane_inv_strea
         mbar_init_fence();
     }
     __syncthreads();
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
     int p = blockIdx.x;
     if (threadIdx.x == 0 && p < total) bulk_load(buf[0], spec + (long long)p * plane, bytes, &bar[0]);
     uint32_t phase[2] = {0u, 0u};
@@ -1805,7 +1818,7 @@ __global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(con
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, R2>;
     constexpr int n = P::n, nxh = P::nxh;
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* s = reinterpret_cast<C*>(sm_raw);  // [n][nxh]
     auto* twy = reinterpret_cast<typename TwT<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
@@ -1818,14 +1831,16 @@ __global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(con
         mbar_init(bar, 1);
         mbar_init_fence();
     }
-    __syncthreads();
-    if (tid == 0)  // n nxh sizeof(C) is a multiple of 16 (n even), the plane start too
-        bulk_load(s, spec + ((long long)c * g.nz + z) * (n * nxh), (uint32_t)(n * nxh * sizeof(C)), bar);
     for (int i = tid; i < n; i += nthr) twy[i] = twp<T, on_int<T>>(g, 1)[i];
     for (int i = tid; i < R2 * P::TWS; i += nthr) {
         const int j = i / P::TWS, p = i - j * P::TWS;
         twx2[i] = p < R1 ? twp<T, on_int<T>>(g, 0)[p * j] : typename TwT<T>::t{};
     }
+    __syncthreads();
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
+    if (tid == 0)  // n nxh sizeof(C) is a multiple of 16 (n even), the plane start too
+        bulk_load(s, spec + ((long long)c * g.nz + z) * (n * nxh), (uint32_t)(n * nxh * sizeof(C)), bar);
     const bool ok = mbar_wait(bar, 0u, g.wait_cycles);
     if (__syncthreads_or(!ok)) {
         if (tid == 0) {
@@ -1849,7 +1864,7 @@ __global__ void __launch_bounds__(BT, 1) k_plane_inv2s(const typename C2<T>::t* 
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, 8>;
     constexpr int n = P::n, nxh = P::nxh, plane = n * nxh;
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* buf[2] = {reinterpret_cast<C*>(sm_raw), reinterpret_cast<C*>(sm_raw) + plane};
     auto* twy = reinterpret_cast<typename TwT<T>::t*>(buf[1] + plane);
@@ -1868,6 +1883,8 @@ __global__ void __launch_bounds__(BT, 1) k_plane_inv2s(const typename C2<T>::t* 
         mbar_init_fence();
     }
     __syncthreads();
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
     int p = blockIdx.x;
     if (tid == 0 && p < total) bulk_load(buf[0], spec + (long long)p * plane, bytes, &bar[0]);
     uint32_t phase[2] = {0u, 0u};
@@ -2005,7 +2022,7 @@ __global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(con
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, 8>;
     constexpr int n = P::n, h = P::h, nxh = P::nxh, R2 = 8;
-    if (skip && *skip) return;
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* s = reinterpret_cast<C*>(sm_raw);  // [n][nxh]
     auto* twy = reinterpret_cast<typename TwT<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
@@ -2017,6 +2034,8 @@ __global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(con
         const int j = i / P::TWS, p = i - j * P::TWS;
         twx2[i] = p < R1 ? twp<T, on_int<T>>(g, 0)[p * j] : typename TwT<T>::t{};
     }
+    pdl_wait();
+    if (skip && load_flag(skip)) return;
     plane_contract<T, true, true>(s, x, K, g, c, z, nxh);
     __syncthreads();
     const int lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
@@ -2152,7 +2171,8 @@ namespace {
 
 template <typename T>
 cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, typename C2<T>::t* spec,
-                       const int* skip, cudaStream_t st, bool vin, int planes = 0, bool butterflies = false) {
+                       const int* skip, cudaStream_t st, bool vin, int planes = 0, bool butterflies = false,
+                       bool pdl = false) {
     // planes > 0: that many z-planes from the ones x, K and spec point at (a chunk of the grid)
     const int nzl = planes > 0 ? planes : g.nz;
     // projection alone, unaligned, FP64 (its lines run in fixed point, in the generic pass only): the generic pass
@@ -2165,8 +2185,7 @@ cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, ty
 #define GFF_FWD2(R, BT)                                                             \
     if (r1 == R && threads == -BT) {                                                \
         allow_smem(k_plane_fwd2<T, R, BT>, sm);                                     \
-        k_plane_fwd2<T, R, BT><<<grid, BT, sm, st>>>(x, K, spec, g, skip);          \
-        return cudaGetLastError();                                                  \
+        return launch_kernel(pdl, k_plane_fwd2<T, R, BT>, grid, BT, sm, st, x, K, spec, g, skip); \
     }
         GFF_FWD2(16, 256)
         GFF_FWD2(16, 512)
@@ -2180,10 +2199,10 @@ cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, ty
     if (K) {
         if (vin) {
             allow_smem(k_plane_fwd<T, true, true>, smA);
-            k_plane_fwd<T, true, true><<<gridA, threads, smA, st>>>(x, K, spec, g, skip);
+            return launch_kernel(pdl, k_plane_fwd<T, true, true>, gridA, threads, smA, st, x, K, spec, g, skip);
         } else {
             allow_smem(k_plane_fwd<T, true, false>, smA);
-            k_plane_fwd<T, true, false><<<gridA, threads, smA, st>>>(x, K, spec, g, skip);
+            return launch_kernel(pdl, k_plane_fwd<T, true, false>, gridA, threads, smA, st, x, K, spec, g, skip);
         }
     } else {
         if constexpr (sizeof(T) == 8)
@@ -2191,39 +2210,36 @@ cudaError_t launch_fwd(const GridDev& g, int threads, const T* x, const T* K, ty
                 allow_smem(k_plane_fwd<T, false, true, false>, smA);
                 allow_smem(k_plane_fwd<T, false, false, false>, smA);
                 if (vin)
-                    k_plane_fwd<T, false, true, false><<<gridA, threads, smA, st>>>(x, nullptr, spec, g, skip);
+                    return launch_kernel(pdl, k_plane_fwd<T, false, true, false>, gridA, threads, smA, st, x, nullptr, spec, g, skip);
                 else
-                    k_plane_fwd<T, false, false, false><<<gridA, threads, smA, st>>>(x, nullptr, spec, g, skip);
-                return cudaGetLastError();
+                    return launch_kernel(pdl, k_plane_fwd<T, false, false, false>, gridA, threads, smA, st, x, nullptr, spec, g, skip);
             }
         if (vin) {
             allow_smem(k_plane_fwd<T, false, true>, smA);
-            k_plane_fwd<T, false, true><<<gridA, threads, smA, st>>>(x, nullptr, spec, g, skip);
+            return launch_kernel(pdl, k_plane_fwd<T, false, true>, gridA, threads, smA, st, x, nullptr, spec, g, skip);
         } else {
             allow_smem(k_plane_fwd<T, false, false>, smA);
-            k_plane_fwd<T, false, false><<<gridA, threads, smA, st>>>(x, nullptr, spec, g, skip);
+            return launch_kernel(pdl, k_plane_fwd<T, false, false>, gridA, threads, smA, st, x, nullptr, spec, g, skip);
         }
     }
-    return cudaGetLastError();
 }
 
 template <typename T, int W, bool FX = on_int<T>>
 cudaError_t launch_z_w(const GridDev& g, int threads, typename C2<T>::t* spec, const ProjArgs& pa, const int* skip,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool pdl = false) {
     const size_t smB = zproj_smem<T>(g, W);
     allow_smem(k_zproj<T, W, FX>, smB);
-    k_zproj<T, W, FX><<<zproj_blocks(g, W), threads, smB, st>>>(spec, g, pa, skip);
-    return cudaGetLastError();
+    return launch_kernel(pdl, k_zproj<T, W, FX>, zproj_blocks(g, W), threads, smB, st, spec, g, pa, skip);
 }
 
 template <typename T>
 cudaError_t launch_z(const GridDev& g, int W, int threads, typename C2<T>::t* spec, const ProjArgs& pa,
-                     const int* skip, cudaStream_t st) {
+                     const int* skip, cudaStream_t st, bool pdl = false) {
     switch (W) {
-        case 4: return launch_z_w<T, 4>(g, threads, spec, pa, skip, st);
-        case 8: return launch_z_w<T, 8>(g, threads, spec, pa, skip, st);
-        case 16: return launch_z_w<T, 16>(g, threads, spec, pa, skip, st);
-        case 32: return launch_z_w<T, 32>(g, threads, spec, pa, skip, st);
+        case 4: return launch_z_w<T, 4>(g, threads, spec, pa, skip, st, pdl);
+        case 8: return launch_z_w<T, 8>(g, threads, spec, pa, skip, st, pdl);
+        case 16: return launch_z_w<T, 16>(g, threads, spec, pa, skip, st, pdl);
+        case 32: return launch_z_w<T, 32>(g, threads, spec, pa, skip, st, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -2232,12 +2248,11 @@ template <typename T> int tune_index() { return sizeof(T) == 8 ? 0 : 1; }
 
 template <typename T>
 cudaError_t launch_zsym(const GridDev& g, typename C2<T>::t* spec, const ProjArgs& pa, const int* skip,
-                        cudaStream_t st) {
+                        cudaStream_t st, bool pdl = false) {
     constexpr int W = zsym_width<T>();
     const size_t sm = zsym_smem<T>(g);
     allow_smem(k_zproj_sym<T, W>, sm);
-    k_zproj_sym<T, W><<<(g.ny * g.nxh + W - 1) / W, 256, sm, st>>>(spec, g, pa, skip);
-    return cudaGetLastError();
+    return launch_kernel(pdl, k_zproj_sym<T, W>, (g.ny * g.nxh + W - 1) / W, 256, sm, st, spec, g, pa, skip);
 }
 
 // ---- TMA z pass: tensor maps and launch
@@ -2301,38 +2316,37 @@ template <typename T> bool ztma_threads_ok(int R1, int threads) {
 
 template <typename T, int W, int R1, int BT>
 cudaError_t launch_z_tma_kb(gff_handle* h, int threads, int blocks, const ProjArgs& pa, const int* skip,
-                            cudaStream_t st) {
+                            cudaStream_t st, bool pdl) {
     const CUtensorMap* tm = zmap<T>(h, W);
     if (!tm) return cudaErrorNotSupported;
     const size_t sm = ztma_smem<T, W>(h->g);
     allow_smem(k_zproj_tma<T, W, R1, BT>, sm);
-    k_zproj_tma<T, W, R1, BT><<<blocks, threads, sm, st>>>(*tm, h->g, pa, skip, h->d_flag + 2);
-    return cudaGetLastError();
+    return launch_kernel(pdl, k_zproj_tma<T, W, R1, BT>, blocks, threads, sm, st, *tm, h->g, pa, skip, h->d_flag + 2);
 }
 template <typename T, int W, int R1>
 cudaError_t launch_z_tma_k(gff_handle* h, int threads, int blocks, const ProjArgs& pa, const int* skip,
-                           cudaStream_t st) {
+                           cudaStream_t st, bool pdl) {
     if (!ztma_threads_ok<T>(R1, threads)) return cudaErrorInvalidValue;
     if constexpr (R1 == 0) {
-        return launch_z_tma_kb<T, W, 0, 512>(h, threads, blocks, pa, skip, st);
+        return launch_z_tma_kb<T, W, 0, 512>(h, threads, blocks, pa, skip, st, pdl);
     } else {
         if constexpr (sizeof(T) == 4)
-            if (threads == 384) return launch_z_tma_kb<T, W, R1, 384>(h, threads, blocks, pa, skip, st);
-        return launch_z_tma_kb<T, W, R1, 256>(h, threads, blocks, pa, skip, st);
+            if (threads == 384) return launch_z_tma_kb<T, W, R1, 384>(h, threads, blocks, pa, skip, st, pdl);
+        return launch_z_tma_kb<T, W, R1, 256>(h, threads, blocks, pa, skip, st, pdl);
     }
 }
 
 // blocks > 0: the TMA z pass with the generic strip; < 0: with the register-staged strip, -blocks blocks
 template <typename T, int W>
 cudaError_t launch_z_tma_w(gff_handle* h, int threads, int blocks, const ProjArgs& pa, const int* skip,
-                           cudaStream_t st) {
-    if (blocks > 0) return launch_z_tma_k<T, W, 0>(h, threads, blocks, pa, skip, st);
+                           cudaStream_t st, bool pdl) {
+    if (blocks > 0) return launch_z_tma_k<T, W, 0>(h, threads, blocks, pa, skip, st, pdl);
     if constexpr (sizeof(T) == 8) {  // FP64: the generic strip, whose lines run in fixed point
-        return launch_z_tma_k<T, W, 0>(h, threads, -blocks, pa, skip, st);
+        return launch_z_tma_k<T, W, 0>(h, threads, -blocks, pa, skip, st, pdl);
     } else {
         switch (z2_radix(h->g)) {
-            case 16: return launch_z_tma_k<T, W, 16>(h, threads, -blocks, pa, skip, st);
-            case 8: return launch_z_tma_k<T, W, 8>(h, threads, -blocks, pa, skip, st);
+            case 16: return launch_z_tma_k<T, W, 16>(h, threads, -blocks, pa, skip, st, pdl);
+            case 8: return launch_z_tma_k<T, W, 8>(h, threads, -blocks, pa, skip, st, pdl);
             default: return cudaErrorInvalidValue;
         }
     }
@@ -2340,10 +2354,10 @@ cudaError_t launch_z_tma_w(gff_handle* h, int threads, int blocks, const ProjArg
 
 template <typename T>
 cudaError_t launch_z_tma(gff_handle* h, int W, int threads, int blocks, const ProjArgs& pa, const int* skip,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool pdl = false) {
     switch (W) {
-        case 8: return launch_z_tma_w<T, 8>(h, threads, blocks, pa, skip, st);
-        case 16: return launch_z_tma_w<T, 16>(h, threads, blocks, pa, skip, st);
+        case 8: return launch_z_tma_w<T, 8>(h, threads, blocks, pa, skip, st, pdl);
+        case 16: return launch_z_tma_w<T, 16>(h, threads, blocks, pa, skip, st, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -2397,7 +2411,8 @@ int z_tma_blocks(gff_handle* h, int W, int threads, bool reg = false) {
 
 template <typename T>
 cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename C2<T>::t* spec, T* y,
-                       const OutArgs& oa, const int* skip, cudaStream_t st, bool vout, int* err, int planes = 0) {
+                       const OutArgs& oa, const int* skip, cudaStream_t st, bool vout, int* err, int planes = 0,
+                       bool pdl = false) {
     // planes > 0 (one block per plane only): that many z-planes from the ones spec and y point at
     const int nzl = planes > 0 ? planes : g.nz;
     if (planes > 0 && blocks != 0 && blocks != -1) return cudaErrorInvalidValue;
@@ -2409,8 +2424,7 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
 #define GFF_INV2S(R, BT)                                                                   \
     if (r1 == R && threads == BT) {                                                        \
         allow_smem(k_plane_inv2s<T, R, BT>, sm);                                           \
-        k_plane_inv2s<T, R, BT><<<-blocks, BT, sm, st>>>(spec, y, g, oa, skip, err);       \
-        return cudaGetLastError();                                                         \
+        return launch_kernel(pdl, k_plane_inv2s<T, R, BT>, -blocks, BT, sm, st, spec, y, g, oa, skip, err); \
     }
         GFF_INV2S(16, 512)
         GFF_INV2S(8, 512)
@@ -2426,8 +2440,7 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
 #define GFF_INV2(R, BT)                                                              \
     if (r1 == R && threads == BT) {                                                  \
         allow_smem(k_plane_inv2<T, R, 8, BT>, sm);                                   \
-        k_plane_inv2<T, R, 8, BT><<<grid, BT, sm, st>>>(spec, y, g, oa, skip, err);  \
-        return cudaGetLastError();                                                   \
+        return launch_kernel(pdl, k_plane_inv2<T, R, 8, BT>, grid, BT, sm, st, spec, y, g, oa, skip, err); \
     }
         GFF_INV2(16, 256)
         GFF_INV2(16, 512)
@@ -2441,23 +2454,21 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
         const size_t sm = plane_stream_smem<T>(g);
         if (vout) {
             allow_smem(k_plane_inv_stream<T, true>, sm);
-            k_plane_inv_stream<T, true><<<blocks, threads, sm, st>>>(spec, y, g, oa, skip, err);
+            return launch_kernel(pdl, k_plane_inv_stream<T, true>, blocks, threads, sm, st, spec, y, g, oa, skip, err);
         } else {
             allow_smem(k_plane_inv_stream<T, false>, sm);
-            k_plane_inv_stream<T, false><<<blocks, threads, sm, st>>>(spec, y, g, oa, skip, err);
+            return launch_kernel(pdl, k_plane_inv_stream<T, false>, blocks, threads, sm, st, spec, y, g, oa, skip, err);
         }
-        return cudaGetLastError();
     }
     const size_t smA = plane_smem_bytes(g.nx, g.ny, sizeof(typename C2<T>::t));
     const dim3 gridA(9, nzl);
     if (vout) {
         allow_smem(k_plane_inv<T, true>, smA);
-        k_plane_inv<T, true><<<gridA, threads, smA, st>>>(spec, y, g, oa, skip, err);
+        return launch_kernel(pdl, k_plane_inv<T, true>, gridA, threads, smA, st, spec, y, g, oa, skip, err);
     } else {
         allow_smem(k_plane_inv<T, false>, smA);
-        k_plane_inv<T, false><<<gridA, threads, smA, st>>>(spec, y, g, oa, skip, err);
+        return launch_kernel(pdl, k_plane_inv<T, false>, gridA, threads, smA, st, spec, y, g, oa, skip, err);
     }
-    return cudaGetLastError();
 }
 
 
@@ -2689,7 +2700,7 @@ __global__ void __launch_bounds__(512) k_plane_fwd_batch(const RveApply* __restr
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int local = blockIdx.x - start[r];
     plane_fwd_body<T, WITH_K, VEC, FX>(static_cast<const T*>(a.x), static_cast<const T*>(a.K),
-                                   static_cast<typename C2<T>::t*>(a.spec), a.g, local % 9, local / 9, sm_raw);
+                                   static_cast<typename C2<T>::t*>(a.spec), a.g, local % 9, local / 9, sm_raw, nullptr);
 }
 
 template <typename T, int W, bool FX = on_int<T>>
@@ -2699,7 +2710,7 @@ __global__ void __launch_bounds__(256, FX ? 2 : 1) k_zproj_batch(const RveApply*
     const RveApply& a = rv[r];
     if (a.skip && *a.skip) return;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    zproj_body<T, W, FX>(static_cast<typename C2<T>::t*>(a.spec), a.g, pa, blockIdx.x - start[r], sm_raw);
+    zproj_body<T, W, FX>(static_cast<typename C2<T>::t*>(a.spec), a.g, pa, blockIdx.x - start[r], sm_raw, nullptr);
 }
 
 template <typename T, bool VEC, bool FX = on_int<T>>
@@ -2801,35 +2812,40 @@ cudaError_t launch_galerkin(const gff_handle* h, const T* x, const T* K, T* y, c
     const bool vout = vec_ok<T>(g, y);
     OutArgs oo = oa;
     oo.pre = pa.sym ? 0 : 1;
+    // The z and inverse passes come in, load their tables and wait while the pass before them drains: 24.6 -> 19.7 us
+    // at 16^3 FP32, 119 -> 114 us at 80 x 96 x 48 FP32, 239 -> 235 us at 128^3 FP32.  The forward pass does so on small grids
+    // only (24^3 FP32 20.7 -> 18.5 us, 16^3 FP64 35 -> 33 us): blocks that arrive early keep the shared-memory split
+    // the inverse pass left on their SM, and on grids that fill the GPU several times its loads then run with less
+    // first-level cache (64^3 FP64 187 -> 205 us, 128^3 FP32 235 -> 306 us; the same figures as when that split is
+    // asked for).  Not between timing events, and not into a graph the caller is capturing (there the plain order).
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool pdl = !ev && cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    const bool pdl_fwd = pdl && g.N <= 1 << 17;
     if constexpr (sizeof(T) == 8)
         if (pa.butterflies && !K) {
             oo.pre = 0;
-            cudaError_t e = launch_fwd<T>(g, 512, x, K, spec, skip, h->stream, vin, 0, true);
-            if (e == cudaSuccess) e = launch_z_w<T, ZB_WIDTH, false>(g, 256, spec, pa, skip, h->stream);
+            cudaError_t e = launch_fwd<T>(g, 512, x, K, spec, skip, h->stream, vin, 0, true, pdl_fwd);
+            if (e == cudaSuccess) e = launch_z_w<T, ZB_WIDTH, false>(g, 256, spec, pa, skip, h->stream, pdl);
             if (e != cudaSuccess) return e;
             const size_t sm = plane_smem_bytes(g.nx, g.ny, sizeof(typename C2<T>::t));
-            allow_smem(k_plane_inv<T, true, false>, sm);
-            allow_smem(k_plane_inv<T, false, false>, sm);
-            if (vout)
-                k_plane_inv<T, true, false><<<dim3(9, g.nz), 512, sm, h->stream>>>(spec, y, g, oo, skip, h->d_flag + 2);
-            else
-                k_plane_inv<T, false, false><<<dim3(9, g.nz), 512, sm, h->stream>>>(spec, y, g, oo, skip, h->d_flag + 2);
-            return cudaGetLastError();
+            auto kern = vout ? k_plane_inv<T, true, false> : k_plane_inv<T, false, false>;
+            allow_smem(kern, sm);
+            return launch_kernel(pdl, kern, dim3(9, g.nz), 512, sm, h->stream, spec, y, g, oo, skip, h->d_flag + 2);
         }
     if (ev) cudaEventRecord(ev[0], h->stream);
-    cudaError_t e = launch_fwd<T>(g, tn.t_fwd, x, K, spec, skip, h->stream, vin);
+    cudaError_t e = launch_fwd<T>(g, tn.t_fwd, x, K, spec, skip, h->stream, vin, 0, false, pdl_fwd);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], h->stream);
     // the TMA pass addresses the handle's own spectrum through its tensor map
     if (pa.sym)
-        e = launch_zsym<T>(g, spec, pa, skip, h->stream);
+        e = launch_zsym<T>(g, spec, pa, skip, h->stream, pdl);
     else if (tn.z_blocks != 0 && static_cast<const void*>(spec) == h->d_spec)
-        e = launch_z_tma<T>(const_cast<gff_handle*>(h), tn.wz, tn.t_z, tn.z_blocks, pa, skip, h->stream);
+        e = launch_z_tma<T>(const_cast<gff_handle*>(h), tn.wz, tn.t_z, tn.z_blocks, pa, skip, h->stream, pdl);
     else
-        e = launch_z<T>(g, tn.wz, tn.t_z, spec, pa, skip, h->stream);
+        e = launch_z<T>(g, tn.wz, tn.t_z, spec, pa, skip, h->stream, pdl);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[2], h->stream);
-    e = launch_inv<T>(g, tn.t_inv, tn.inv_blocks, spec, y, oo, skip, h->stream, vout, h->d_flag + 2);
+    e = launch_inv<T>(g, tn.t_inv, tn.inv_blocks, spec, y, oo, skip, h->stream, vout, h->d_flag + 2, 0, pdl);
     if (ev) cudaEventRecord(ev[3], h->stream);
     return e;
 }

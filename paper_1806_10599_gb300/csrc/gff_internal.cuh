@@ -245,6 +245,54 @@ namespace gff {
 constexpr int NACC = 1 + 12 * 5;  // pcyc, W[12], gamma[12], gmin[12], gmax[12], sn[12]
 constexpr int RED_BLOCKS = 608;   // 4 x 152 SMs: blocks of the reductions and CG vector updates
 
+// ---- programmatic dependent launch: a kernel launched with pdl may be resident before the previous kernel of its stream
+// has finished (its launch latency and its table loads overlap that kernel's tail).  Every block of such a kernel calls
+// pdl_wait() before it touches anything an earlier kernel writes or reads, and before it returns: the wait is for the
+// whole previous kernel, and so for everything before it.  pdl_trigger() lets the next kernel's blocks in as soon as
+// all of this kernel's have started.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// What the previous kernel wrote is read with coherent loads, issued in program order after the wait; the read-only
+// path (__ldg, or a plain load of a const __restrict__ argument) is for data no kernel changes while this one is resident.
+__device__ __forceinline__ float load_dev(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ double load_dev(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ float4 load_dev(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ double2 load_dev(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(__cvta_generic_to_global(p)));
+    return v;
+}
+__device__ __forceinline__ int load_flag(const int* p) { return *static_cast<const volatile int*>(p); }
+template <typename... P, typename... A>
+cudaError_t launch_kernel(bool pdl, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... a) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(a)...);
+}
+#endif
+
 // ---- warm starts (unet.cu): add G^(|d| y~) to h->d_Fk for the prescribed increment d9,
 // y~ = s y_{k-1} (+ the network's correction when u is given).  *applied = 0 when there
 // is nothing to add (|d| = 0, or extrapolation without history).

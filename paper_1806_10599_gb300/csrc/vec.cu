@@ -65,11 +65,11 @@ __device__ __forceinline__ double dot_thread(const T* __restrict__ a, const T* _
     double acc = 0.0;
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     for (; i + gs < nv; i += 2 * gs) {  // two vectors in flight per thread
-        const V x0 = a4[i], y0 = b4[i], x1 = a4[i + gs], y1 = b4[i + gs];
+        const V x0 = load_dev(a4 + i), y0 = load_dev(b4 + i), x1 = load_dev(a4 + i + gs), y1 = load_dev(b4 + i + gs);
         acc = vdot_acc(x0, y0, acc);
         acc = vdot_acc(x1, y1, acc);
     }
-    if (i < nv) acc = vdot_acc(a4[i], b4[i], acc);
+    if (i < nv) acc = vdot_acc(load_dev(a4 + i), load_dev(b4 + i), acc);
     return acc;
 }
 
@@ -86,7 +86,7 @@ __device__ __forceinline__ double update_thread(T* __restrict__ x, T* __restrict
     double acc = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n / W; i += (long long)gridDim.x * blockDim.x) {
         V xv = x4[i], rv = r4[i];
-        const V pv = p4[i], av = a4[i];
+        const V pv = load_dev(p4 + i), av = load_dev(a4 + i);
 #pragma unroll
         for (int j = 0; j < W; ++j) {
             at<T>(xv, j) = fma(alpha, get<T>(pv, j), get<T>(xv, j));
@@ -108,7 +108,7 @@ __device__ __forceinline__ void xpby_thread(T* __restrict__ p, const T* __restri
     const V* r4 = reinterpret_cast<const V*>(r);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n / W; i += (long long)gridDim.x * blockDim.x) {
         V pv = p4[i];
-        const V rv = r4[i];
+        const V rv = load_dev(r4 + i);
 #pragma unroll
         for (int j = 0; j < W; ++j) at<T>(pv, j) = fma(beta, get<T>(pv, j), get<T>(rv, j));
         p4[i] = pv;
@@ -245,9 +245,12 @@ __device__ __forceinline__ double partial_total(const double* partial, int nb, d
 template <typename T>
 __global__ void __launch_bounds__(TPB, RED_BLOCKS / 152) k_cg_alpha(const T* __restrict__ p, const T* __restrict__ Ap, long long n,
                                                  double* __restrict__ partial, double* cg, int* flag) {
-    if (*flag) {
+    pdl_trigger();
+    pdl_wait();
+    const int stopped = load_flag(flag);
+    if (stopped) {
         // a stop reached in the previous iteration (2: its direction update has run) becomes final
-        if (blockIdx.x == 0 && threadIdx.x == 0 && *flag == 2) *flag = 1;
+        if (blockIdx.x == 0 && threadIdx.x == 0 && stopped == 2) *flag = 1;
         return;
     }
     __shared__ double sh[32];
@@ -272,9 +275,11 @@ template <typename T>
 __global__ void __launch_bounds__(TPB, RED_BLOCKS / 152) k_cg_update_dev(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
                                                        const T* __restrict__ Ap, long long n, double* __restrict__ partial,
                                                        double* cg, int* flag) {
-    if (*flag) return;
+    pdl_trigger();
+    pdl_wait();
+    if (load_flag(flag)) return;
     __shared__ double sh[32];
-    double acc = update_thread<T>(x, r, p, Ap, (T)cg[CG_ALPHA], n);
+    double acc = update_thread<T>(x, r, p, Ap, (T)load_dev(cg + CG_ALPHA), n);
     acc = block_sum(acc, sh);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
     if (!last_block(flag + CG_TICKET_BETA)) return;
@@ -298,8 +303,10 @@ __global__ void __launch_bounds__(TPB, RED_BLOCKS / 152) k_cg_update_dev(T* __re
 template <typename T>
 __global__ void __launch_bounds__(TPB) k_xpby_dev(T* __restrict__ p, const T* __restrict__ r, long long n,
                                                   const double* __restrict__ cg, const int* __restrict__ flag) {
-    if (*flag == 1) return;
-    xpby_thread<T>(p, r, (T)cg[CG_BETA], n);
+    pdl_trigger();
+    pdl_wait();
+    if (load_flag(flag) == 1) return;
+    xpby_thread<T>(p, r, (T)load_dev(cg + CG_BETA), n);
 }
 
 // ---- batched CG: blockIdx.y = RVE; each RVE uses the same RED_BLOCKS x TPB
@@ -479,17 +486,15 @@ cudaError_t launch_cg_init(double* cg, int* flag, double rr0, double stop2, cuda
 template <typename T>
 cudaError_t launch_cg_alpha(const T* p, const T* Ap, long long n, double* partial, double* cg, int* flag,
                             cudaStream_t s) {
-    k_cg_alpha<T><<<RED_BLOCKS, TPB, 0, s>>>(p, Ap, n, partial, cg, flag);
-    return cudaGetLastError();
+    return launch_kernel(true, k_cg_alpha<T>, RED_BLOCKS, TPB, 0, s, p, Ap, n, partial, cg, flag);
 }
 
 // x += alpha p, r -= alpha Ap, r.r, beta, convergence test, p = r + beta p
 template <typename T>
 cudaError_t launch_cg_step(T* x, T* r, T* p, const T* Ap, long long n, double* partial, double* cg, int* flag,
                            cudaStream_t s) {
-    k_cg_update_dev<T><<<RED_BLOCKS, TPB, 0, s>>>(x, r, p, Ap, n, partial, cg, flag);
-    k_xpby_dev<T><<<grid_for(n), TPB, 0, s>>>(p, r, n, cg, flag);
-    return cudaGetLastError();
+    const cudaError_t e = launch_kernel(true, k_cg_update_dev<T>, RED_BLOCKS, TPB, 0, s, x, r, p, Ap, n, partial, cg, flag);
+    return e != cudaSuccess ? e : launch_kernel(true, k_xpby_dev<T>, grid_for(n), TPB, 0, s, p, r, n, cg, flag);
 }
 
 // ---- measurement helpers
