@@ -435,7 +435,7 @@ gff_status setup(Batch& B) {
         std::vector<int> s_pl, s_zr, s_zc;
         const gff_handle* rep = B.h[sc.rves[0]];  // the class's own tuned shapes
         Tune tres = rep->tune[0];
-        if (B.mixed) tres.wz = ZB_WIDTH, tres.t_z = 256;  // the FP64-butterfly residual's width
+        if (B.mixed) tres.wz = ZB_WIDTH, tres.t_z = ZB_THREADS;  // the FP64-butterfly residual's strip
         sc.res = class_launch<double>(rc, B.d_res + cbase, spl, szr, tres, false, s_pl, s_zr);
         if (B.mixed)
             sc.cg = class_launch<float>(gc, B.d_cga + cbase, spl, szc, rep->tune[1], true, s_pl, s_zc);

@@ -2824,13 +2824,15 @@ cudaError_t launch_galerkin(const gff_handle* h, const T* x, const T* K, T* y, c
     if constexpr (sizeof(T) == 8)
         if (pa.butterflies && !K) {
             oo.pre = 0;
-            cudaError_t e = launch_fwd<T>(g, 512, x, K, spec, skip, h->stream, vin, 0, true, pdl_fwd);
-            if (e == cudaSuccess) e = launch_z_w<T, ZB_WIDTH, false>(g, 256, spec, pa, skip, h->stream, pdl);
-            if (e != cudaSuccess) return e;
+            // 256 threads a plane where two planes share an SM, else 512; 128 in z: 64^3, 320 us (512 and 256: 370 us)
             const size_t sm = plane_smem_bytes(g.nx, g.ny, sizeof(typename C2<T>::t));
+            const int bt = 2 * sm <= SMEM_MAX ? 256 : 512;
+            cudaError_t e = launch_fwd<T>(g, bt, x, K, spec, skip, h->stream, vin, 0, true, pdl_fwd);
+            if (e == cudaSuccess) e = launch_z_w<T, ZB_WIDTH, false>(g, ZB_THREADS, spec, pa, skip, h->stream, pdl);
+            if (e != cudaSuccess) return e;
             auto kern = vout ? k_plane_inv<T, true, false> : k_plane_inv<T, false, false>;
             allow_smem(kern, sm);
-            return launch_kernel(pdl, kern, dim3(9, g.nz), 512, sm, h->stream, spec, y, g, oo, skip, h->d_flag + 2);
+            return launch_kernel(pdl, kern, dim3(9, g.nz), bt, sm, h->stream, spec, y, g, oo, skip, h->d_flag + 2);
         }
     if (ev) cudaEventRecord(ev[0], h->stream);
     cudaError_t e = launch_fwd<T>(g, tn.t_fwd, x, K, spec, skip, h->stream, vin, 0, false, pdl_fwd);

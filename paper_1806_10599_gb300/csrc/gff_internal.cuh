@@ -331,7 +331,7 @@ cudaError_t fill_rq2(const GridDev& g, double* tab, cudaStream_t st);
 bool make_axis_plan(int n, AxisPlan& p);
 int axis_freq_of_pos(int pos, const AxisPlan& p);
 // columns per block of the FP64-butterfly z pass (ProjArgs::butterflies)
-constexpr int ZB_WIDTH = 8;
+constexpr int ZB_WIDTH = 8, ZB_THREADS = 128;
 // Blocks of the z pass: one per tensor row (3) and W (ky, kx) columns.
 inline int zproj_blocks(const GridDev& g, int W) { return 3 * (int)(((long long)g.ny * g.nxh + W - 1) / W); }
 // Times every candidate launch shape of the three kernels on the handle's own
