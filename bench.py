@@ -361,12 +361,13 @@ FWD2_END = b"template <typename T> constexpr int zproj_width()"
 # with the register-staged inverse, and its own section
 SOURCE_REGIONS = {"k_plane_fwd": [(None, PASS1_END)],
                   "k_plane_fwd2": [(None, PASS1_END), (PLAN_START, PLAN_END), (FWD2_START, FWD2_END)]}
-PROFILE_FILES = {"k_plane_fwd": "k_plane_fwd_fp64_64cube.md", "k_plane_fwd2": "k_plane_fwd2_fp64_64cube.md"}
+PROFILE_FILES = {"k_plane_fwd": "apply_fp64_64cube.md"}
 
 
 def kernel_source_sha1(kernel):
-    """sha1 of the source regions of fft_proj.cu that `kernel` is built from."""
-    src = open(os.path.join(ROOT, "paper_1806_10599_gb300", "csrc", "fft_proj.cu"), "rb").read()
+    """sha1 of the integer butterflies and the source regions of fft_proj.cu that `kernel` is built from."""
+    csrc = os.path.join(ROOT, "paper_1806_10599_gb300", "csrc")
+    src = b"".join(open(os.path.join(csrc, f), "rb").read() for f in ("fixed_bfly.cuh", "fft_proj.cu"))
     parts = []
     for a, b in SOURCE_REGIONS[kernel]:
         i = 0 if a is None else src.find(a)
