@@ -353,7 +353,7 @@ __device__ __forceinline__ void line_keys(const double2* s, int* keys, int n, in
 // holds the 64-bit integers.  me + de62: the biased exponent of bit 62 after the stage.
 template <int R, bool INV, bool FIRST, bool LAST, int CM, int CNB>
 __device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* keys, int n, int len, int NLF, float invNLF,
-                                         int SF, int NLS, int SS, int ES, int tid, int nthr, int de62, bool rin,
+                                         int SF, int NLS, int SS, int ES, int tid, int nthr, int dn, int de62, bool rin,
                                          bool rout) {
     const int m = CM ? CM : len / R, nb = CNB ? CNB : n / R, twstep = CNB ? 1 : n / len;
     const int total = NLF * nb * NLS, st = m * ES;
@@ -379,11 +379,11 @@ __device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* 
                 f[q] = fx::Cq{fx::to_fixed(v.x, key), fx::to_fixed(v.y, key)};
             }
         } else {
-            constexpr int H = FIRST ? 0 : fx::headroom(R);
+            const int H = FIRST ? 0 : dn;
 #pragma unroll
             for (int q = 0; q < R; ++q) {
                 const longlong2 v = reinterpret_cast<const longlong2&>(base[q * st]);
-                f[q] = fx::Cq{fx::shift_down<H>(v.x), fx::shift_down<H>(v.y)};
+                f[q] = fx::Cq{fx::shift_down(v.x, H), fx::shift_down(v.y, H)};
             }
         }
         if (INV && j) {
@@ -412,20 +412,20 @@ __device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* 
 // follow 16), and 4 and 8 alone are plans: only those places are compiled.
 template <int R, bool INV>
 __device__ __forceinline__ void fx_stage_any(bool first, bool last, double2* s, const int4* tw, const int* keys, int n, int len,
-                                             int NLF, float invNLF, int SF, int NLS, int SS, int ES, int tid, int nthr, int de62, bool rin, bool rout) {
+                                             int NLF, float invNLF, int SF, int NLS, int SS, int ES, int tid, int nthr, int dn, int de62, bool rin, bool rout) {
     constexpr bool head = R == 16 || R == 8 || R == 4 || R == 2, tail = R == 5 || R == 3;
     if (first && last) {
         if constexpr (R == 8 || R == 4)
-            fx_stage<R, INV, true, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+            fx_stage<R, INV, true, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
     } else if (first) {
         if constexpr (INV ? tail : head)
-            fx_stage<R, INV, true, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+            fx_stage<R, INV, true, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
     } else if (last) {
         if constexpr (INV ? head : tail)
-            fx_stage<R, INV, false, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+            fx_stage<R, INV, false, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
     } else {
         if constexpr (tail || R == 2)
-            fx_stage<R, INV, false, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout);
+            fx_stage<R, INV, false, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
     }
 }
 
@@ -444,7 +444,7 @@ __host__ __device__ inline int fx_top(int R) {
 // exponent of bit 62 after a forward transform, relative to the line's largest
 __device__ __forceinline__ int fx_out_exp(const AxisPlan& pl) {
     int e = 62 - fx_top(pl.radix[0]);
-    for (int i = 1; i < pl.nst; ++i) e += fx::headroom(pl.radix[i]);
+    for (int i = 1; i < pl.nst; ++i) e += pl.shift[0][i];
     return e;
 }
 
@@ -464,15 +464,16 @@ __device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const Axis
 #define GFF_FX2(A, B)                                                                                                  \
     if (r1 == A && r2 == B) {                                                                                          \
         if (!INV) {                                                                                                    \
-            fx_stage<A, false, true, false, B, B>(s, tw, keys, n, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, 0,       \
+            fx_stage<A, false, true, false, B, B>(s, tw, keys, n, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, 0, 0,    \
                                                   false, rout);                                                        \
             fx_stage<B, false, false, true, 1, A>(s, tw, keys, n, B, NLF, invNLF, SF, NLS, SS, ES, tid, nthr,          \
-                                                  62 - fx::Top<A>::v + fx::headroom(B), false, rout);                  \
+                                                  fx::headroom(B), 62 - fx::Top<A>::v + fx::headroom(B), false, rout); \
         } else {                                                                                                       \
-            fx_stage<B, true, true, false, 1, A>(s, tw, keys, n, B, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, 0, rin,   \
-                                                 false);                                                               \
+            fx_stage<B, true, true, false, 1, A>(s, tw, keys, n, B, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, 0, 0,     \
+                                                 rin, false);                                                          \
             fx_stage<A, true, false, true, B, B>(s, tw, keys, n, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr,           \
-                                                 62 - fx::Top<B>::v + fx::headroom(A) + extra, rin, false);            \
+                                                 fx::headroom(A), 62 - fx::Top<B>::v + fx::headroom(A) + extra, rin,   \
+                                                 false);                                                               \
         }                                                                                                              \
         return;                                                                                                        \
     }
@@ -490,11 +491,12 @@ __device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const Axis
     for (int i = 0; i < pl.nst; ++i) {
         const int R = pl.radix[INV ? pl.nst - 1 - i : i];
         const bool first = i == 0, last = i == pl.nst - 1;
+        const int dn = pl.shift[INV][i];
         if (INV) len *= R;
 #define GFF_FX(RR)                                                                                                     \
     case RR:                                                                                                           \
-        de62 += first ? 62 - fx::Top<RR>::v : fx::headroom(RR);                                                        \
-        fx_stage_any<RR, INV>(first, last, s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, de62, rin, rout); \
+        de62 += first ? 62 - fx::Top<RR>::v : dn;                                                                      \
+        fx_stage_any<RR, INV>(first, last, s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout); \
         break;
         switch (R) {
             GFF_FX(16)
@@ -2118,6 +2120,18 @@ template <typename K> void allow_smem(K kern, size_t bytes) {
 
 }  // namespace
 
+// the bits the FP64 integers give up before each stage, in the order the stages run
+static void plan_shifts(AxisPlan& p) {
+    for (int inv = 0; inv < 2; ++inv) {
+        double bound = 0.0;
+        for (int i = 0; i < p.nst; ++i) {
+            const int R = p.radix[inv ? p.nst - 1 - i : i];
+            if (i == 0) bound = fx_top(R) + 1.5 + fx::log2_radix(R);
+            p.shift[inv][i] = i == 0 ? 0 : fx::stage_shift(R, bound);
+        }
+    }
+}
+
 bool make_axis_plan(int n, AxisPlan& p) {
     if (n < 4 || n > MAXN || (n & 1)) return false;
     int m = n, a2 = 0, a3 = 0, a5 = 0;
@@ -2134,6 +2148,7 @@ bool make_axis_plan(int n, AxisPlan& p) {
             p.nst = 2;
             p.radix[0] = pr[0];
             p.radix[1] = pr[1];
+            plan_shifts(p);
             return true;
         }
     while (a2 >= 4) { p.radix[p.nst++] = 16; a2 -= 4; }
@@ -2142,7 +2157,9 @@ bool make_axis_plan(int n, AxisPlan& p) {
     if (a2 == 1) p.radix[p.nst++] = 2;
     for (int i = 0; i < a5; ++i) p.radix[p.nst++] = 5;
     for (int i = 0; i < a3; ++i) p.radix[p.nst++] = 3;
-    return p.nst <= MAXST;
+    if (p.nst > MAXST) return false;
+    plan_shifts(p);
+    return true;
 }
 
 int axis_freq_of_pos(int pos, const AxisPlan& p) {

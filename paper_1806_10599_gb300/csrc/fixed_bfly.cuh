@@ -9,11 +9,14 @@
 // clocks here with both conversions; conversions are half of that, hence one
 // each way per line and not per stage.
 // Precision: the aligned values carry 57 (first radix 16) to 60 bits below the
-// line's largest; a later stage of radix R gives up log2 R of them as headroom
-// (rounded), while sums grow.  One rounding to 53 bits at the end replaces one
-// per addition.  Against 64-bit references on the GPU: projection at 16^3
-// 2.2e-16 relative (FP64 butterflies 2.7e-16), operator at 128^3 9.2e-16
-// (1.0e-15, mostly the contraction).
+// line's largest; a later stage shifts its inputs down by what its growth needs
+// (stage_shift), while sums grow; shifts and products round to the nearest.  One
+// rounding to 53 bits at the end replaces one per addition.  Relative L2 error
+// against an extended-precision reference (one tensor row, mean stress twice the
+// fluctuation), FP64 butterflies -> integers: projections 16^3 2.4e-16 -> 1.3e-16,
+// 64^3 3.7e-16 -> 1.8e-16, 54 x 90 x 100 4.3e-16 -> 2.7e-16, 128 x 64 x 80 2.8e-16 ->
+// 2.8e-16; operators with their contraction 64^3 5.1e-16 -> 2.6e-16, 54 x 90 x 100
+// 6.4e-16 -> 3.7e-16, 108 x 96 x 50 6.0e-16 -> 3.1e-16.
 // Range: a line whose largest exponent is near overflow or the subnormals, or
 // which holds an infinity or a NaN, runs its stages in FP64 instead (fp64_bfly),
 // so those propagate as they always did.
@@ -43,22 +46,32 @@ __device__ __forceinline__ void split(long long a, int& h, int& l) {
     l = (int)a;
     h = (int)((unsigned)(a >> 32) + ((unsigned)l >> 31));
 }
+// The product (r 2^32 + p) / 2^62 from its partial sums r (high by high) and p (the cross terms, in units 2^32 lower),
+// to the nearest integer: p starts at HALF, and the two low bits come from p.  (Left at zero, as the high word of the
+// product shifted up by two has them, every product is a multiple of four units and about two too small, a bias that
+// adds up over the stages of a plan.)
+constexpr long long HALF = 1LL << 29;
+__device__ __forceinline__ long long join(long long r, long long p) {
+    r += (int)(p >> 32);
+    const unsigned lo = __funnelshift_l((unsigned)p, (unsigned)r, 2);
+    const unsigned hi = __funnelshift_l((unsigned)r, (unsigned)((unsigned long long)r >> 32), 2);
+    return (long long)((unsigned long long)hi << 32 | lo);
+}
 // a c / 2^62 for |a| < 2^62.5: the low-by-low partial product (below a quarter unit) is dropped
 __device__ __forceinline__ long long mul1(long long a, Limbs c) {
     int ah, al;
     split(a, ah, al);
-    const long long p = (long long)ah * c.l + (long long)al * c.h;
-    const long long r = (long long)ah * c.h + (long long)(int)(p >> 32);
-    return (long long)((unsigned long long)r << 2);
+    const long long p = HALF + (long long)ah * c.l + (long long)al * c.h;
+    return join((long long)ah * c.h, p);
 }
-// (a ca + b cb) / 2^62 for |a|, |b| < 2^61 and |ca| + |cb| <= 1.5
+// (a ca + b cb) / 2^62 for |a|, |b| < 2^61.2 (two inputs of radix 5) and |ca| + |cb| <= 1.54 (its sines): the high
+// halves are below 2^29.2 and the low ones at most 2^31, so |p| < 2 2^60.2 + 1.54 2^61 < 2^62.5 and |r| < 1.54 2^59.2
 __device__ __forceinline__ long long mul2(long long a, Limbs ca, long long b, Limbs cb) {
     int ah, al, bh, bl;
     split(a, ah, al);
     split(b, bh, bl);
-    const long long p = (long long)ah * ca.l + (long long)al * ca.h + (long long)bh * cb.l + (long long)bl * cb.h;
-    const long long r = (long long)ah * ca.h + (long long)bh * cb.h + (long long)(int)(p >> 32);
-    return (long long)((unsigned long long)r << 2);
+    const long long p = HALF + (long long)ah * ca.l + (long long)al * ca.h + (long long)bh * cb.l + (long long)bl * cb.h;
+    return join((long long)ah * ca.h + (long long)bh * cb.h, p);
 }
 
 // Twiddle w = (x + i y), 62 fractional bits, as limbs (xh, xl, yh, yl); a w, or a conj(w) when CONJ, for |a| < 2^62.5
@@ -69,11 +82,9 @@ template <bool CONJ> __device__ __forceinline__ Cq twmul(Cq a, int4 w) {
     const int nh = -w.z, nl = -w.w;  // (l > -2^31: limbs_of)
     const int rh = CONJ ? w.z : nh, rl = CONJ ? w.w : nl;  // re = ax wx + ay r
     const int ih = CONJ ? nh : w.z, il = CONJ ? nl : w.w;  // im = ay wx + ax i
-    const long long p = (long long)xh * w.y + (long long)xl * w.x + (long long)yh * rl + (long long)yl * rh;
-    const long long re = (long long)xh * w.x + (long long)yh * rh + (long long)(int)(p >> 32);
-    const long long q = (long long)yh * w.y + (long long)yl * w.x + (long long)xh * il + (long long)xl * ih;
-    const long long im = (long long)yh * w.x + (long long)xh * ih + (long long)(int)(q >> 32);
-    return Cq{(long long)((unsigned long long)re << 2), (long long)((unsigned long long)im << 2)};
+    const long long p = HALF + (long long)xh * w.y + (long long)xl * w.x + (long long)yh * rl + (long long)yl * rh;
+    const long long q = HALF + (long long)yh * w.y + (long long)yl * w.x + (long long)xh * il + (long long)xl * ih;
+    return Cq{join((long long)xh * w.x + (long long)yh * rh, p), join((long long)yh * w.x + (long long)xh * ih, q)};
 }
 // the twiddle as FP64 (for the butterflies that stay in FP64)
 __device__ __forceinline__ double2 tw_fp64(int4 w) {
@@ -105,7 +116,19 @@ template <> struct Top<5> { static constexpr int v = 58; };
 template <> struct Top<4> { static constexpr int v = 59; };
 template <> struct Top<3> { static constexpr int v = 59; };
 
-// bits of headroom a later stage of radix R shifts its inputs down for
+// Bits by which the stage after others shifts its inputs down: what takes their moduli from 2^bound to 2^62.5 / R; bound
+// (log2, after the first stage Top + 1.5 + log2 R) becomes the stage's own.  The fractions count: a plan 4, 5, 5 gives up
+// 3 + 2 bits, not twice the 3 that a radix 5 may grow by, which halves the rounding of its last stage.
+inline double log2_radix(int R) {
+    return R == 16 ? 4.0 : R == 8 ? 3.0 : R == 5 ? 2.321928094887362 : R == 4 ? 2.0 : R == 3 ? 1.584962500721156 : 1.0;
+}
+inline int stage_shift(int R, double& bound) {
+    int k = 0;
+    while (bound - k > 62.5 - log2_radix(R) + 1e-9) ++k;
+    bound += log2_radix(R) - k;
+    return k;
+}
+// stage_shift of the second stage of a plan of two powers of two or one and a 3 or 5, either way round
 __host__ __device__ constexpr int headroom(int R) { return R == 16 ? 4 : R == 8 || R == 5 ? 3 : R == 4 || R == 3 ? 2 : 1; }
 
 // The butterflies of the FP64 code (fft_proj.cu), on integers.
@@ -242,9 +265,7 @@ __device__ __forceinline__ double from_fixed(long long v, int e62) {
 __device__ __forceinline__ int key_max(int m, double d) { return max(m, __double2hiint(d) & 0x7fffffff); }
 
 // v / 2^k to the nearest integer
-template <int k> __device__ __forceinline__ long long shift_down(long long v) {
-    return k ? (v + ((1LL << k) >> 1)) >> k : v;
-}
+__device__ __forceinline__ long long shift_down(long long v, int k) { return (v + ((1LL << k) >> 1)) >> k; }
 
 // exponents this far from both ends of the range leave room for the growth of a line and for its last bit
 constexpr int ME_MIN = 80, ME_MAX = 0x7f0;

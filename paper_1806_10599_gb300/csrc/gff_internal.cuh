@@ -38,6 +38,7 @@ struct AxisPlan {
     int n;
     int nst;
     int radix[MAXST];
+    int shift[2][MAXST];  // FP64 on integers: bits the inputs of the i-th stage to run are shifted down (forward, inverse)
 };
 
 // Read-only tables of one grid, resident on the device.
