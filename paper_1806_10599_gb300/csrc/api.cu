@@ -830,12 +830,8 @@ GFF_EXPORT gff_status gff_autotune(gff_handle* h, int* tiles_out) {
 
 GFF_EXPORT gff_status gff_project(gff_handle* h, int precision, const uint8_t* mask9, const void* x_dev, void* y_dev) {
     if (!h || !x_dev || !y_dev || x_dev == y_dev) return fail(h, GFF_ERR_ARG, "bad project args");
-    ProjArgs pa = proj_args(h, mask9);
+    const ProjArgs pa = proj_args(h, mask9);
     const OutArgs oa = out_args(h, 1.0, nullptr);
-    // The mean of a stress field dominates its lines, and longer lines on integers leave the fluctuations fewer bits.
-    // Error against 64 bits, FP64 butterflies and integers: 16^3 2.5e-16 and 2.2e-16, 32^3 2.9e-16 and 2.8e-16,
-    // 48 x 40 x 36 3.2e-16 and 4.2e-16, 64^3 3.7e-16 and 4.2e-16, 54 x 90 x 100 3.9e-16 and 7.1e-16.
-    pa.butterflies = !pa.sym && std::max({h->grid.nx, h->grid.ny, h->grid.nz}) > 32;
     if (precision == GFF_PREC_FP64) {
         GFF_TRY(launch_galerkin<double>(h, (const double*)x_dev, (const double*)nullptr, (double*)y_dev, pa, oa,
                                         h->d_spec));

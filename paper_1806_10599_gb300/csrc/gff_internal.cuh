@@ -64,10 +64,10 @@ struct ProjArgs {
     int kind;        // GFF_PROJ_*
     float mask[9];   // 1 = stress-controlled component (zero frequency keeps it)
     int sym = 0;     // 1: small-strain variant, projection onto compatible symmetric fields
-    // FP64 data, no K: 1: transforms by FP64 butterflies instead of integers (gff_project on long axes).  The residuals of mixed precision, which
-    // round to FP32 right after: a residual that differs in its last bits moves the converged fields by 1e-8 (rounding
-    // of the FP32 vectors, amplified by the soft plastic modes), and runs and state files of earlier builds would no
-    // longer be repeated bit for bit.  These projections are 4 % of a mixed increment.
+    // FP64 data, no K: 1: transforms by FP64 butterflies instead of integers.  Set for the residuals of mixed precision
+    // (finite strain), which round to FP32 right after: a residual that differs in its last bits moves the converged
+    // fields by 1e-8 (rounding of the FP32 vectors, amplified by the soft plastic modes), and runs and state files of
+    // earlier builds would no longer be repeated bit for bit.  These projections are 4 % of a mixed increment.
     int butterflies = 0;
 };
 

@@ -74,3 +74,27 @@ def test_error_against_extended_precision(shape):
     ref = extended_projection(x, shape)
     d = y.astype(np.longdouble) - ref
     assert float(np.sqrt((d * d).sum() / (ref * ref).sum())) <= BOUND
+
+
+@pytest.mark.parametrize("tuned", [False, True])
+@pytest.mark.parametrize("shape", SHAPES + [(64, 8, 8), (16, 64, 64), (40, 36, 48)])
+def test_projections_take_the_arithmetic_of_operators(shape, tuned):
+    """One arithmetic at every size and with every launch shape: with K = identity
+    the operator is the bare projection, bit for bit."""
+    torch = torch_cuda()
+    g = gff()
+    h = identity_handle(g, shape)
+    try:
+        if tuned:
+            g.gff_autotune(h)
+        X = torch.from_numpy(field(shape)).cuda()
+        Y, Z = torch.empty_like(X), torch.empty_like(X)
+        for mask in (None, [0, 1, 1, 1, 1, 1, 1, 0, 1]):
+            m = None if mask is None else np.array(mask, dtype=np.uint8)
+            g.gff_apply_operator(h, g.GFF_PREC_FP64, m, X, Y)
+            g.gff_project(h, g.GFF_PREC_FP64, m, X, Z)
+            g.gff_sync(h)
+            assert torch.equal(Y, Z)
+    finally:
+        torch.cuda.synchronize()
+        g.gff_destroy(h)
