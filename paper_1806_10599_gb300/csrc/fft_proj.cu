@@ -2489,9 +2489,9 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
 }
 
 
-// fastest candidate of one kernel: run(i) launches candidate i `reps` times
-template <typename F>
-cudaError_t pick_fastest(int ncand, const bool* valid, int reps, cudaStream_t st, F run, int* best) {
+// fastest candidate of one kernel: set() lays out its input, run(i) launches candidate i, `reps` times in the timed part
+template <typename S, typename F>
+cudaError_t pick_fastest(int ncand, const bool* valid, int reps, cudaStream_t st, S set, F run, int* best) {
     cudaEvent_t e0, e1;
     cudaError_t e = cudaEventCreate(&e0);
     if (e != cudaSuccess) return e;
@@ -2504,7 +2504,8 @@ cudaError_t pick_fastest(int ncand, const bool* valid, int reps, cudaStream_t st
     *best = -1;
     for (int i = 0; i < ncand && e == cudaSuccess; ++i) {
         if (!valid[i]) continue;
-        e = run(i);  // warm-up (also sets the shared-memory attribute)
+        e = set();
+        if (e == cudaSuccess) e = run(i);  // warm-up (also sets the shared-memory attribute)
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
         for (int r = 0; r < reps && e == cudaSuccess; ++r) e = run(i);
         if (e == cudaSuccess) e = cudaEventRecord(e1, st);
@@ -2572,13 +2573,39 @@ int inv2s_blocks(const GridDev& g, int threads) {
     return n < total ? n : total;
 }
 
+// The launch order of an apply's passes outside timing and capture (launch_galerkin): which start while the pass before
+// drains
+inline bool forward_starts_early(const GridDev& g) { return g.N <= 1 << 17; }
+
+// Values of either sign with moduli in [1, 2), by integer operations.
+__device__ __forceinline__ double tune_value(unsigned r, double) {
+    return __hiloint2double((int)(0x3ff00000u | (r & 0x800fffffu)), (int)(r * 2654435761u));
+}
+__device__ __forceinline__ float tune_value(unsigned r, float) { return __uint_as_float(0x3f800000u | (r & 0x807fffffu)); }
+template <typename T> __global__ void __launch_bounds__(256) k_tune_fill(T* p, long long n) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        unsigned r = (unsigned)i * 0x9e3779b1u;  // (a hash: neighbours differ in every bit)
+        r = (r ^ (r >> 15)) * 0x85ebca6bu;
+        p[i] = tune_value(r ^ (r >> 13), T(0));
+    }
+}
+template <typename T> cudaError_t tune_fill(T* p, long long n, cudaStream_t st) {
+    k_tune_fill<T><<<608, 256, 0, st>>>(p, n);
+    return cudaGetLastError();
+}
+
+// x, K and what the passes make of them hold values like a field's: an FP64 line of zeros leaves its integer stages at
+// once, and shapes compared on zeros are compared without their transforms (at 80 x 96 x 48 that took the inverse pass of
+// 512 threads, 328 us per apply, for the one of 256, 312 us).  The passes are launched as an apply launches them.
 template <typename T>
 cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     using C = typename C2<T>::t;
     const GridDev& g = h->g;
     C* spec = reinterpret_cast<C*>(h->d_spec);
     cudaStream_t st = h->stream;
-    const int reps = 3;
+    const int reps = g.N <= 1 << 17 ? 10 : 3;  // passes of a few microseconds differ by less than one
+    const bool pdl_fwd = forward_starts_early(g);
+    auto nothing = [] { return cudaSuccess; };
     Tune& tn = h->tune[tune_index<T>()];
     const bool vin = vec_ok<T>(g, x) && vec_ok<T>(g, K);
     // forward pass: 256 or 512 threads, or (two-stage plans, nx = ny) the register-staged pass (-256, -512)
@@ -2587,7 +2614,9 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     const int tp[4] = {256, 512, -256, -512};
     const bool tv[4] = {true, true, f2, f2};
     int b = -1;
-    cudaError_t e = pick_fastest(4, tv, reps, st, [&](int i) { return launch_fwd<T>(g, tp[i], x, K, spec, nullptr, st, vin); }, &b);
+    cudaError_t e = pick_fastest(4, tv, reps, st, nothing, [&](int i) {
+        return launch_fwd<T>(g, tp[i], x, K, spec, nullptr, st, vin, 0, false, pdl_fwd);
+    }, &b);
     if (e != cudaSuccess) return e;
     tn.t_fwd = tp[b];
     // z pass: one block per strip (W 4..32, 128 or 256 threads), or the persistent TMA pass (W 8, 16; 256, 512)
@@ -2611,10 +2640,16 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     ProjArgs pa;
     pa.kind = GFF_PROJ_CONTINUOUS;
     for (int c = 0; c < 9; ++c) pa.mask[c] = 0.f;
-    e = pick_fastest(NZC, zv, reps, st, [&](int i) {
-        return zb[i] != 0 ? launch_z_tma<T>(h, wz[i], tz[i], zb[i], pa, nullptr, st)
-                     : launch_z<T>(g, wz[i], tz[i], spec, pa, nullptr, st);
-    }, &b);
+    // (in place: the spectrum shrinks by 1 / N with every FP64 launch, and is laid out anew for every candidate)
+    auto spectrum = [&] { return launch_fwd<T>(g, tn.t_fwd, x, K, spec, nullptr, st, vin); };
+    auto z_pass = [&](int i) {
+        return zb[i] != 0 ? launch_z_tma<T>(h, wz[i], tz[i], zb[i], pa, nullptr, st, true)
+                     : launch_z<T>(g, wz[i], tz[i], spec, pa, nullptr, st, true);
+    };
+    e = pick_fastest(NZC, zv, reps, st, spectrum, z_pass, &b);
+    if (e != cudaSuccess) return e;
+    e = spectrum();  // projected, as the inverse pass finds it
+    if (e == cudaSuccess) e = z_pass(b);
     if (e != cudaSuccess) return e;
     tn.wz = wz[b];
     tn.t_z = tz[b];
@@ -2632,7 +2667,9 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     const bool r2 = staged && inv2_radix(g) > 0 && inv2_smem<T>(g) <= SMEM_MAX;
     const bool iv[8] = {true, true, ib[2] > 0, ib[3] > 0, r2, r2, ib[6] < -1, ib[7] < -1};
     int* err = h->d_flag + 2;
-    e = pick_fastest(8, iv, reps, st, [&](int i) { return launch_inv<T>(g, ti[i], ib[i], spec, y, oa, nullptr, st, vout, err); }, &b);
+    e = pick_fastest(8, iv, reps, st, nothing, [&](int i) {
+        return launch_inv<T>(g, ti[i], ib[i], spec, y, oa, nullptr, st, vout, err, 0, true);
+    }, &b);
     if (e != cudaSuccess) return e;
     tn.t_inv = ti[b];
     tn.inv_blocks = ib[b];
@@ -2684,12 +2721,11 @@ cudaError_t autotune_galerkin(gff_handle* h) {
     // timings are taken at the default wait budget, whatever the handle's is
     const long long wait = h->g.wait_cycles;
     h->g.wait_cycles = BULK_WAIT_CYCLES;
-    // the kernels' cost does not depend on the values: the handle's vectors serve as inputs
-    cudaError_t e = cudaMemsetAsync(h->d_x, 0, 9 * h->N * sizeof(double), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_x32, 0, 9 * h->N * sizeof(float), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_K32, 0, 81 * h->N * sizeof(float), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->d_Ap, 0, 9 * h->N * sizeof(double), h->stream);
-    // K: the tangent buffer is only read (its contents do not matter for timing)
+    // the handle's vectors serve as inputs; a valid tangent is read as it is, the place of one that is not is filled
+    cudaError_t e = tune_fill(h->d_x, 9 * h->N, h->stream);
+    if (e == cudaSuccess) e = tune_fill(h->d_x32, 9 * h->N, h->stream);
+    if (e == cudaSuccess) e = tune_fill(h->d_K32, 81 * h->N, h->stream);
+    if (e == cudaSuccess && !h->K_valid) e = tune_fill(h->d_K, 81 * h->N, h->stream);
     if (e == cudaSuccess) e = autotune_prec<double>(h, h->d_x, h->d_Ap, h->d_K);
     if (e == cudaSuccess) e = autotune_prec<float>(h, h->d_x32, h->d_Ap32, h->d_K32);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -2837,7 +2873,7 @@ cudaError_t launch_galerkin(const gff_handle* h, const T* x, const T* K, T* y, c
     // asked for).  Not between timing events, and not into a graph the caller is capturing (there the plain order).
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool pdl = !ev && cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-    const bool pdl_fwd = pdl && g.N <= 1 << 17;
+    const bool pdl_fwd = pdl && forward_starts_early(g);
     if constexpr (sizeof(T) == 8)
         if (pa.butterflies && !K) {
             oo.pre = 0;
