@@ -309,13 +309,14 @@ __device__ __forceinline__ void fft2_lines(typename C2<T>::t* s, const typename 
 }
 
 // ---------------------------------------------------------------- FP64 lines in fixed point (fixed_bfly.cuh)
-// The stage of a line the integers do not take, in FP64.  Out of line: it is the exception.
+// The stage of a line the integers do not take, in FP64, and its results over 2^down.  Out of line: it is the exception.
 template <int R, bool INV>
-__device__ __noinline__ void fp64_bfly(double2* base, int st, const int4* tw, int pstep) {
+__device__ __noinline__ void fp64_bfly(double2* base, int st, const int4* tw, int pstep, int down) {
     double2 v[R];
     for (int q = 0; q < R; ++q) v[q] = base[q * st];
     bfly<R, INV>(v, pstep != 0, [&](int p) { return fx::tw_fp64(tw[p * pstep]); });
-    for (int q = 0; q < R; ++q) base[q * st] = v[q];
+    const double sc = __hiloint2double((1023 - down) << 20, 0);
+    for (int q = 0; q < R; ++q) base[q * st] = cscale(v[q], sc);
 }
 
 // Largest exponent key of every line (l as in run_stage) into keys[l]: eight lanes per line, four
@@ -328,18 +329,16 @@ __device__ __forceinline__ void line_keys(const double2* s, int* keys, int n, in
     const int part = rows ? lane & 7 : lane >> 2, sub = rows ? lane >> 3 : lane & 3;
     for (int l0 = (tid >> 5) * 4; l0 < L; l0 += (nthr >> 5) * 4) {  // warp-uniform
         const int l = l0 + sub;
-        int mk = 0;
+        fx::Key key;
         if (l < L) {
             int lf;
             const int ls = divmod_f(l, NLF, invNLF, lf);
             const double2* b = s + ls * SS + lf * SF;
 #pragma unroll 4
-            for (int e = part; e < n; e += 8) {
-                const double2 v = b[e * ES];
-                mk = fx::key_max(fx::key_max(mk, v.x), v.y);
-            }
+            for (int e = part; e < n; e += 8) key.add(b[e * ES]);
         }
         const int o = rows ? 1 : 4;
+        int mk = key.get();
         mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, o));
         mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, 2 * o));
         mk = max(mk, __shfl_xor_sync(0xffffffffu, mk, 4 * o));
@@ -350,11 +349,11 @@ __device__ __forceinline__ void line_keys(const double2* s, int* keys, int n, in
 // One radix stage of every line, tasks as in run_stage (m = CM, nb = CNB where not 0).  FIRST:
 // aligns the line's values to its largest exponent (rin: they are integers aligned for this stage
 // already); LAST: rounds back to FP64 (rout: leaves the integers); between stages the shared memory
-// holds the 64-bit integers.  me + de62: the biased exponent of bit 62 after the stage.
+// holds the 64-bit integers.  me + de62: the biased exponent of bit 62 after the stage.  LAST: the results over 2^down.
 template <int R, bool INV, bool FIRST, bool LAST, int CM, int CNB>
 __device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* keys, int n, int len, int NLF, float invNLF,
                                          int SF, int NLS, int SS, int ES, int tid, int nthr, int dn, int de62, bool rin,
-                                         bool rout) {
+                                         bool rout, int down = 0) {
     const int m = CM ? CM : len / R, nb = CNB ? CNB : n / R, twstep = CNB ? 1 : n / len;
     const int total = NLF * nb * NLS, st = m * ES;
     for (int idx = tid; idx < total; idx += nthr) {
@@ -367,7 +366,7 @@ __device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* 
         const int lk = keys[lsl * NLF + lf], me = lk >> 20;
         if (lk == 0) continue;
         if (me < fx::ME_MIN || me > fx::ME_MAX) {
-            fp64_bfly<R, INV>(base, st, tw, j * twstep);
+            fp64_bfly<R, INV>(base, st, tw, j * twstep, LAST ? down : 0);
             continue;
         }
         fx::Cq f[R];
@@ -396,7 +395,7 @@ __device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* 
             for (int p = 1; p < R; ++p) f[p] = fx::twmul<false>(f[p], tw[p * j * twstep]);
         }
         if (LAST && !rout) {
-            const int e62 = me + de62;
+            const int e62 = me + de62 - down;
 #pragma unroll
             for (int q = 0; q < R; ++q)
                 base[q * st] = make_double2(fx::from_fixed(f[q].x, e62), fx::from_fixed(f[q].y, e62));
@@ -412,17 +411,18 @@ __device__ __forceinline__ void fx_stage(double2* s, const int4* tw, const int* 
 // follow 16), and 4 and 8 alone are plans: only those places are compiled.
 template <int R, bool INV>
 __device__ __forceinline__ void fx_stage_any(bool first, bool last, double2* s, const int4* tw, const int* keys, int n, int len,
-                                             int NLF, float invNLF, int SF, int NLS, int SS, int ES, int tid, int nthr, int dn, int de62, bool rin, bool rout) {
+                                             int NLF, float invNLF, int SF, int NLS, int SS, int ES, int tid, int nthr, int dn, int de62, bool rin, bool rout,
+                                             int down) {
     constexpr bool head = R == 16 || R == 8 || R == 4 || R == 2, tail = R == 5 || R == 3;
     if (first && last) {
         if constexpr (R == 8 || R == 4)
-            fx_stage<R, INV, true, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
+            fx_stage<R, INV, true, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout, down);
     } else if (first) {
         if constexpr (INV ? tail : head)
             fx_stage<R, INV, true, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
     } else if (last) {
         if constexpr (INV ? head : tail)
-            fx_stage<R, INV, false, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
+            fx_stage<R, INV, false, true, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout, down);
     } else {
         if constexpr (tail || R == 2)
             fx_stage<R, INV, false, false, 0, 0>(s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout);
@@ -436,8 +436,8 @@ __device__ __forceinline__ int* fx_line_keys() {
     return keys;
 }
 // Integers as they enter or leave a transform: IN: aligned for its first stage, their keys given; OUT: left as they are
-// after its last stage, their exponents me + fx_out_exp(plan).
-enum { FX_FP64 = 0, FX_IN = 1, FX_OUT = 2 };
+// after its last stage, their exponents me + fx_out_exp(plan).  Times FX_DOWN: the results over that power of two.
+enum { FX_FP64 = 0, FX_IN = 1, FX_OUT = 2, FX_DOWN = 4 };
 __host__ __device__ inline int fx_top(int R) {
     return R == 16 ? fx::Top<16>::v : R == 8 ? fx::Top<8>::v : R == 5 ? fx::Top<5>::v : R == 4 ? fx::Top<4>::v : R == 3 ? fx::Top<3>::v : fx::Top<2>::v;
 }
@@ -454,6 +454,7 @@ __device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const Axis
     const int n = pl.n;
     const float invNLF = 1.0f / (float)NLF;
     const bool rin = INV && (io & FX_IN), rout = !INV && (io & FX_OUT);
+    const int down = INV ? io / FX_DOWN : 0;
     if (!rin) {
         line_keys(s, keys, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr);
         __syncthreads();
@@ -473,7 +474,7 @@ __device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const Axis
                                                  rin, false);                                                          \
             fx_stage<A, true, false, true, B, B>(s, tw, keys, n, n, NLF, invNLF, SF, NLS, SS, ES, tid, nthr,           \
                                                  fx::headroom(A), 62 - fx::Top<B>::v + fx::headroom(A) + extra, rin,   \
-                                                 false);                                                               \
+                                                 false, down);                                                         \
         }                                                                                                              \
         return;                                                                                                        \
     }
@@ -496,7 +497,7 @@ __device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const Axis
 #define GFF_FX(RR)                                                                                                     \
     case RR:                                                                                                           \
         de62 += first ? 62 - fx::Top<RR>::v : dn;                                                                      \
-        fx_stage_any<RR, INV>(first, last, s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout); \
+        fx_stage_any<RR, INV>(first, last, s, tw, keys, n, len, NLF, invNLF, SF, NLS, SS, ES, tid, nthr, dn, de62, rin, rout, down); \
         break;
         switch (R) {
             GFF_FX(16)
@@ -946,9 +947,11 @@ __device__ __forceinline__ void zrow_proj(typename C2<T>::t& u, typename C2<T>::
         v = cscale(t, d);
     }
 }
-// The FP64 projection also applies the inverse transform's 1 / N (sc; the masks come multiplied by it): it costs nothing in
-// the factor r = sc / |q|^2, which the grid's table holds (a division per frequency is half of the FP64 operations of
+// The FP64 projection also applies the inverse transform's 1 / N, but for a power of two near sqrt(N) that the last stage
+// of the inverse takes off its exponents (half_exp; the whole 1 / N here left small fields, 1e-317 say, a few bits of
+// the subnormals).  sc = 2^half_exp / N, which the masks come multiplied by, costs nothing in the factor r = sc / |q|^2, which the grid's table holds (a division per frequency is half of the FP64 operations of
 // this pass), and saves the plane pass an FP64 operation per voxel.
+__device__ __forceinline__ int half_exp(const GridDev& g) { return (32 - __clz((int)g.N)) >> 1; }
 __device__ __forceinline__ void zrow_proj64(double2& u, double2& v, int kx, int ky, int kz, int nx, int ny, int nz, double m0,
                                             double m1, double m2, double sc, const double* rq2, long long at,
                                             const ZTables<double>& tb) {
@@ -979,7 +982,7 @@ __device__ __forceinline__ void zrow_proj64(double2& u, double2& v, int kx, int 
 // the table: one thread per position (pz, py, kx) of the half spectrum, both kinds; the expression above
 __global__ void __launch_bounds__(256) k_fill_rq2(GridDev g, double* tab) {
     const int nF = g.ny * g.nxh, total = g.nz * nF;
-    const double sc = 1.0 / (double)g.N;
+    const double sc = scalbn(1.0 / (double)g.N, half_exp(g));
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * total; i += gridDim.x * blockDim.x) {
         const int kind = i / total, e = i - kind * total;
         const int pz = e / nF, f = e - pz * nF, py = f / g.nxh, kx = f - py * g.nxh;
@@ -1003,7 +1006,7 @@ __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev&
     for (int e = tid; e < nz * W; e += nthr) s[e] = zpack<T>(s[e], s[nz * W + e], zcol<T>(tb.colk[e % W], tb));
     __syncthreads();
     fft_lines<T, false, FX>(s, as_tw<T, FX>(tb.twz), g.az, W, 1, 2, 2 * nz * W, W, tid, nthr);
-    const T sc = FX ? (T)1 / (T)g.N : (T)1;
+    const T sc = FX ? (T)scalbn(1.0 / (double)g.N, half_exp(g)) : (T)1;
     const T m0 = (T)pa.mask[3 * row] * sc, m1 = (T)pa.mask[3 * row + 1] * sc, m2 = (T)pa.mask[3 * row + 2] * sc;
     for (int e = tid; e < nz * W; e += nthr) {
         const int w = e % W, pz = e / W;
@@ -1440,12 +1443,14 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
         if constexpr (FX) {
             // FP64: one row per warp; aligned to the largest value of both half spectra, one bit below the first
             // stage's alignment (|A| + |B|), and merged as integers
-            int mkey = 0;
+            fx::Key row_key;
 #pragma unroll
             for (int t = 0; t < SPLIT_K<T>; ++t)
-                if (kg + SPLIT_G<T> * t <= kh)
-                    mkey = fx::key_max(fx::key_max(fx::key_max(fx::key_max(mkey, A[t].x), A[t].y), B[t].x), B[t].y);
-            mkey = (int)__reduce_max_sync(0xffffffffu, (unsigned)mkey);
+                if (kg + SPLIT_G<T> * t <= kh) {
+                    row_key.add(A[t]);
+                    row_key.add(B[t]);
+                }
+            const int mkey = (int)__reduce_max_sync(0xffffffffu, (unsigned)row_key.get());
             if (lane == 0) fx_line_keys()[r] = mkey;
             const int me = mkey >> 20;
             if (me >= fx::ME_MIN && me <= fx::ME_MAX) {
@@ -1483,11 +1488,12 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
         }
     }
     __syncthreads();
-    fft_lines<T, true, FX>(s, as_tw<T, FX>(twx), g.ax, half, 2 * ls, 1, 0, 1, tid, nthr, FX_IN);  // rows fastest, as in pass 1
+    fft_lines<T, true, FX>(s, as_tw<T, FX>(twx), g.ax, half, 2 * ls, 1, 0, 1, tid, nthr,
+                             FX_IN + (FX && oa.pre ? FX_DOWN * half_exp(g) : 0));  // rows fastest, as in pass 1
     T sc = (T)oa.scale;
     const T ad = (T)oa.add[c];
     if constexpr (FX) {
-        if (oa.pre) {  // the z pass has applied |scale|
+        if (oa.pre) {  // the z pass and the last stage have applied |scale|
             sc = sc < 0 ? -1.0 : 1.0;
             if (ad == 0) {
                 plane_store<T, VEC, true>(s, y + c * N, pl, g, sc, ad);
@@ -2640,7 +2646,7 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     ProjArgs pa;
     pa.kind = GFF_PROJ_CONTINUOUS;
     for (int c = 0; c < 9; ++c) pa.mask[c] = 0.f;
-    // (in place: the spectrum shrinks by 1 / N with every FP64 launch, and is laid out anew for every candidate)
+    // (in place: the spectrum changes its size with every launch, and is laid out anew for every candidate)
     auto spectrum = [&] { return launch_fwd<T>(g, tn.t_fwd, x, K, spec, nullptr, st, vin); };
     auto z_pass = [&](int i) {
         return zb[i] != 0 ? launch_z_tma<T>(h, wz[i], tz[i], zb[i], pa, nullptr, st, true)

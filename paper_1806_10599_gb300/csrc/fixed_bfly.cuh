@@ -262,7 +262,16 @@ __device__ __forceinline__ double from_fixed(long long v, int e62) {
     return __hiloint2double((int)h, (int)(unsigned)r);
 }
 
-__device__ __forceinline__ int key_max(int m, double d) { return max(m, __double2hiint(d) & 0x7fffffff); }
+// Largest exponent key of a line's values: their high words without the sign, and bit 0 where a low word is not zero
+// (below 2^-1042 the high word is zero), so that only a line of zeros has key 0.
+struct Key {
+    int m = 0, low = 0;
+    __device__ __forceinline__ void add(const double2& v) {
+        m = max(max(m, __double2hiint(v.x) & 0x7fffffff), __double2hiint(v.y) & 0x7fffffff);
+        low |= __double2loint(v.x) | __double2loint(v.y);
+    }
+    __device__ __forceinline__ int get() const { return m | (low != 0 ? 1 : 0); }
+};
 
 // v / 2^k to the nearest integer
 __device__ __forceinline__ long long shift_down(long long v, int k) { return (v + ((1LL << k) >> 1)) >> k; }

@@ -54,7 +54,7 @@ struct GridDev {
     const int* fqz;          // [nz]
     const double* qt64[2][3];  // [kind][axis][k]: q~ (continuous) or q~' (discrete) per FFT index
     const float* qt32[2][3];
-    const double* rq2[2];      // [kind][nz][ny nxh] in the order of the half spectrum: 1 / (N |q|^2), 0 where the projection
+    const double* rq2[2];      // [kind][nz][ny nxh] in the order of the half spectrum: 2^half_exp / (N |q|^2), 0 where the projection
                                // is zero or special (null: the z pass divides instead)
     long long wait_cycles;     // budget of the first wait on each bulk load (BULK_WAIT_CYCLES by default)
 };
@@ -75,7 +75,7 @@ struct ProjArgs {
 struct OutArgs {
     double scale;
     double add[9];
-    int pre = 1;  // FP64: 1: the z pass has multiplied by 1 / N = |scale| already; 0 (small strain): it has not
+    int pre = 1;  // FP64: 1: 1 / N = |scale| is shared by the z pass and the last stage (half_exp); 0 (small strain): not applied yet
 };
 
 // ---- batched launches: one launch serves several RVEs of different sizes.
