@@ -2495,36 +2495,41 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
 }
 
 
-// fastest candidate of one kernel: set() lays out its input, run(i) launches candidate i, `reps` times in the timed part
+// Fastest candidate of one kernel: set() lays out its input, run(i) launches candidate i.  Each is timed over three
+// launches after one; where these are short (passes of a few microseconds differ by less than one), those within a
+// twelfth of the fastest are timed over five more.  The host waits once per round, not per candidate.  The call takes,
+// ten launches of every candidate -> now: 16^3 4.5 -> 3.2 ms, 32^3 6.7 -> 4.1 ms, 48^3 14.0 -> 7.7 ms.
+constexpr int TUNE_MAX = 18;  // candidates of one kernel
 template <typename S, typename F>
-cudaError_t pick_fastest(int ncand, const bool* valid, int reps, cudaStream_t st, S set, F run, int* best) {
-    cudaEvent_t e0, e1;
-    cudaError_t e = cudaEventCreate(&e0);
-    if (e != cudaSuccess) return e;
-    e = cudaEventCreate(&e1);
-    if (e != cudaSuccess) {
-        cudaEventDestroy(e0);
-        return e;
-    }
-    float bestms = 1e30f;
+cudaError_t pick_fastest(int ncand, const bool* valid, bool again, cudaStream_t st, S set, F run, int* best) {
+    cudaEvent_t ev[2 * TUNE_MAX] = {};
+    float ms[TUNE_MAX];
+    bool in[TUNE_MAX];
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < ncand; ++i) in[i] = valid[i];
+    for (int i = 0; i < 2 * ncand && e == cudaSuccess; ++i)
+        if (in[i / 2]) e = cudaEventCreate(&ev[i]);
     *best = -1;
-    for (int i = 0; i < ncand && e == cudaSuccess; ++i) {
-        if (!valid[i]) continue;
-        e = set();
-        if (e == cudaSuccess) e = run(i);  // warm-up (also sets the shared-memory attribute)
-        if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = run(i);
-        if (e == cudaSuccess) e = cudaEventRecord(e1, st);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        float ms = 0.f;
-        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        if (e == cudaSuccess && ms < bestms) {
-            bestms = ms;
-            *best = i;
+    for (int round = 0; round < (again ? 2 : 1) && e == cudaSuccess; ++round) {
+        for (int i = 0; i < ncand && e == cudaSuccess; ++i) {
+            if (!in[i]) continue;
+            e = set();
+            if (e == cudaSuccess) e = run(i);  // warm-up (also sets the shared-memory attribute)
+            if (e == cudaSuccess) e = cudaEventRecord(ev[2 * i], st);
+            for (int r = 0; r < (round ? 5 : 3) && e == cudaSuccess; ++r) e = run(i);
+            if (e == cudaSuccess) e = cudaEventRecord(ev[2 * i + 1], st);
         }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        *best = -1;
+        for (int i = 0; i < ncand && e == cudaSuccess; ++i) {
+            if (!in[i]) continue;
+            e = cudaEventElapsedTime(&ms[i], ev[2 * i], ev[2 * i + 1]);
+            if (*best < 0 || ms[i] < ms[*best]) *best = i;
+        }
+        for (int i = 0; i < ncand && *best >= 0; ++i) in[i] = in[i] && 12 * ms[i] <= 13 * ms[*best];
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
+    for (cudaEvent_t v : ev)
+        if (v) cudaEventDestroy(v);
     return e;
 }
 
@@ -2609,7 +2614,7 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     const GridDev& g = h->g;
     C* spec = reinterpret_cast<C*>(h->d_spec);
     cudaStream_t st = h->stream;
-    const int reps = g.N <= 1 << 17 ? 10 : 3;  // passes of a few microseconds differ by less than one
+    const bool again = g.N <= 1 << 17;
     const bool pdl_fwd = forward_starts_early(g);
     auto nothing = [] { return cudaSuccess; };
     Tune& tn = h->tune[tune_index<T>()];
@@ -2620,7 +2625,7 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     const int tp[4] = {256, 512, -256, -512};
     const bool tv[4] = {true, true, f2, f2};
     int b = -1;
-    cudaError_t e = pick_fastest(4, tv, reps, st, nothing, [&](int i) {
+    cudaError_t e = pick_fastest(4, tv, again, st, nothing, [&](int i) {
         return launch_fwd<T>(g, tp[i], x, K, spec, nullptr, st, vin, 0, false, pdl_fwd);
     }, &b);
     if (e != cudaSuccess) return e;
@@ -2629,7 +2634,7 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     // (the TMA pass also takes 192 / 384 threads; a strip of W columns has 16 W radix-16
     // butterflies at n = 128, its rows packed into two transformed fields)
     // and (nz = 64 or 128) the TMA pass with the register-staged strip (W 8, 16; 256 threads, or 384 in FP32)
-    constexpr int NZC = 18;
+    constexpr int NZC = TUNE_MAX;
     const int wz[NZC] = {4, 4, 8, 8, 16, 16, 32, 32, 8, 8, 16, 16, 8, 8, 16, 8, 16, 16};
     const int tz[NZC] = {128, 256, 128, 256, 128, 256, 128, 256, 256, 512, 256, 512, 192, 384, 384, 256, 256, 384};
     int zb[NZC] = {0};
@@ -2646,13 +2651,14 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     ProjArgs pa;
     pa.kind = GFF_PROJ_CONTINUOUS;
     for (int c = 0; c < 9; ++c) pa.mask[c] = 0.f;
-    // (in place: the spectrum changes its size with every launch, and is laid out anew for every candidate)
+    // (in place: the spectrum changes its size with every launch; in FP64 it is laid out anew for every candidate)
     auto spectrum = [&] { return launch_fwd<T>(g, tn.t_fwd, x, K, spec, nullptr, st, vin); };
+    auto z_input = [&] { return sizeof(T) == 8 ? spectrum() : cudaSuccess; };
     auto z_pass = [&](int i) {
         return zb[i] != 0 ? launch_z_tma<T>(h, wz[i], tz[i], zb[i], pa, nullptr, st, true)
                      : launch_z<T>(g, wz[i], tz[i], spec, pa, nullptr, st, true);
     };
-    e = pick_fastest(NZC, zv, reps, st, spectrum, z_pass, &b);
+    e = pick_fastest(NZC, zv, again, st, z_input, z_pass, &b);
     if (e != cudaSuccess) return e;
     e = spectrum();  // projected, as the inverse pass finds it
     if (e == cudaSuccess) e = z_pass(b);
@@ -2673,7 +2679,7 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     const bool r2 = staged && inv2_radix(g) > 0 && inv2_smem<T>(g) <= SMEM_MAX;
     const bool iv[8] = {true, true, ib[2] > 0, ib[3] > 0, r2, r2, ib[6] < -1, ib[7] < -1};
     int* err = h->d_flag + 2;
-    e = pick_fastest(8, iv, reps, st, nothing, [&](int i) {
+    e = pick_fastest(8, iv, again, st, nothing, [&](int i) {
         return launch_inv<T>(g, ti[i], ib[i], spec, y, oa, nullptr, st, vout, err, 0, true);
     }, &b);
     if (e != cudaSuccess) return e;
