@@ -426,7 +426,7 @@ GFF_EXPORT gff_status gff_create(const gff_grid* grid, const gff_options* opt, g
     h->g.ny = grid->ny;
     h->g.nz = grid->nz;
     h->g.nxh = h->nxh;
-    h->g.N = h->N;
+    set_voxels(h->g, h->N);
     h->g.wait_cycles = BULK_WAIT_CYCLES;
     *out = h;
     if ((st = build_tables(h)) != GFF_OK) return st;

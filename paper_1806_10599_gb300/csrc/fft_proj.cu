@@ -948,10 +948,10 @@ __device__ __forceinline__ void zrow_proj(typename C2<T>::t& u, typename C2<T>::
     }
 }
 // The FP64 projection also applies the inverse transform's 1 / N, but for a power of two near sqrt(N) that the last stage
-// of the inverse takes off its exponents (half_exp; the whole 1 / N here left small fields, 1e-317 say, a few bits of
-// the subnormals).  sc = 2^half_exp / N, which the masks come multiplied by, costs nothing in the factor r = sc / |q|^2, which the grid's table holds (a division per frequency is half of the FP64 operations of
+// of the inverse takes off its exponents (GridDev::half_exp; the whole 1 / N here left small fields, 1e-317 say, a few
+// bits of the subnormals).  sc = 2^half_exp / N, which the masks come multiplied by, costs nothing in the factor
+// r = sc / |q|^2, which the grid's table holds (a division per frequency is half of the FP64 operations of
 // this pass), and saves the plane pass an FP64 operation per voxel.
-__device__ __forceinline__ int half_exp(const GridDev& g) { return (32 - __clz((int)g.N)) >> 1; }
 __device__ __forceinline__ void zrow_proj64(double2& u, double2& v, int kx, int ky, int kz, int nx, int ny, int nz, double m0,
                                             double m1, double m2, double sc, const double* rq2, long long at,
                                             const ZTables<double>& tb) {
@@ -982,7 +982,7 @@ __device__ __forceinline__ void zrow_proj64(double2& u, double2& v, int kx, int 
 // the table: one thread per position (pz, py, kx) of the half spectrum, both kinds; the expression above
 __global__ void __launch_bounds__(256) k_fill_rq2(GridDev g, double* tab) {
     const int nF = g.ny * g.nxh, total = g.nz * nF;
-    const double sc = scalbn(1.0 / (double)g.N, half_exp(g));
+    const double sc = g.zscale;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * total; i += gridDim.x * blockDim.x) {
         const int kind = i / total, e = i - kind * total;
         const int pz = e / nF, f = e - pz * nF, py = f / g.nxh, kx = f - py * g.nxh;
@@ -1006,7 +1006,7 @@ __device__ __forceinline__ void zproj_strip(typename C2<T>::t* s, const GridDev&
     for (int e = tid; e < nz * W; e += nthr) s[e] = zpack<T>(s[e], s[nz * W + e], zcol<T>(tb.colk[e % W], tb));
     __syncthreads();
     fft_lines<T, false, FX>(s, as_tw<T, FX>(tb.twz), g.az, W, 1, 2, 2 * nz * W, W, tid, nthr);
-    const T sc = FX ? (T)scalbn(1.0 / (double)g.N, half_exp(g)) : (T)1;
+    const T sc = FX ? (T)g.zscale : (T)1;
     const T m0 = (T)pa.mask[3 * row] * sc, m1 = (T)pa.mask[3 * row + 1] * sc, m2 = (T)pa.mask[3 * row + 2] * sc;
     for (int e = tid; e < nz * W; e += nthr) {
         const int w = e % W, pz = e / W;
@@ -1489,7 +1489,7 @@ __device__ __forceinline__ void plane_inv_compute(typename C2<T>::t* s, T* __res
     }
     __syncthreads();
     fft_lines<T, true, FX>(s, as_tw<T, FX>(twx), g.ax, half, 2 * ls, 1, 0, 1, tid, nthr,
-                             FX_IN + (FX && oa.pre ? FX_DOWN * half_exp(g) : 0));  // rows fastest, as in pass 1
+                             FX_IN + (FX && oa.pre ? FX_DOWN * g.half_exp : 0));  // rows fastest, as in pass 1
     T sc = (T)oa.scale;
     const T ad = (T)oa.add[c];
     if constexpr (FX) {
@@ -3173,7 +3173,7 @@ __attribute__((visibility("default"))) gff_status gff_project_noalloc(const gff_
     g.ny = grid->ny;
     g.nz = grid->nz;
     g.nxh = grid->nx / 2 + 1;
-    g.N = N;
+    set_voxels(g, N);
     g.wait_cycles = BULK_WAIT_CYCLES;
     for (int a = 0; a < 3; ++a) {
         g.tw64[a] = dt->tw64[a];

@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
 #include <string>
 
@@ -56,8 +57,18 @@ struct GridDev {
     const float* qt32[2][3];
     const double* rq2[2];      // [kind][nz][ny nxh] in the order of the half spectrum: 2^half_exp / (N |q|^2), 0 where the projection
                                // is zero or special (null: the z pass divides instead)
+    int half_exp;              // FP64 on integers: 1 / N is applied as 2^half_exp / N (near 1 / sqrt(N)) by the z pass and
+    double zscale;             // 2^-half_exp by the last stage of the inverse; zscale = 2^half_exp / N
     long long wait_cycles;     // budget of the first wait on each bulk load (BULK_WAIT_CYCLES by default)
 };
+
+inline void set_voxels(GridDev& g, long long N) {
+    int bits = 0;
+    while (bits < 62 && (N >> bits) > 0) ++bits;  // (0 for the sizes that are refused next)
+    g.N = N;
+    g.half_exp = bits / 2;
+    g.zscale = std::ldexp(1.0 / (double)N, g.half_exp);
+}
 
 // Projection parameters of one call.
 struct ProjArgs {
