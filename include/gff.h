@@ -192,8 +192,9 @@ gff_status gff_apply_operator_host(gff_handle* h, int precision, const uint8_t* 
  * gff_cg_kernels_timed: durations in ms, averaged over `reps`, of the vector
  * kernels of one conjugate-gradient iteration on this handle's work vectors
  * (overwritten): ms_out[0] the dot product p.Ap with alpha, [1] x += alpha p,
- * r -= alpha Ap with the new r.r and beta, [2] p = r + beta p.  Algorithmic
- * traffic per element: 2, 6 and 3 vector accesses.
+ * r -= alpha Ap with the new r.r and beta, [2] p = r + beta p, each kernel
+ * alone (in the solver a launch starts while the kernel before it drains).
+ * Algorithmic traffic per element: 2, 6 and 3 vector accesses.
  * gff_measure_fp64_peak: FP64 FMA throughput of the current GPU (independent
  * FMA chains on every SM, best of 5 launches timed with CUDA events), in
  * GFLOP/s (2 flops per FMA); ms_out (may be NULL) the launch's duration.

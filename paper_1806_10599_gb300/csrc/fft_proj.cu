@@ -22,7 +22,7 @@
 // The common lengths (16 ... 128) have two-stage plans with compile-time
 // radices (fft2_lines); the others run the generic stages.  FP64 lines run
 // their stages on 64-bit integers (fft_lines_fx, fixed_bfly.cuh); at 128^3 the
-// FP64 apply takes 1.15 ms where FP64 butterflies took 2.71 ms (forward pass
+// FP64 apply takes 1.16 ms where FP64 butterflies took 2.71 ms (forward pass
 // 1.22 -> 0.60, z 0.64 -> 0.25, inverse 0.86 -> 0.31 ms).  What bounds it now:
 // the forward pass the 81 FP64 multiply-adds per voxel of K:x (0.27 ms at the
 // FP64 pipe's rate), before the row transforms and not under them, since one
@@ -514,7 +514,8 @@ __device__ __noinline__ void fft_lines_fx(double2* s, const int4* tw, const Axis
 }
 
 // Whole transform of a batch of lines; ends with a barrier.  Not inlined:
-// every kernel calls the same four instances (precision x direction).
+// every kernel calls the same six instances (FP32, FP64 on integers,
+// FP64 butterflies; two directions each).
 template <typename T, bool INV>
 __device__ __noinline__ void fft_lines_fp(typename C2<T>::t* s, const typename C2<T>::t* tw, const AxisPlan& pl, int NLF, int SF, int NLS, int SS, int ES,
                                            int tid, int nthr) {
@@ -553,7 +554,7 @@ __device__ __noinline__ void fft_lines_fp(typename C2<T>::t* s, const typename C
     }
 }
 
-// FX: FP64 data on integers (everything but the residuals of mixed precision, ProjArgs::butterflies)
+// FX: FP64 data on integers (everything but the finite-strain residuals of mixed precision, ProjArgs::butterflies)
 template <typename T, bool INV, bool FX>
 __device__ __forceinline__ void fft_lines(typename C2<T>::t* s, const TwP<T, FX>* tw, const AxisPlan& pl, int NLF, int SF,
                                           int NLS, int SS, int ES, int tid, int nthr, int io = 0) {
@@ -1254,15 +1255,12 @@ template <typename T, int W> size_t ztma_smem(const GridDev& g) {
 
 // R1 = 0: any nz (zproj_strip), up to BT = 512 threads; R1 = 16 / 8: nz = 128 / 64 with
 // the register-staged strip (zstrip2), whose fused middle stage holds 16 complex values
-// (u and v of one radix-8 butterfly): BT = 256 threads, two blocks per SM in FP32 and one
-// in FP64 (whose pipe, not the warps in flight, sets the pace; a cap of 128 registers
-// spills), or (FP32) BT = 384, one block per SM
-template <typename T, int W, int R1, int BT> constexpr int ztma_min_blocks() {
-    return (R1 && sizeof(T) == 4 && BT == 256) ? 2 : 1;
-}
+// (u and v of one radix-8 butterfly), in FP32 only: BT = 256 threads, two blocks per SM, or
+// BT = 384, one block per SM
+template <int R1, int BT> constexpr int ztma_min_blocks() { return (R1 && BT == 256) ? 2 : 1; }
 
 template <typename T, int W, int R1, int BT>
-__global__ void __launch_bounds__(BT, ztma_min_blocks<T, W, R1, BT>())
+__global__ void __launch_bounds__(BT, ztma_min_blocks<R1, BT>())
     k_zproj_tma(const __grid_constant__ CUtensorMap tm, GridDev g, ProjArgs pa, const int* __restrict__ skip,
                 int* __restrict__ err) {
     using C = typename C2<T>::t;
@@ -1739,7 +1737,7 @@ __device__ __forceinline__ void inv2_x1(typename C2<T>::t* s, int wg, int lane) 
 }
 
 template <typename T, int R1, int R2>
-__device__ __forceinline__ void inv2_x2(const typename C2<T>::t* s, const typename TwT<T>::t* twx2, T* __restrict__ yp,
+__device__ __forceinline__ void inv2_x2(const typename C2<T>::t* s, const typename C2<T>::t* twx2, T* __restrict__ yp,
                                         T sc, T ad, int wg, int lane) {
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, R2>;
@@ -1761,12 +1759,12 @@ __device__ __forceinline__ void inv2_x2(const typename C2<T>::t* s, const typena
 
 // blocks per SM the register budget is set for: FP32 planes of 68 KB fit three
 // to an SM (256 threads at <= 85 registers) or two (512 threads at <= 64)
-template <typename T, int BT> constexpr int inv2_min_blocks() { return sizeof(T) == 4 ? (BT == 256 ? 3 : 2) : 1; }
+template <int BT> constexpr int inv2_min_blocks() { return BT == 256 ? 3 : 2; }
 
 // Y1 .. X2 of one plane already in shared memory s (twiddle tables loaded); writes plane (c, z) of y.
 template <typename T, int R1, int R2>
-__device__ __forceinline__ void inv2_compute(typename C2<T>::t* s, const typename TwT<T>::t* twy,
-                                             const typename TwT<T>::t* twx2, T* __restrict__ y, const GridDev& g,
+__device__ __forceinline__ void inv2_compute(typename C2<T>::t* s, const typename C2<T>::t* twy,
+                                             const typename C2<T>::t* twx2, T* __restrict__ y, const GridDev& g,
                                              const OutArgs& oa, const int c, const int z) {
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, R2>;
@@ -1819,7 +1817,7 @@ __device__ __forceinline__ void inv2_compute(typename C2<T>::t* s, const typenam
     }}
 
 template <typename T, int R1, int R2, int BT>
-__global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(const typename C2<T>::t* __restrict__ spec,
+__global__ void __launch_bounds__(BT, inv2_min_blocks<BT>()) k_plane_inv2(const typename C2<T>::t* __restrict__ spec,
                                                                       T* __restrict__ y, GridDev g, OutArgs oa,
                                                                       const int* __restrict__ skip,
                                                                       int* __restrict__ err) {
@@ -1829,7 +1827,7 @@ __global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(con
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* s = reinterpret_cast<C*>(sm_raw);  // [n][nxh]
-    auto* twy = reinterpret_cast<typename TwT<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
+    auto* twy = reinterpret_cast<typename C2<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
     auto* twx2 = twy + n;                     // [R2][R1 + 1]: W_n^(p j) of the x axis
     uint64_t* bar =
         reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(twx2 + R2 * P::TWS) + 7) & ~uintptr_t(7));
@@ -1839,10 +1837,10 @@ __global__ void __launch_bounds__(BT, inv2_min_blocks<T, BT>()) k_plane_inv2(con
         mbar_init(bar, 1);
         mbar_init_fence();
     }
-    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, on_int<T>>(g, 1)[i];
+    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, false>(g, 1)[i];
     for (int i = tid; i < R2 * P::TWS; i += nthr) {
         const int j = i / P::TWS, p = i - j * P::TWS;
-        twx2[i] = p < R1 ? twp<T, on_int<T>>(g, 0)[p * j] : typename TwT<T>::t{};
+        twx2[i] = p < R1 ? twp<T, false>(g, 0)[p * j] : C{};
     }
     __syncthreads();
     pdl_wait();
@@ -1875,15 +1873,15 @@ __global__ void __launch_bounds__(BT, 1) k_plane_inv2s(const typename C2<T>::t* 
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* buf[2] = {reinterpret_cast<C*>(sm_raw), reinterpret_cast<C*>(sm_raw) + plane};
-    auto* twy = reinterpret_cast<typename TwT<T>::t*>(buf[1] + plane);
+    auto* twy = reinterpret_cast<typename C2<T>::t*>(buf[1] + plane);
     auto* twx2 = twy + n;
     uint64_t* bar = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(twx2 + 8 * P::TWS) + 7) & ~uintptr_t(7));
     const uint32_t bytes = (uint32_t)(plane * sizeof(C));  // a multiple of 16 (n even)
     const int total = 9 * g.nz, tid = threadIdx.x, nthr = blockDim.x;
-    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, on_int<T>>(g, 1)[i];
+    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, false>(g, 1)[i];
     for (int i = tid; i < 8 * P::TWS; i += nthr) {
         const int j = i / P::TWS, q = i - j * P::TWS;
-        twx2[i] = q < R1 ? twp<T, on_int<T>>(g, 0)[q * j] : typename TwT<T>::t{};
+        twx2[i] = q < R1 ? twp<T, false>(g, 0)[q * j] : C{};
     }
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -1959,7 +1957,7 @@ int inv2_radix(const GridDev& g) {
 // (Forming K:x in registers at the X1 positions, scalar loads 8 voxels apart,
 // measured 1.3x slower in FP32 at 128^3 than these 16-byte loads.)
 template <typename T, int R1>
-__device__ __forceinline__ void fwd2_x1(typename C2<T>::t* s, const typename TwT<T>::t* twx2, int wg, int lane) {
+__device__ __forceinline__ void fwd2_x1(typename C2<T>::t* s, const typename C2<T>::t* twx2, int wg, int lane) {
     using C = typename C2<T>::t;
     using P = Inv2Plan<R1, 8>;
     const int k = lane / P::L2, j = lane % P::L2;
@@ -2020,10 +2018,10 @@ __device__ __forceinline__ void fwd2_x2(typename C2<T>::t* s, int wg, int lane) 
     (void)n;
 }
 
-template <typename T, int BT> constexpr int fwd2_min_blocks() { return sizeof(T) == 4 ? (BT == 256 ? 3 : 2) : 1; }
+template <int BT> constexpr int fwd2_min_blocks() { return BT == 256 ? 3 : 2; }
 
 template <typename T, int R1, int BT>
-__global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(const T* __restrict__ x,
+__global__ void __launch_bounds__(BT, fwd2_min_blocks<BT>()) k_plane_fwd2(const T* __restrict__ x,
                                                                            const T* __restrict__ K,
                                                                            typename C2<T>::t* __restrict__ spec,
                                                                            GridDev g, const int* __restrict__ skip) {
@@ -2033,14 +2031,14 @@ __global__ void __launch_bounds__(BT, fwd2_min_blocks<T, BT>()) k_plane_fwd2(con
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C* s = reinterpret_cast<C*>(sm_raw);  // [n][nxh]
-    auto* twy = reinterpret_cast<typename TwT<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
+    auto* twy = reinterpret_cast<typename C2<T>::t*>(s + n * nxh);  // [n]: W_n^k of the y axis
     auto* twx2 = twy + n;                     // [8][R1 + 1]: W_n^(p j) of the x axis
     const int c = blockIdx.x, z = blockIdx.y;
     const int tid = threadIdx.x, nthr = blockDim.x;
-    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, on_int<T>>(g, 1)[i];
+    for (int i = tid; i < n; i += nthr) twy[i] = twp<T, false>(g, 1)[i];
     for (int i = tid; i < R2 * P::TWS; i += nthr) {
         const int j = i / P::TWS, p = i - j * P::TWS;
-        twx2[i] = p < R1 ? twp<T, on_int<T>>(g, 0)[p * j] : typename TwT<T>::t{};
+        twx2[i] = p < R1 ? twp<T, false>(g, 0)[p * j] : C{};
     }
     pdl_wait();
     if (skip && load_flag(skip)) return;
@@ -2331,7 +2329,8 @@ int z2_radix(const GridDev& g) {
     return (g.az.radix[0] == 16 || g.az.radix[0] == 8) ? g.az.radix[0] : 0;
 }
 
-// block threads of the TMA z pass: any up to 512 for the generic strip; 256, or 384 in FP32, for zstrip2
+// block threads of the TMA z pass: any up to 512 for the generic strip; 256, or 384 in FP32, for zstrip2 (in FP64 these
+// shapes are accepted and run the generic strip)
 template <typename T> bool ztma_threads_ok(int R1, int threads) {
     if (!R1) return threads > 0 && threads <= 512;
     return threads == 256 || (sizeof(T) == 4 && threads == 384);
@@ -2353,8 +2352,7 @@ cudaError_t launch_z_tma_k(gff_handle* h, int threads, int blocks, const ProjArg
     if constexpr (R1 == 0) {
         return launch_z_tma_kb<T, W, 0, 512>(h, threads, blocks, pa, skip, st, pdl);
     } else {
-        if constexpr (sizeof(T) == 4)
-            if (threads == 384) return launch_z_tma_kb<T, W, R1, 384>(h, threads, blocks, pa, skip, st, pdl);
+        if (threads == 384) return launch_z_tma_kb<T, W, R1, 384>(h, threads, blocks, pa, skip, st, pdl);
         return launch_z_tma_kb<T, W, R1, 256>(h, threads, blocks, pa, skip, st, pdl);
     }
 }
@@ -2407,8 +2405,7 @@ int z_tma_blocks_k(gff_handle* h, int threads) {
     if constexpr (R1 == 0) {
         return z_tma_blocks_kb<T, W, 0, 512>(h, threads);
     } else {
-        if constexpr (sizeof(T) == 4)
-            if (threads == 384) return z_tma_blocks_kb<T, W, R1, 384>(h, threads);
+        if (threads == 384) return z_tma_blocks_kb<T, W, R1, 384>(h, threads);
         return z_tma_blocks_kb<T, W, R1, 256>(h, threads);
     }
 }
@@ -2878,11 +2875,13 @@ cudaError_t launch_galerkin(const gff_handle* h, const T* x, const T* K, T* y, c
     OutArgs oo = oa;
     oo.pre = pa.sym ? 0 : 1;
     // The z and inverse passes come in, load their tables and wait while the pass before them drains: 24.6 -> 19.7 us
-    // at 16^3 FP32, 119 -> 114 us at 80 x 96 x 48 FP32, 239 -> 235 us at 128^3 FP32.  The forward pass does so on small grids
-    // only (24^3 FP32 20.7 -> 18.5 us, 16^3 FP64 35 -> 33 us): blocks that arrive early keep the shared-memory split
-    // the inverse pass left on their SM, and on grids that fill the GPU several times its loads then run with less
-    // first-level cache (64^3 FP64 187 -> 205 us, 128^3 FP32 235 -> 306 us; the same figures as when that split is
-    // asked for).  Not between timing events, and not into a graph the caller is capturing (there the plain order).
+    // at 16^3 FP32, 119 -> 114 us at 80 x 96 x 48 FP32, 239 -> 235 us at 128^3 FP32.  The forward pass does so up to 2^17
+    // voxels (forward_starts_early): applies in FP32 and FP64 without -> with, 32^3 22.4 -> 20.8 and 51.6 -> 51.4 us, 40^3
+    // 32.8 -> 30.7 and 89.6 -> 87.9 us, 48^3 41.1 -> 38.9 and 128.5 -> 128.0 us, 64 x 32 x 64 34.9 -> 32.6 and 106.7 ->
+    // 106.1 us.  Blocks that arrive early keep the shared-memory split the inverse pass left on their SM; while field
+    // loads went through the first-level cache, that made grids which fill the GPU several times slower (128^3 FP32 235
+    // -> 306 us).  Since they leave no line there, 60^3 gains too (84.0 -> 81.0 and 202.8 -> 200.4 us), and 64^3 (39.4
+    // -> 37.6 and 171.9 -> 169.7 us); larger grids are not measured, and the line stays.  Not between timing events, and not into a graph the caller is capturing (there the plain order).
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool pdl = !ev && cudaStreamIsCapturing(h->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
     const bool pdl_fwd = pdl && forward_starts_early(g);
@@ -3018,8 +3017,10 @@ template cudaError_t launch_galerkin_host<float>(gff_handle*, const float*, floa
 // themselves: code embedded in a host application whose allocator owns the
 // whole device-memory budget, or loops that cannot afford the device-wide
 // synchronisation a cudaMalloc/cudaFree may imply.  It runs the same three
-// kernels as gff_project, but its scratch -- the half spectrum and the grid
-// tables -- is the file-scope array below, which every GPU that loads the
+// kernels as gff_project, at fixed launch shapes, with twiddles to the 53 bits
+// of the device's sincospi (a handle's have 62) and a division per frequency in
+// place of the handle's table of projection factors; its scratch -- the half
+// spectrum and the grid tables -- is the file-scope array below, which every GPU that loads the
 // library holds until the process exits.  The paper has no counterpart.
 namespace gff {
 namespace {

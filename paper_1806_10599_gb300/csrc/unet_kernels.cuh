@@ -59,7 +59,7 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint
 // block four warps = 64 MW voxels.  Each output's sum runs over t and then ci whatever the split, so the bits do not
 // depend on it.  Bound: the loads of the weight fragments (two 4-byte loads per tile of 8 channels and k16 step), hence
 // MW tiles of voxels per fragment where the grid is large enough to fill the GPU all the same, and the channels split
-// over blocks where it is not (conv_shape in unet.cu).
+// over blocks where it is not (launch_conv_nt in unet.cu).
 template <int NT, int MW, bool RELU>
 __global__ void __launch_bounds__(128) k_conv3(const bf16* __restrict__ in, int sin, int cin,
                                                const bf16* __restrict__ W, int cout, const float* __restrict__ bias,

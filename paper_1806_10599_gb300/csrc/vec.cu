@@ -555,7 +555,10 @@ cudaError_t measure_fp64_fma(double* out, int blocks, int iters, int reps, cudaS
 // Times the CG vector kernels of one iteration on the vectors x, r, p, Ap
 // (n elements, overwritten with a ramp first): ms[0] p.Ap (partial sums and
 // alpha), ms[1] x += alpha p, r -= alpha Ap with r.r (and beta), ms[2]
-// p = r + beta p; averages over `reps` iterations.
+// p = r + beta p; averages over `reps` iterations.  An event between two
+// launches makes the second wait for the first to end, so these are the times
+// of the kernels one by one; the solver's launches (launch_cg_alpha,
+// launch_cg_step) start while the kernel before drains.
 template <typename T>
 cudaError_t time_cg_kernels(T* x, T* r, T* p, T* Ap, long long n, double* partial, double* cg, int* flag,
                             cudaStream_t s, int reps, float* ms) {
