@@ -2493,12 +2493,12 @@ cudaError_t launch_inv(const GridDev& g, int threads, int blocks, const typename
 
 
 // Fastest candidate of one kernel: set() lays out its input, run(i) launches candidate i.  Each is timed over three
-// launches after one; where these are short (passes of a few microseconds differ by less than one), those within a
-// twelfth of the fastest are timed over five more.  The host waits once per round, not per candidate.  The call takes,
-// ten launches of every candidate -> now: 16^3 4.5 -> 3.2 ms, 32^3 6.7 -> 4.1 ms, 48^3 14.0 -> 7.7 ms.
+// launches after one.  Where these are short there is a second round: of those within a twelfth of the fastest, over
+// five launches (keep = 0), or of the `keep` fastest, over three calls of run2(i), the whole apply with candidate i.  The
+// host waits once per round, not per candidate.
 constexpr int TUNE_MAX = 18;  // candidates of one kernel
-template <typename S, typename F>
-cudaError_t pick_fastest(int ncand, const bool* valid, bool again, cudaStream_t st, S set, F run, int* best) {
+template <typename S, typename F, typename G>
+cudaError_t pick_fastest(int ncand, const bool* valid, bool again, int keep, cudaStream_t st, S set, F run, G run2, int* best) {
     cudaEvent_t ev[2 * TUNE_MAX] = {};
     float ms[TUNE_MAX];
     bool in[TUNE_MAX];
@@ -2510,10 +2510,11 @@ cudaError_t pick_fastest(int ncand, const bool* valid, bool again, cudaStream_t 
     for (int round = 0; round < (again ? 2 : 1) && e == cudaSuccess; ++round) {
         for (int i = 0; i < ncand && e == cudaSuccess; ++i) {
             if (!in[i]) continue;
+            auto go = [&] { return round && keep ? run2(i) : run(i); };
             e = set();
-            if (e == cudaSuccess) e = run(i);  // warm-up (also sets the shared-memory attribute)
+            if (e == cudaSuccess) e = go();  // warm-up (also sets the shared-memory attribute)
             if (e == cudaSuccess) e = cudaEventRecord(ev[2 * i], st);
-            for (int r = 0; r < (round ? 5 : 3) && e == cudaSuccess; ++r) e = run(i);
+            for (int r = 0; r < (round && !keep ? 5 : 3) && e == cudaSuccess; ++r) e = go();
             if (e == cudaSuccess) e = cudaEventRecord(ev[2 * i + 1], st);
         }
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -2523,7 +2524,12 @@ cudaError_t pick_fastest(int ncand, const bool* valid, bool again, cudaStream_t 
             e = cudaEventElapsedTime(&ms[i], ev[2 * i], ev[2 * i + 1]);
             if (*best < 0 || ms[i] < ms[*best]) *best = i;
         }
-        for (int i = 0; i < ncand && *best >= 0; ++i) in[i] = in[i] && 12 * ms[i] <= 13 * ms[*best];
+        for (int i = 0; i < ncand && e == cudaSuccess; ++i) {  // (ranks count `valid`: part of `in` is decided already)
+            if (!valid[i]) continue;
+            int faster = 0;
+            for (int j = 0; j < ncand; ++j) faster += valid[j] && ms[j] < ms[i];
+            in[i] = keep ? faster < keep : 12 * ms[i] <= 13 * ms[*best];
+        }
     }
     for (cudaEvent_t v : ev)
         if (v) cudaEventDestroy(v);
@@ -2604,7 +2610,11 @@ template <typename T> cudaError_t tune_fill(T* p, long long n, cudaStream_t st) 
 
 // x, K and what the passes make of them hold values like a field's: an FP64 line of zeros leaves its integer stages at
 // once, and shapes compared on zeros are compared without their transforms (at 80 x 96 x 48 that took the inverse pass of
-// 512 threads, 328 us per apply, for the one of 256, 312 us).  The passes are launched as an apply launches them.
+// 512 threads, 328 us per apply, for the one of 256, 312 us).  The passes are launched as an apply launches them.  Up to
+// 2^14 voxels a pass takes no longer than the host does to launch it, and its time alone says little: there passes run one
+// after the other in the first round, and the three best are compared in whole applies in the second (shapes by passes
+// alone -> by applies, FP32 applies, median of ten handles: 10 x 24 x 10 26.1 -> 23.1 us, 12^3 22.8 -> 22.7 us, 16^3 18.8
+// -> 18.1 us).  Both precisions take 4.0 ms at 16^3, 5.5 ms at 24^3, 3.5 ms at 32^3, 6.7 ms at 48^3, 43 ms at 128^3.
 template <typename T>
 cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     using C = typename C2<T>::t;
@@ -2612,7 +2622,8 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     C* spec = reinterpret_cast<C*>(h->d_spec);
     cudaStream_t st = h->stream;
     const bool again = g.N <= 1 << 17;
-    const bool pdl_fwd = forward_starts_early(g);
+    const int keep = g.N <= 1 << 14 ? 3 : 0;
+    const bool pdl = !keep, pdl_fwd = pdl && forward_starts_early(g);
     auto nothing = [] { return cudaSuccess; };
     Tune& tn = h->tune[tune_index<T>()];
     const bool vin = vec_ok<T>(g, x) && vec_ok<T>(g, K);
@@ -2621,9 +2632,28 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     const bool f2 = staged && inv2_radix(g) > 0 && fwd2_smem<T>(g) <= SMEM_MAX;
     const int tp[4] = {256, 512, -256, -512};
     const bool tv[4] = {true, true, f2, f2};
+    ProjArgs pa;
+    pa.kind = GFF_PROJ_CONTINUOUS;
+    for (int c = 0; c < 9; ++c) pa.mask[c] = 0.f;
+    OutArgs oa;
+    oa.scale = 1.0;
+    for (int c = 0; c < 9; ++c) oa.add[c] = 0.0;
+    const bool vout = vec_ok<T>(g, y);
+    int* err = h->d_flag + 2;
+    auto whole = [&](const Tune& t) {
+        cudaError_t e = launch_fwd<T>(g, t.t_fwd, x, K, spec, nullptr, st, vin, 0, false, true);
+        if (e == cudaSuccess)
+            e = t.z_blocks != 0 ? launch_z_tma<T>(h, t.wz, t.t_z, t.z_blocks, pa, nullptr, st, true)
+                                : launch_z<T>(g, t.wz, t.t_z, spec, pa, nullptr, st, true);
+        return e == cudaSuccess ? launch_inv<T>(g, t.t_inv, t.inv_blocks, spec, y, oa, nullptr, st, vout, err, 0, true) : e;
+    };
     int b = -1;
-    cudaError_t e = pick_fastest(4, tv, again, st, nothing, [&](int i) {
+    cudaError_t e = pick_fastest(4, tv, again, keep, st, nothing, [&](int i) {
         return launch_fwd<T>(g, tp[i], x, K, spec, nullptr, st, vin, 0, false, pdl_fwd);
+    }, [&](int i) {
+        Tune t = tn;
+        t.t_fwd = tp[i];
+        return whole(t);
     }, &b);
     if (e != cudaSuccess) return e;
     tn.t_fwd = tp[b];
@@ -2645,17 +2675,20 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
         zb[i] = staged ? -z_tma_blocks<T>(h, wz[i], tz[i], true) : 0;
         zv[i] = zb[i] < 0;
     }
-    ProjArgs pa;
-    pa.kind = GFF_PROJ_CONTINUOUS;
-    for (int c = 0; c < 9; ++c) pa.mask[c] = 0.f;
-    // (in place: the spectrum changes its size with every launch; in FP64 it is laid out anew for every candidate)
+    // In place: the spectrum changes its size with every launch, in FP64 by nz 2^half_exp / N, at most six bits down.  There
+    // it is laid out anew for every fourth candidate, long before its lines leave the integers.
     auto spectrum = [&] { return launch_fwd<T>(g, tn.t_fwd, x, K, spec, nullptr, st, vin); };
-    auto z_input = [&] { return sizeof(T) == 8 ? spectrum() : cudaSuccess; };
+    int laid = 0;
+    auto z_input = [&] { return sizeof(T) == 8 && laid++ % 4 == 0 ? spectrum() : cudaSuccess; };
     auto z_pass = [&](int i) {
-        return zb[i] != 0 ? launch_z_tma<T>(h, wz[i], tz[i], zb[i], pa, nullptr, st, true)
-                     : launch_z<T>(g, wz[i], tz[i], spec, pa, nullptr, st, true);
+        return zb[i] != 0 ? launch_z_tma<T>(h, wz[i], tz[i], zb[i], pa, nullptr, st, pdl)
+                          : launch_z<T>(g, wz[i], tz[i], spec, pa, nullptr, st, pdl);
     };
-    e = pick_fastest(NZC, zv, again, st, z_input, z_pass, &b);
+    e = pick_fastest(NZC, zv, again, keep, st, z_input, z_pass, [&](int i) {
+        Tune t = tn;
+        t.wz = wz[i], t.t_z = tz[i], t.z_blocks = zb[i];
+        return whole(t);
+    }, &b);
     if (e != cudaSuccess) return e;
     e = spectrum();  // projected, as the inverse pass finds it
     if (e == cudaSuccess) e = z_pass(b);
@@ -2663,21 +2696,20 @@ cudaError_t autotune_prec(gff_handle* h, T* x, T* y, const T* K) {
     tn.wz = wz[b];
     tn.t_z = tz[b];
     tn.z_blocks = zb[b];
-    OutArgs oa;
-    oa.scale = 1.0;
-    for (int c = 0; c < 9; ++c) oa.add[c] = 0.0;
     // one block per plane with 256 or 512 threads, the persistent streamed pass with 512 or 1024,
     // or (two-stage plans, nx = ny) the register-staged pass with 256 or 512, one block per plane, or
     // persistent with two plane buffers (512, or 1024 in FP32)
-    const bool vout = vec_ok<T>(g, y);
     const int ti[8] = {256, 512, inv_stream_max_threads<T>() / 2, inv_stream_max_threads<T>(), 256, 512, 512, 1024};
     int ib[8] = {0, 0, inv_stream_blocks<T>(g, 512, vout), inv_stream_blocks<T>(g, 1024, vout), -1, -1,
                  staged ? -inv2s_blocks<T>(g, 512) : 0, staged ? -inv2s_blocks<T>(g, 1024) : 0};
     const bool r2 = staged && inv2_radix(g) > 0 && inv2_smem<T>(g) <= SMEM_MAX;
     const bool iv[8] = {true, true, ib[2] > 0, ib[3] > 0, r2, r2, ib[6] < -1, ib[7] < -1};
-    int* err = h->d_flag + 2;
-    e = pick_fastest(8, iv, again, st, nothing, [&](int i) {
-        return launch_inv<T>(g, ti[i], ib[i], spec, y, oa, nullptr, st, vout, err, 0, true);
+    e = pick_fastest(8, iv, again, keep, st, nothing, [&](int i) {
+        return launch_inv<T>(g, ti[i], ib[i], spec, y, oa, nullptr, st, vout, err, 0, pdl);
+    }, [&](int i) {
+        Tune t = tn;
+        t.t_inv = ti[i], t.inv_blocks = ib[i];
+        return whole(t);
     }, &b);
     if (e != cudaSuccess) return e;
     tn.t_inv = ti[b];
